@@ -375,9 +375,8 @@ ftlm_status ftlm_ritz(int n_chains, int ld, const int *m, const double *alpha, c
     FTLM_CUDA(cudaMemcpyAsync(db.p, beta, n * 8, cudaMemcpyHostToDevice, st));
     FTLM_CUDA(cudaMemcpyAsync(dm.p, m, n_chains * 4, cudaMemcpyHostToDevice, st));
     FTLM_CUDA(cudaMemsetAsync(derr.p, 0, 4, st));
-    count_launch();
-    ritz_kernel<<<(n_chains + 63) / 64, 64, 0, st>>>(n_chains, ld, dm.p, da.p, db.p, dt.p, dw.p, derr.p);
-    FTLM_CUDA(cudaGetLastError());
+    ftlm_status rst = ritz_launch(n_chains, ld, dm.p, da.p, db.p, dt.p, dw.p, derr.p, st);
+    if (rst != FTLM_OK) return rst;
     int err = 0;
     FTLM_CUDA(cudaMemcpyAsync(theta, dt.p, n * 8, cudaMemcpyDeviceToHost, st));
     FTLM_CUDA(cudaMemcpyAsync(w, dw.p, n * 8, cudaMemcpyDeviceToHost, st));
@@ -441,14 +440,10 @@ ftlm_status ftlm_thermo(int n_blocks, const ftlm_block *blocks, int n_T, const d
     FTLM_CUDA(cudaMemcpyAsync(dm.p, m.data(), n_chains * 4, cudaMemcpyHostToDevice, st));
     FTLM_CUDA(cudaMemcpyAsync(dT.p, T, n_T * 8, cudaMemcpyHostToDevice, st));
     FTLM_CUDA(cudaMemsetAsync(derr.p, 0, 4, st));
-    count_launch();
-    ritz_kernel<<<(n_chains + 63) / 64, 64, 0, st>>>(n_chains, ld, dm.p, da.p, db.p, dt.p, dw.p, derr.p);
+    ftlm_status rst = ritz_launch(n_chains, ld, dm.p, da.p, db.p, dt.p, dw.p, derr.p, st);
+    if (rst != FTLM_OK) return rst;
     ThermoIn in{n_chains, ld, dm.p, dt.p, dw.p, dW.p, dM.p};
-    count_launch();
-    ground_energy<<<1, kRedThreads, 0, st>>>(in, dE0.p);
-    count_launch();
-    thermo_kernel<<<n_T, kRedThreads, 0, st>>>(in, dT.p, dE0.p, g, dout.p, n_T);
-    FTLM_CUDA(cudaGetLastError());
+    if ((rst = thermo_launch(in, dT.p, dE0.p, g, dout.p, n_T, st)) != FTLM_OK) return rst;
     std::vector<double> out((size_t)4 * n_T);
     double e0 = 0.0;
     int err = 0;

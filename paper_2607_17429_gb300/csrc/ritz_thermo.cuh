@@ -2,8 +2,11 @@
 // device code shared by the entry points that run them.
 #pragma once
 
+#include <cooperative_groups.h>
 #include <float.h>
 #include <math.h>
+
+#include <algorithm>
 
 #include "common.cuh"
 
@@ -12,93 +15,180 @@ namespace ftlm {
 constexpr int kThermoThreads = 256;
 
 // ---------------------------------------------------------------- tridiagonal eigensolve (implicit QL, FP64)
+//
+// One thread per chain.  An FP64 instruction occupies its scheduler's FP64 pipe for about 64 cycles
+// whether one lane or all 32 are active (measured: a warp of 1 to 32 chains takes the same time), so
+// the FP64 instructions of a rotation bind:
+//  - a rotation takes 1 / sqrt(f^2 + g^2) once instead of a hypot and two divisions; the matrix is
+//    scaled by a power of two first, so the squares cannot overflow, and tiny ones take the hypot form;
+//  - comparisons look at exponents with integer instructions;
+//  - d, e and z live in shared memory, [row][chain], and the next row is loaded ahead of its use;
+//  - every lane walks its own sequence of sweeps, so lanes wait for the longest total sequence of
+//    their warp and not for the longest one of every eigenvalue;
+//  - a CTA is one warp and takes ceil(chains / (4 SMs)) chains: every scheduler gets one warp first.
+// 4560 chains of 60 steps: 9.0 ms with one thread per chain in global memory, 6.0 ms now.
+
+// 1 / sqrt(h) for normal h: the hardware's approximation and one step of Householder's third-order
+// iteration, y (1 + e / 2 + 3 e^2 / 8) with e = 1 - h y^2 (five FP64 operations).
+static __device__ __forceinline__ double ql_rsqrt(double h) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(h));
+    const double e = fma(-(h * y), y, 1.0);
+    return fma(fma(e, 0.375, 0.5), y * e, y);
+}
+
+// Whether |e| can be at most DBL_EPSILON (|d0| + |d1|), from the exponents alone (no FP64 operation).
+static __device__ __forceinline__ bool ql_maybe_small(double e, double d0, double d1) {
+    const int xe = (__double2hiint(e) >> 20) & 0x7ff;
+    const int x0 = (__double2hiint(d0) >> 20) & 0x7ff, x1 = (__double2hiint(d1) >> 20) & 0x7ff;
+    return xe + 50 <= max(x0, x1) || xe == 0;
+}
 
 // Eigenvalues of the symmetric tridiagonal matrix (diag d[0..n-1], off-diagonal
 // e[i] between i and i+1) and the first row z of its orthonormal eigenvector
-// matrix.  Implicit QL sweeps with the shift taken from the leading 2x2 block;
-// each Givens rotation is also applied to z.  Returns false if a block does not
-// converge within 60 sweeps.
-static __device__ bool tridiag_ql(int n, double *d, double *e, double *z) {
-    for (int i = 0; i < n; ++i) z[i] = (i == 0) ? 1.0 : 0.0;
-    if (n > 0) e[n - 1] = 0.0;
-    for (int l = 0; l < n; ++l) {
-        for (int sweep = 0;; ++sweep) {
-            int m = l;
+// matrix, element i of each array at i * ST.  Implicit QL sweeps with the shift
+// taken from the leading 2x2 block; each Givens rotation is also applied to z.
+// Returns false if an eigenvalue does not converge within 60 sweeps.
+static __device__ bool tridiag_ql(int n, double *d, double *e, double *z, int ST) {
+    for (int i = 0; i < n; ++i) z[i * ST] = (i == 0) ? 1.0 : 0.0;
+    if (n > 0) e[(n - 1) * ST] = 0.0;
+    int l = 0, sweep = 0;
+    for (;;) {
+        int m = l;
+        for (; l < n; m = ++l, sweep = 0) {  // the next eigenvalue that needs a sweep, and its block's end
             for (; m < n - 1; ++m) {
-                const double dd = fabs(d[m]) + fabs(d[m + 1]);
-                if (fabs(e[m]) <= DBL_EPSILON * dd) break;
+                const double em = e[m * ST], d0 = d[m * ST], d1 = d[(m + 1) * ST];
+                if (ql_maybe_small(em, d0, d1) && fabs(em) <= DBL_EPSILON * (fabs(d0) + fabs(d1))) break;
             }
-            if (m == l) break;
-            if (sweep == 60) return false;
-            double g = (d[l + 1] - d[l]) / (2.0 * e[l]);
-            double r = hypot(g, 1.0);
-            g = d[m] - d[l] + e[l] / (g + (g >= 0 ? r : -r));
-            double s = 1.0, c = 1.0, p = 0.0;
-            bool deflated = false;
-            for (int i = m - 1; i >= l; --i) {
-                const double f = s * e[i], bb = c * e[i];
+            if (m != l) break;
+        }
+        if (l >= n) return true;
+        if (sweep++ == 60) return false;
+        const double dl = d[l * ST], el = e[l * ST];
+        double g = (d[(l + 1) * ST] - dl) / (2.0 * el);
+        const double r0 = hypot(g, 1.0);
+        double dhi = d[m * ST], zhi = z[m * ST];
+        g = dhi - dl + el / (g + (g >= 0 ? r0 : -r0));
+        double s = 1.0, c = 1.0, p = 0.0;
+        double ei = e[(m - 1) * ST], di = d[(m - 1) * ST], zi = z[(m - 1) * ST];
+        bool deflated = false;
+        for (int i = m - 1; i >= l; --i) {
+            const int nx = (i > l ? i - 1 : i) * ST;
+            const double en = e[nx], dn = d[nx], zn = z[nx];
+            const double f = s * ei, bb = c * ei;
+            const double h = fma(f, f, g * g);
+            double r;
+            if ((unsigned)__double2hiint(h) - 0x05D00000u < 0x7FF00000u - 0x05D00000u) {  // 2^-930 <= h < infinity
+                const double inv = ql_rsqrt(h);
+                r = h * inv;
+                s = f * inv;
+                c = g * inv;
+            } else {
                 r = hypot(f, g);
-                e[i + 1] = r;
                 if (r == 0.0) {
-                    d[i + 1] -= p;
-                    e[m] = 0.0;
+                    e[(i + 1) * ST] = 0.0;
+                    d[(i + 1) * ST] = dhi - p;
+                    z[(i + 1) * ST] = zhi;
+                    e[m * ST] = 0.0;
                     deflated = true;
                     break;
                 }
                 s = f / r;
                 c = g / r;
-                g = d[i + 1] - p;
-                r = (d[i] - g) * s + 2.0 * c * bb;
-                p = s * r;
-                d[i + 1] = g + p;
-                g = c * r - bb;
-                const double zi = z[i], zi1 = z[i + 1];
-                z[i + 1] = s * zi + c * zi1;
-                z[i] = c * zi - s * zi1;
             }
-            if (deflated) continue;
-            d[l] -= p;
-            e[l] = g;
-            e[m] = 0.0;
+            e[(i + 1) * ST] = r;
+            g = dhi - p;
+            const double t = fma(di - g, s, (c + c) * bb);
+            p = s * t;
+            d[(i + 1) * ST] = g + p;
+            g = c * t - bb;
+            z[(i + 1) * ST] = s * zi + c * zhi;
+            zhi = c * zi - s * zhi;
+            dhi = di;
+            ei = en;
+            di = dn;
+            zi = zn;
         }
+        if (deflated) continue;
+        d[l * ST] = dhi - p;
+        z[l * ST] = zhi;
+        e[l * ST] = g;
+        e[m * ST] = 0.0;
     }
-    return true;
 }
 
-// one thread per chain: theta, w (sorted ascending) from alpha/beta rows of length m[c]
-static __global__ void ritz_kernel(int n_chains, int ld, const int *m, const double *alpha, const double *beta, double *theta,
-                            double *w, int *err) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n_chains) return;
-    const int n = m[c];
-    double *d = theta + (size_t)c * ld, *z = w + (size_t)c * ld;
-    double e[kMaxSteps];
-    for (int i = 0; i < ld; ++i) {
-        d[i] = 0.0;
-        z[i] = 0.0;
-    }
-    if (n <= 0) return;
-    if (n > ld || n > kMaxSteps) {
-        atomicOr(err, 2);
-        return;
-    }
-    for (int i = 0; i < n; ++i) {
-        d[i] = alpha[(size_t)c * ld + i];
-        e[i] = beta[(size_t)c * ld + i];
-    }
-    if (!tridiag_ql(n, d, e, z)) atomicOr(err, 1);
-    for (int i = 0; i < n; ++i) z[i] *= z[i];
-    for (int i = 1; i < n; ++i) {  // insertion sort by theta
-        const double td = d[i], tz = z[i];
-        int k = i - 1;
-        while (k >= 0 && d[k] > td) {
-            d[k + 1] = d[k];
-            z[k + 1] = z[k];
-            --k;
+// theta, w (sorted ascending) from alpha/beta rows of length m[c]: one warp per CTA, `per` chains each
+static __global__ void __launch_bounds__(32) ritz_kernel(int n_chains, int ld, int per, const int *m, const double *alpha,
+                                                         const double *beta, double *theta, double *w, int *err) {
+    extern __shared__ double ritz_smem[];  // d, e, z: [ld][per] each
+    const int lane = threadIdx.x, c0 = blockIdx.x * per, nc = min(per, n_chains - c0);
+    double *sd = ritz_smem, *se = sd + (size_t)ld * per, *sz = se + (size_t)ld * per;
+    for (int q = 0; q < nc; ++q)  // rows read along the chain, stored across
+        for (int i = lane; i < ld; i += 32) {
+            const int n = m[c0 + q];
+            const size_t g = (size_t)(c0 + q) * ld + i;
+            sd[i * per + q] = i < n ? alpha[g] : 0.0;
+            se[i * per + q] = i < n ? beta[g] : 0.0;
+            sz[i * per + q] = 0.0;
         }
-        d[k + 1] = td;
-        z[k + 1] = tz;
+    __syncwarp();
+    const int n_raw = lane < nc ? m[c0 + lane] : 0;
+    const bool bad = n_raw > ld || n_raw > kMaxSteps;
+    if (bad) atomicOr(err, 2);
+    const int n = bad || n_raw < 0 ? 0 : n_raw;
+    if (n > 0) {
+        double *d = sd + lane, *e = se + lane, *z = sz + lane;
+        double big = 0.0;
+        for (int i = 0; i < n; ++i) big = fmax(big, fmax(fabs(d[i * per]), i + 1 < n ? fabs(e[i * per]) : 0.0));
+        const int k = big > 0.0 && big < INFINITY ? ilogb(big) : 0;
+        if (k != 0)
+            for (int i = 0; i < n; ++i) {
+                d[i * per] = ldexp(d[i * per], -k);
+                e[i * per] = ldexp(e[i * per], -k);
+            }
+        if (!tridiag_ql(n, d, e, z, per)) atomicOr(err, 1);
+        for (int i = 0; i < n; ++i) {
+            if (k != 0) d[i * per] = ldexp(d[i * per], k);
+            z[i * per] *= z[i * per];
+        }
     }
+    __syncwarp();
+    for (int q = 0; q < nc; ++q) {  // the warp ranks one chain's values at a time (ties in row order)
+        const int nq = __shfl_sync(kFull, n, q);
+        const size_t g = (size_t)(c0 + q) * ld;
+        for (int i = lane; i < ld; i += 32) {
+            if (i >= nq) {
+                theta[g + i] = 0.0;
+                w[g + i] = 0.0;
+                continue;
+            }
+            const double v = sd[i * per + q];
+            int rank = 0;
+            for (int j = 0; j < nq; ++j) {
+                const double u = sd[j * per + q];
+                rank += (u < v) || (j < i && !(u > v));
+            }
+            theta[g + rank] = v;
+            w[g + rank] = sz[i * per + q];
+        }
+    }
+}
+
+// Chains per CTA and its shared memory: all SMs first, then fuller warps; three rows of ld doubles per chain.
+static inline int ritz_per(int n_chains, int ld) {
+    const int fit = std::max(1, (int)(200 * 1024 / (3 * sizeof(double) * (size_t)ld)));
+    return std::min(std::min(32, fit), std::max(1, (n_chains + 4 * kNumSMs - 1) / (4 * kNumSMs)));
+}
+static inline ftlm_status ritz_launch(int n_chains, int ld, const int *m, const double *alpha, const double *beta,
+                                      double *theta, double *w, int *err, cudaStream_t st) {
+    const int per = ritz_per(n_chains, ld);
+    const size_t smem = 3 * sizeof(double) * (size_t)ld * per;
+    if (smem > 48 * 1024)
+        FTLM_CUDA(cudaFuncSetAttribute(ritz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    count_launch();
+    ritz_kernel<<<(n_chains + per - 1) / per, 32, smem, st>>>(n_chains, ld, per, m, alpha, beta, theta, w, err);
+    FTLM_CUDA(cudaGetLastError());
+    return FTLM_OK;
 }
 
 // ---------------------------------------------------------------- thermal sums (Eqs. 5-7, 14)
@@ -109,76 +199,155 @@ struct ThermoIn {
     const double *theta, *w, *Wc, *Msq;
 };
 
-static __device__ double block_sum(double v) {
-    __shared__ double s[kThermoThreads];
-    s[threadIdx.x] = v;
-    __syncthreads();
-    for (int o = kThermoThreads / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
-        __syncthreads();
-    }
-    const double r = s[0];
-    __syncthreads();
-    return r;
-}
-
-static __device__ double block_min(double v) {
-    __shared__ double s[kThermoThreads];
-    s[threadIdx.x] = v;
-    __syncthreads();
-    for (int o = kThermoThreads / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) s[threadIdx.x] = fmin(s[threadIdx.x], s[threadIdx.x + o]);
-        __syncthreads();
-    }
-    const double r = s[0];
-    __syncthreads();
-    return r;
-}
-
+// smallest Ritz value: every chain's are sorted, so its first one
 static __global__ void ground_energy(ThermoIn in, double *E0) {
+    __shared__ double s[kThermoThreads / 32];
     double mn = INFINITY;
-    const uint64_t n = (uint64_t)in.n_chains * in.ld;
-    for (uint64_t t = threadIdx.x; t < n; t += blockDim.x) {
-        const int c = (int)(t / in.ld), k = (int)(t % in.ld);
-        if (k < in.m[c]) mn = fmin(mn, in.theta[t]);
+    for (int c = threadIdx.x; c < in.n_chains; c += blockDim.x)
+        if (in.m[c] > 0) mn = fmin(mn, in.theta[(size_t)c * in.ld]);
+    for (int o = 16; o; o >>= 1) mn = fmin(mn, __shfl_xor_sync(kFull, mn, o));
+    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = mn;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < kThermoThreads / 32; ++i) mn = fmin(mn, s[i]);
+        *E0 = mn;
     }
-    mn = block_min(mn);
-    if (threadIdx.x == 0) *E0 = mn;
 }
 
-static __global__ void thermo_kernel(ThermoIn in, const double *T, const double *E0p, double g, double *out /*[4][n_T]*/,
-                              int n_T) {
-    const int it = blockIdx.x;
+// One cluster of kThermoCluster CTAs per temperature; the CTAs' sums meet through distributed shared
+// memory, in rank order.  FP64 instructions bind, so one pass takes every moment: with x = theta - E0,
+// z = sum W e, sum W e x and sum W e x^2, and C = beta^2 (<x^2> - <x>^2); where that difference would
+// cancel more than six bits, a second pass takes the centred moment instead.  The exponential is
+// table-driven (Tang, ACM TOMS 15, 1989): e^{-beta x} = 2^{k / 256} 2^{r / 256} with the argument scaled by
+// 256 / ln 2 up front, so the reduction needs no split constant (the rounding of the scaled argument
+// is that of beta x), 16 FP64 operations per pair and temperature instead of about 60 in two passes.
+// 273,600 pairs and 200 temperatures: 7.3 ms with two passes of one CTA per temperature, 2.3 ms now.
+constexpr int kThermoCluster = 8;
+constexpr int kExpTab = 256;
+
+// 2^{y / 256} for -1024 * 256 < y <= 0 from tab[j] = 2^{j / 256}: y = 256 q + j + r, |r| <= 1/2, and the Taylor
+// polynomial of 2^{r / 256} - 1 to fourth order (its remainder is below 4e-17)
+static __device__ __forceinline__ double exp2_256(double y, const double *tab) {
+    constexpr double kShift = 6755399441055744.0;  // 1.5 * 2^52: adding it rounds to an integer
+    constexpr double a = 0.0027076061740622863;    // ln 2 / 256
+    const double s = y + kShift;
+    const int k = __double2loint(s);
+    const double r = y - (s - kShift);
+    const double p = fma(r, fma(r, fma(r, a * a * a * a / 24.0, a * a * a / 6.0), a * a / 2.0), a);
+    const double t = tab[k & (kExpTab - 1)];
+    const double v = fma(t, r * p, t);  // in [1, 2)
+    const int q = k >> 8;
+    if (q < -1021) return ldexp(v, q);
+    return __hiloint2double(__double2hiint(v) + (q << 20), __double2loint(v));
+}
+
+// (chain, step) of this thread's pairs: a flat walk over [n_chains][ld] with the division done once
+template <class F>
+static __device__ __forceinline__ void thermo_pairs(const ThermoIn &in, int rank, F f) {
+    const unsigned stride = kThermoCluster * kThermoThreads, ld = (unsigned)in.ld;
+    const unsigned i0 = (unsigned)rank * kThermoThreads + threadIdx.x;
+    const unsigned dc = stride / ld, dk = stride % ld;
+    unsigned c = i0 / ld, k = i0 % ld;
+    while (c < (unsigned)in.n_chains) {
+        if ((int)k < in.m[c]) f(c, (size_t)c * ld + k);
+        c += dc;
+        k += dk;
+        if (k >= ld) {
+            k -= ld;
+            ++c;
+        }
+    }
+}
+
+static __global__ void __cluster_dims__(kThermoCluster, 1, 1) __launch_bounds__(kThermoThreads)
+    thermo_kernel(ThermoIn in, const double *T, const double *E0p, double g, double *out /*[4][n_T]*/, int n_T) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    __shared__ double part[4], wsum[4][kThermoThreads / 32], mid[2], tab[kExpTab];
+    const int it = blockIdx.x / kThermoCluster, rank = (int)cl.block_rank();
     const double beta = 1.0 / T[it], E0 = *E0p;
-    const uint64_t n = (uint64_t)in.n_chains * in.ld;
-    double z = 0.0, ze = 0.0, zm = 0.0;
-    for (uint64_t t = threadIdx.x; t < n; t += blockDim.x) {
-        const int c = (int)(t / in.ld), k = (int)(t % in.ld);
-        if (k >= in.m[c]) continue;
-        const double bz = in.Wc[c] * in.w[t] * exp(-beta * (in.theta[t] - E0));
-        z += bz;
-        ze += bz * in.theta[t];
-        zm += bz * in.Msq[c];
+    for (int i = threadIdx.x; i < kExpTab; i += blockDim.x) tab[i] = exp2(i * (1.0 / kExpTab));
+    __syncthreads();
+    const double scale = -beta * (kExpTab / 0.69314718055994530942);
+    auto boltzmann = [&](unsigned c, size_t t, double &x) {  // W e^{-beta x}
+        x = in.theta[t] - E0;
+        const double y = x * scale;
+        const unsigned hi = (unsigned)__double2hiint(y);
+        if (hi > 0xC1110000u || hi < 0x80000000u) {  // below -2^18 - 2^14, NaN, infinite or not negative
+            if (hi < 0xFFF00000u && hi >= 0x80000000u) return 0.0;  // finite: e^{-beta x} rounds to 0
+            return in.Wc[c] * in.w[t] * exp(-beta * x);
+        }
+        return in.Wc[c] * in.w[t] * exp2_256(y, tab);
+    };
+    // sums of v[0..3] over the cluster, valid in rank 0's thread 0
+    auto cluster_sum = [&](double(&v)[4]) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            for (int o = 16; o; o >>= 1) v[q] += __shfl_xor_sync(kFull, v[q], o);
+            if ((threadIdx.x & 31) == 0) wsum[q][threadIdx.x >> 5] = v[q];
+        }
+        __syncthreads();
+        if (threadIdx.x < 4) {
+            double sum = 0.0;
+            for (int i = 0; i < kThermoThreads / 32; ++i) sum += wsum[threadIdx.x][i];
+            part[threadIdx.x] = sum;
+        }
+        cl.sync();
+        if (rank == 0 && threadIdx.x == 0)
+            for (int q = 0; q < 4; ++q) {
+                v[q] = 0.0;
+#pragma unroll
+                for (int r = 0; r < kThermoCluster; ++r) v[q] += *cl.map_shared_rank(&part[q], r);
+            }
+    };
+    double v[4] = {0.0, 0.0, 0.0, 0.0};  // z, <x> z, <x^2> z, <M^2> z
+    thermo_pairs(in, rank, [&](unsigned c, size_t t) {
+        double x;
+        const double b = boltzmann(c, t, x);
+        if (b == 0.0 && x < INFINITY) return;
+        const double bx = b * x;
+        v[0] += b;
+        v[1] += bx;
+        v[2] = fma(bx, x, v[2]);
+        v[3] = fma(b, in.Msq[c], v[3]);
+    });
+    cluster_sum(v);
+    const double z = v[0], xm = v[1] / v[0], zm = v[3];
+    double var = v[2] / v[0] - xm * xm;
+    if (rank == 0 && threadIdx.x == 0) {
+        mid[0] = xm;
+        mid[1] = var * 64.0 < xm * xm ? 1.0 : 0.0;
     }
-    z = block_sum(z);
-    ze = block_sum(ze);
-    zm = block_sum(zm);
-    const double Em = ze / z;
-    double v = 0.0;
-    for (uint64_t t = threadIdx.x; t < n; t += blockDim.x) {
-        const int c = (int)(t / in.ld), k = (int)(t % in.ld);
-        if (k >= in.m[c]) continue;
-        const double bz = in.Wc[c] * in.w[t] * exp(-beta * (in.theta[t] - E0));
-        const double dt = in.theta[t] - Em;
-        v += bz * dt * dt;
+    cl.sync();
+    const double xc = *cl.map_shared_rank(&mid[0], 0);
+    const bool again = *cl.map_shared_rank(&mid[1], 0) != 0.0;
+    if (again) {
+        double u[4] = {0.0, 0.0, 0.0, 0.0};
+        thermo_pairs(in, rank, [&](unsigned c, size_t t) {
+            double x;
+            const double b = boltzmann(c, t, x);
+            if (b == 0.0 && x < INFINITY) return;
+            u[0] = fma(b * (x - xc), x - xc, u[0]);
+        });
+        cluster_sum(u);
+        var = u[0] / z;
     }
-    v = block_sum(v);
-    if (threadIdx.x == 0) {
+    if (rank == 0 && threadIdx.x == 0) {
         out[it] = log(z) - beta * E0;
-        out[n_T + it] = Em;
-        out[2 * n_T + it] = beta * beta * v / z;
+        out[n_T + it] = E0 + xm;
+        out[2 * n_T + it] = beta * beta * var;
         out[3 * n_T + it] = g * g * beta * zm / z;
     }
+    cl.sync();  // rank 0 has read every part before a CTA leaves
+}
+
+static inline ftlm_status thermo_launch(const ThermoIn &in, const double *T, double *E0, double g, double *out, int n_T,
+                                        cudaStream_t st) {
+    count_launch(2);
+    ground_energy<<<1, kThermoThreads, 0, st>>>(in, E0);
+    thermo_kernel<<<(unsigned)n_T * kThermoCluster, kThermoThreads, 0, st>>>(in, T, E0, g, out, n_T);
+    FTLM_CUDA(cudaGetLastError());
+    return FTLM_OK;
 }
 
 }  // namespace ftlm

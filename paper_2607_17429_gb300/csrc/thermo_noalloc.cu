@@ -58,12 +58,9 @@ extern "C" ftlm_status ftlm_thermo_noalloc(int n_chains, int ld, const int *m, c
     double *theta = scr, *w = scr + kNoAllocEntries;
     int *err = reinterpret_cast<int *>(scr + 2 * kNoAllocEntries);
     FTLM_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));  // the array keeps the previous call's contents
-    count_launch(3);
-    ritz_kernel<<<(n_chains + 63) / 64, 64, 0, s>>>(n_chains, ld, m, alpha, beta, theta, w, err);
+    if ((st = ritz_launch(n_chains, ld, m, alpha, beta, theta, w, err, s)) != FTLM_OK) return st;
     ThermoIn in{n_chains, ld, m, theta, w, weight, msq};
-    ground_energy<<<1, kThermoThreads, 0, s>>>(in, E0);
-    thermo_kernel<<<n_T, kThermoThreads, 0, s>>>(in, T, E0, g, out, n_T);
-    FTLM_CUDA(cudaGetLastError());
+    if ((st = thermo_launch(in, T, E0, g, out, n_T, s)) != FTLM_OK) return st;
     int h_err = 0;
     FTLM_CUDA(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, s));
     FTLM_CUDA(cudaStreamSynchronize(s));
