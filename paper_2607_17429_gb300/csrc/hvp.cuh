@@ -99,6 +99,7 @@ template <typename VT>
 struct HvpPart {
     uint64_t n_reps;
     uint64_t tile0;          // first tile of this part in the launch's tile order
+    int tile_reps;           // representatives per tile of this part
     const HvRec *rec;        // [n_reps], ascending labels; rec.off = index * W
     const uint32_t *bucket;  // [n_buckets + 1]
     uint64_t n_buckets;
@@ -132,7 +133,6 @@ struct HvpArgs {
     HvpPart<VT> part0;           // the part when n_parts == 1
     const HvpPart<VT> *parts;    // device array when n_parts > 1
     uint64_t n_tiles;
-    int tile_reps;
     int B, BT, lgBT, nbuf, tma;
     int esize;               // bytes of one stored vector element (sizeof(VT), or 2 for FP16 storage)
     int stage_elems;         // stored elements of one staging buffer
@@ -484,8 +484,8 @@ __global__ void __launch_bounds__(hvp_max_threads<VT, SH>(), 1) hvp_kernel(const
         }
         const HvpPart<VT> &P = a.n_parts == 1 ? a.part0 : a.parts[p];
         const uint64_t n_reps = P.n_reps;
-        const uint64_t r0 = (t - P.tile0) * (uint64_t)a.tile_reps;
-        const uint64_t r1 = min(r0 + (uint64_t)a.tile_reps, n_reps);
+        const uint64_t r0 = (t - P.tile0) * (uint64_t)P.tile_reps;
+        const uint64_t r1 = min(r0 + (uint64_t)P.tile_reps, n_reps);
         const HvRec *rec = P.rec;
         const VT *sqrtS = P.sqrtS;
         const ST *__restrict__ x = static_cast<const ST *>(P.x);
@@ -908,7 +908,6 @@ ftlm_status hvp_launch_t(HvpArgs<VT> a, const HvpGeom &geo, cudaStream_t stream)
     auto kern = hvp_kernel<VT, ST, SH, GPL, HALF, MODE>;
     a.nbuf = geo.nbuf;
     a.tma = geo.tma;
-    a.tile_reps = geo.tile_reps;
     a.rho_smem = geo.rho_smem;
     a.own = geo.own;
     const size_t smem = hvp_smem_t<VT, ST, SH, GPL, HALF, MODE>(a, geo.warps, geo.nbuf);

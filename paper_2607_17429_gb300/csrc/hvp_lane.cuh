@@ -121,8 +121,8 @@ __global__ void __launch_bounds__(kLaneThreads) hvp_lane_kernel(const __grid_con
             cur_part = p;
         }
         const HvpPart<VT> &P = a.n_parts == 1 ? a.part0 : a.parts[p];
-        const uint64_t rep = (t - P.tile0) * (uint64_t)a.tile_reps + threadIdx.x;
-        if (rep >= P.n_reps) continue;
+        const uint64_t rep = (t - P.tile0) * (uint64_t)P.tile_reps + threadIdx.x;
+        if (rep >= P.n_reps || (int)threadIdx.x >= P.tile_reps) continue;
         const ST *__restrict__ x = static_cast<const ST *>(P.x);
         ST *__restrict__ y = static_cast<ST *>(P.y);
         const uint64_t n_elems = P.n_reps * (uint64_t)D;
@@ -249,7 +249,6 @@ int hvp_lane_occupancy_t(const HvpArgs<VT> &a, int warps, int) {
 
 template <typename VT, typename ST, int D>
 ftlm_status hvp_lane_launch_t(HvpArgs<VT> a, const HvpGeom &geo, cudaStream_t stream) {
-    a.tile_reps = geo.tile_reps;
     hvp_lane_kernel<VT, ST, D><<<(unsigned)geo.grid, kLaneThreads, hvp_lane_smem<VT, ST, D>(a), stream>>>(a);
     count_launch();
     FTLM_CUDA(cudaGetLastError());

@@ -26,7 +26,7 @@ struct HvpOps {
     int (*occupancy)(const HvpArgs<VT> &, int warps, int nbuf);
     ftlm_status (*launch)(HvpArgs<VT>, const HvpGeom &, cudaStream_t);
     int max_threads;
-    int tile_fixed;  // representatives per tile fixed by the kernel (0: chosen with the geometry)
+    int tile_fixed;  // one thread per representative: the CTA's threads, the most a tile takes (0: warp kernels)
 };
 
 #define FTLM_HVP_OPS_M(VT, ST, SH, GPL, HALF, MODE)                                              \

@@ -160,31 +160,28 @@ __global__ void __launch_bounds__(kLzThreads) lzp_start(const __grid_constant__ 
 // Rows of every representative are consecutive W-row segments, so element e of a part has row
 // (e / B) mod W and chain e mod B; a CTA covers W B 2^k elements at a time, VEC neighbours per thread
 // (four chains of one row with 8- or 16-byte loads when B is a multiple of four, else one), so every
-// thread keeps its (row, chains), hence one block, one set of coefficients and VEC accumulators, over
-// the CTA's contiguous run of tiles.  A CTA that reaches the next part writes its |w|^2 per (block,
-// chain) of the last one: the CTAs' runs and the parts are both ordered, so (CTA c, part p) owns slot
-// c + p of norm_part, and the finalize kernel reads only the CTAs that touched its part.  Per part the
-// elements of equal (row, chain) meet in a fixed tree and a block's rows are added in order.  (Every CTA
-// walking every part, with 256 terms scanned per (block, chain): 1.17 ms a step for the six s = 3/2
-// icosahedron sectors M = 0..5 at 24 chains, 0.12 ms now; the icosidodecahedron's 5.3 GB a step at
-// 8 chains 0.84 ms before, 0.74 ms now.)
+// thread keeps its (row, chains), hence one block, one set of coefficients and VEC accumulators.  A CTA
+// takes one run of representatives of one part; a part's runs depend on the part alone, so a set gives
+// the same sums in any mix.  Per run the elements of equal (row, chain) meet in a fixed tree and a
+// block's rows are added in order.  (Every CTA walking every part, with 256 terms scanned per (block,
+// chain): 1.17 ms a step for the six s = 3/2 icosahedron sectors M = 0..5 at 24 chains, 0.12 ms now;
+// the icosidodecahedron's 5.3 GB a step at 8 chains 0.84 ms before, 0.74 ms now.)
 constexpr int kUpdElems = 1024;  // elements of a CTA at a time, at most (W B <= 1024)
 constexpr int kUpdThreads = 1024;  // threads per SM aimed at
+constexpr int kUpdMinSteps = 8;    // loop steps of a run, at least (its reduction costs about two)
 
 template <typename VT>
 struct LzUpd {
     int n_parts, W, B, K, has_prev, n_sub;  // n_sub: representatives side by side in a CTA (a power of two)
     int zrow[kPMaxK + 1];       // first row of each block in a segment, then W
     int blk_of_row[32];         // block of each row of a segment
-    int tile_reps;
-    uint64_t n_tiles, chunk;    // tiles in all, tiles per CTA
-    const uint64_t *tile0, *ntile;  // [n_parts]
+    const uint64_t *run0, *run_reps;  // [n_parts]: first run of each part, representatives per run
     const uint64_t *elem0;      // [n_parts + 1] first element of each part in the vectors
     const int *entry0;          // [n_parts] p * K * B
     void *y;                    // in: H u_j, out: w (storage type)
     const void *u, *up;
     const VT *coef;             // [entries][3]
-    double *norm_part;          // [gridDim.x + n_parts][K][B]
+    double *norm_part;          // [runs][K][B]
 };
 
 // VEC neighbouring stored elements, one load or store
@@ -223,13 +220,11 @@ __global__ void __launch_bounds__(VEC == 1 ? kUpdElems : kUpdElems / VEC) lzp_up
     __shared__ double red[kUpdElems];
     const int B = a.B, WB = a.W * a.B, K = a.K, tid = threadIdx.x;
     const int tb = tid * VEC % WB, k = a.blk_of_row[tb / B], b = tb % B;
-    const uint64_t t1 = min((blockIdx.x + 1) * a.chunk, a.n_tiles), T = (uint64_t)blockDim.x * VEC;
-    uint64_t t = blockIdx.x * a.chunk;
-    if (t >= t1) return;
+    const uint64_t run = blockIdx.x, T = (uint64_t)blockDim.x * VEC;
     int p = 0;
-    for (int hi = a.n_parts - 1; p < hi;) {  // last part whose first tile is <= t
+    for (int hi = a.n_parts - 1; p < hi;) {  // last part whose first run is <= run (parts without runs come before it)
         const int mid = (p + hi + 1) >> 1;
-        if (a.tile0[mid] <= t)
+        if (a.run0[mid] <= run)
             p = mid;
         else
             hi = mid - 1;
@@ -237,72 +232,65 @@ __global__ void __launch_bounds__(VEC == 1 ? kUpdElems : kUpdElems / VEC) lzp_up
     ST *__restrict__ y = static_cast<ST *>(a.y);
     const ST *__restrict__ u = static_cast<const ST *>(a.u);
     const ST *__restrict__ up = static_cast<const ST *>(a.up);
-    for (; t < t1; ++p) {
-        const uint64_t pt0 = a.tile0[p], pt1 = pt0 + a.ntile[p];
-        if (pt1 <= t) continue;  // a part without representatives
-        const uint64_t te = min(t1, pt1);
-        const uint64_t p0 = a.elem0[p], p1 = a.elem0[p + 1], per_tile = (uint64_t)a.tile_reps * WB;
-        const uint64_t end = min(p1, p0 + (te - pt0) * per_tile);
-        const VT *c = a.coef + ((size_t)a.entry0[p] + k * B + b) * 3;
-        VT cy[VEC], cu[VEC], cp[VEC];
+    const uint64_t len = a.run_reps[p] * (uint64_t)WB, start = a.elem0[p] + (run - a.run0[p]) * len;
+    const uint64_t end = min(a.elem0[p + 1], start + len);
+    const VT *c = a.coef + ((size_t)a.entry0[p] + k * B + b) * 3;
+    VT cy[VEC], cu[VEC], cp[VEC];
+#pragma unroll
+    for (int v = 0; v < VEC; ++v) {
+        cy[v] = c[3 * v];
+        cu[v] = c[3 * v + 1];
+        cp[v] = a.has_prev ? c[3 * v + 2] : (VT)0;
+    }
+    DotAcc<VT> acc[VEC];
+#pragma unroll
+    for (int v = 0; v < VEC; ++v) acc[v].zero();
+    auto step = [&](uint64_t e, const VT(&yv)[VEC], const VT(&uv)[VEC], const VT(&pv)[VEC]) {
+        alignas(16) ST ws[VEC];
 #pragma unroll
         for (int v = 0; v < VEC; ++v) {
-            cy[v] = c[3 * v];
-            cu[v] = c[3 * v + 1];
-            cp[v] = a.has_prev ? c[3 * v + 2] : (VT)0;
+            ws[v] = st_put<VT, ST>(cy[v] * yv[v] - cu[v] * uv[v] - cp[v] * pv[v]);
+            const VT w = st_get<VT, ST>(ws[v]);
+            acc[v].add(w, w);
         }
-        DotAcc<VT> acc[VEC];
+        upd_store<ST, VEC>(y + e, ws);
+    };
+    constexpr int U = VEC == 1 ? 4 : 2;  // steps in flight per thread
+    uint64_t e = start + (uint64_t)tid * VEC;
+    for (; e + (U - 1) * T < end; e += U * T) {
+        VT yv[U][VEC], uv[U][VEC], pv[U][VEC];
 #pragma unroll
-        for (int v = 0; v < VEC; ++v) acc[v].zero();
-        auto step = [&](uint64_t e, const VT(&yv)[VEC], const VT(&uv)[VEC], const VT(&pv)[VEC]) {
-            alignas(16) ST ws[VEC];
+        for (int q = 0; q < U; ++q) {
+            upd_load<VT, ST, VEC>(y + e + q * T, yv[q]);
+            upd_load<VT, ST, VEC>(u + e + q * T, uv[q]);
 #pragma unroll
-            for (int v = 0; v < VEC; ++v) {
-                ws[v] = st_put<VT, ST>(cy[v] * yv[v] - cu[v] * uv[v] - cp[v] * pv[v]);
-                const VT w = st_get<VT, ST>(ws[v]);
-                acc[v].add(w, w);
-            }
-            upd_store<ST, VEC>(y + e, ws);
-        };
-        constexpr int U = VEC == 1 ? 4 : 2;  // steps in flight per thread
-        uint64_t e = p0 + (t - pt0) * per_tile + (uint64_t)tid * VEC;
-        for (; e + (U - 1) * T < end; e += U * T) {
-            VT yv[U][VEC], uv[U][VEC], pv[U][VEC];
-#pragma unroll
-            for (int q = 0; q < U; ++q) {
-                upd_load<VT, ST, VEC>(y + e + q * T, yv[q]);
-                upd_load<VT, ST, VEC>(u + e + q * T, uv[q]);
-#pragma unroll
-                for (int v = 0; v < VEC; ++v) pv[q][v] = (VT)0;
-                if (a.has_prev) upd_load<VT, ST, VEC>(up + e + q * T, pv[q]);
-            }
-#pragma unroll
-            for (int q = 0; q < U; ++q) step(e + q * T, yv[q], uv[q], pv[q]);
-        }
-        for (; e < end; e += T) {
-            VT yv[VEC], uv[VEC], pv[VEC];
-            upd_load<VT, ST, VEC>(y + e, yv);
-            upd_load<VT, ST, VEC>(u + e, uv);
-#pragma unroll
-            for (int v = 0; v < VEC; ++v) pv[v] = (VT)0;
-            if (a.has_prev) upd_load<VT, ST, VEC>(up + e, pv);
-            step(e, yv, uv, pv);
+            for (int v = 0; v < VEC; ++v) pv[q][v] = (VT)0;
+            if (a.has_prev) upd_load<VT, ST, VEC>(up + e + q * T, pv[q]);
         }
 #pragma unroll
-        for (int v = 0; v < VEC; ++v) red[tid * VEC + v] = acc[v].value();
+        for (int q = 0; q < U; ++q) step(e + q * T, yv[q], uv[q], pv[q]);
+    }
+    for (; e < end; e += T) {
+        VT yv[VEC], uv[VEC], pv[VEC];
+        upd_load<VT, ST, VEC>(y + e, yv);
+        upd_load<VT, ST, VEC>(u + e, uv);
+#pragma unroll
+        for (int v = 0; v < VEC; ++v) pv[v] = (VT)0;
+        if (a.has_prev) upd_load<VT, ST, VEC>(up + e, pv);
+        step(e, yv, uv, pv);
+    }
+#pragma unroll
+    for (int v = 0; v < VEC; ++v) red[tid * VEC + v] = acc[v].value();
+    __syncthreads();
+    for (int h = a.n_sub >> 1; h; h >>= 1) {
+        for (int i = tid; i < h * WB; i += blockDim.x) red[i] += red[i + h * WB];
         __syncthreads();
-        for (int h = a.n_sub >> 1; h; h >>= 1) {
-            for (int i = tid; i < h * WB; i += blockDim.x) red[i] += red[i + h * WB];
-            __syncthreads();
-        }
-        for (int i = tid; i < K * B; i += blockDim.x) {
-            const int kk = i / B, bb = i % B;
-            double sum = 0.0;
-            for (int r = a.zrow[kk]; r < a.zrow[kk + 1]; ++r) sum += red[r * B + bb];
-            a.norm_part[((size_t)blockIdx.x + p) * K * B + i] = sum;
-        }
-        __syncthreads();
-        t = te;
+    }
+    for (int i = tid; i < K * B; i += blockDim.x) {
+        const int kk = i / B, bb = i % B;
+        double sum = 0.0;
+        for (int r = a.zrow[kk]; r < a.zrow[kk + 1]; ++r) sum += red[r * B + bb];
+        a.norm_part[(size_t)run * K * B + i] = sum;
     }
 }
 
@@ -319,8 +307,8 @@ struct LzState {
 
 // One CTA per part and 32 (block, chain) entries: a lane per entry, eight warps over slices of the
 // per-CTA partials of the CTAs that processed tiles of the part (fixed association: it depends on the
-// partial count only).  chunk > 0: CTA c took the tiles [c chunk, (c + 1) chunk) and its partial of part
-// p is in slot c + p; chunk = 0: CTA t mod grid took tile t and wrote [p][CTA].
+// partial count only).  grid = 0: one partial per tile (or run); else CTA t mod grid took tile t and wrote
+// [p][CTA].
 // mode 0: start-vector norms; 1: alpha_j and the update coefficients; 2: beta_{j+1}.
 // With `scaled` (FP16 storage) the update writes sigma w instead of w, sigma the
 // per-block power of two 2^floor(log2(sqrt(rows) / (16 Hmax))) with Hmax = |J|
@@ -334,29 +322,26 @@ struct LzState {
 constexpr int kFinSlices = 8;
 
 __global__ void __launch_bounds__(32 * kFinSlices)
-    lzp_finalize(int mode, int j, int K, int B, int grid, uint64_t chunk, const uint64_t *tile0, const uint64_t *ntile,
-                 const double *part, LzState st, double tol, int scaled) {
+    lzp_finalize(int mode, int j, int K, int B, int grid, const uint64_t *tile0, const uint64_t *ntile, const double *part,
+                 LzState st, double tol, int scaled) {
     const int p = blockIdx.x, KB = K * B;
     const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5, t = blockIdx.y * 32 + lane;
     __shared__ double sl_sum[kFinSlices][32];
     const int k = t / B, b = t % B;
     const size_t e = ((size_t)p * K + k) * B + b;
     const uint64_t nt = ntile[p], t0 = tile0[p];
-    uint64_t n, c0, base;  // partial i sits in row base + (c0 + i) mod grid
-    if (chunk) {
-        c0 = t0 / chunk;
-        n = nt ? (t0 + nt - 1) / chunk - c0 + 1 : 0;
-        base = (uint64_t)p;
-    } else {
-        n = nt >= (uint64_t)grid ? (uint64_t)grid : nt;
-        c0 = nt >= (uint64_t)grid ? 0 : t0 % (uint64_t)grid;
-        base = (uint64_t)p * grid;
+    uint64_t n = nt, c0 = 0, base = t0, wrap = nt;  // partial i sits in row base + (c0 + i) mod wrap
+    if (grid) {
+        wrap = (uint64_t)grid;
+        n = min(nt, wrap);
+        c0 = nt >= wrap ? 0 : t0 % wrap;
+        base = (uint64_t)p * wrap;
     }
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
     if (t < KB) {
         auto at = [&](uint64_t i) {
             uint64_t c = c0 + i;
-            if (c >= (uint64_t)grid) c -= (uint64_t)grid;
+            if (c >= wrap) c -= wrap;
             return part[(base + c) * KB + t];
         };
         constexpr uint64_t S = kFinSlices;
@@ -609,34 +594,34 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
         la.key0 = (uint32_t)seed;
         la.norm_part = lz_part.p;
         const uint64_t *hv_t0 = tiles.p, *hv_nt = tiles.p + P, *lz_t0 = tiles.p + 2 * P, *lz_nt = tiles.p + 3 * P;
-        // flat update: W B 2^k elements per CTA at a time, contiguous runs of tiles of 8 steps
+        // flat update: W B 2^k elements per CTA at a time, one run of representatives per CTA
         const int WB = ps0->W * B, up_vec = B % 4 == 0 ? 4 : 1;
         int n_sub = 1;
         while (2 * n_sub * WB <= (up_vec == 4 ? kUpdElems : kUpdElems / 2)) n_sub *= 2;
         const int up_threads = n_sub * WB / up_vec;
-        const int up_tile = 8 * n_sub;
-        std::vector<uint64_t> elem0(P + 1), ut(2 * (size_t)P);  // update tiles: first, count
+        const uint64_t up_ctas = (uint64_t)sms * std::max(1, std::min(8, kUpdThreads / up_threads));
+        std::vector<uint64_t> elem0(P + 1), ut(3 * (size_t)P);  // runs: first, count, representatives
         std::vector<int> ent(P);
-        uint64_t up_tiles = 0;
+        uint64_t up_runs = 0;
         for (int p = 0; p <= P; ++p) elem0[p] = row0[p] * (uint64_t)B;
         for (int p = 0; p < P; ++p) {
+            const uint64_t n = sets[p].sec->n_reps, steps = (n + n_sub - 1) / n_sub;
+            const uint64_t len = n_sub * std::max<uint64_t>(kUpdMinSteps, (steps + up_ctas - 1) / up_ctas);
             ent[p] = p * K * B;
-            ut[p] = up_tiles;
-            ut[P + p] = (sets[p].sec->n_reps + up_tile - 1) / up_tile;
-            up_tiles += ut[P + p];
+            ut[p] = up_runs;
+            ut[P + p] = (n + len - 1) / len;
+            ut[2 * P + p] = len;
+            up_runs += ut[P + p];
         }
-        const uint64_t up_ctas = (uint64_t)sms * std::max(1, std::min(8, kUpdThreads / up_threads));
-        const uint64_t up_chunk = std::max<uint64_t>(1, (up_tiles + up_ctas - 1) / up_ctas);
-        const int up_grid = (int)std::max<uint64_t>(1, (up_tiles + up_chunk - 1) / up_chunk);
         DevBuf<double> up_part;
-        FTLM_CUDA(up_part.alloc(((size_t)P + up_grid) * K * B));
+        FTLM_CUDA(up_part.alloc(std::max<uint64_t>(1, up_runs) * K * B));
         DevBuf<uint64_t> d_elem0, d_ut;
         DevBuf<int> d_ent;
         FTLM_CUDA(d_elem0.alloc(P + 1));
-        FTLM_CUDA(d_ut.alloc(2 * (size_t)P));
+        FTLM_CUDA(d_ut.alloc(3 * (size_t)P));
         FTLM_CUDA(d_ent.alloc(P));
         FTLM_CUDA(cudaMemcpyAsync(d_elem0.p, elem0.data(), (P + 1) * 8, cudaMemcpyHostToDevice, stream));
-        FTLM_CUDA(cudaMemcpyAsync(d_ut.p, ut.data(), 2 * (size_t)P * 8, cudaMemcpyHostToDevice, stream));
+        FTLM_CUDA(cudaMemcpyAsync(d_ut.p, ut.data(), 3 * (size_t)P * 8, cudaMemcpyHostToDevice, stream));
         FTLM_CUDA(cudaMemcpyAsync(d_ent.p, ent.data(), P * sizeof(int), cudaMemcpyHostToDevice, stream));
         const dim3 fin_grid(P, (K * B + 31) / 32);
         constexpr int kFinThreads = 32 * kFinSlices;
@@ -653,11 +638,8 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
                 for (int d = 0; d < ps0->dims[k]; ++d) U.blk_of_row[r++] = k;
             for (int k = 0; k < K; ++k) U.zrow[k + 1] = U.zrow[k] + ps0->dims[k];
             U.n_sub = n_sub;
-            U.tile_reps = up_tile;
-            U.n_tiles = up_tiles;
-            U.chunk = up_chunk;
-            U.tile0 = d_ut.p;
-            U.ntile = d_ut.p + P;
+            U.run0 = d_ut.p;
+            U.run_reps = d_ut.p + 2 * P;
             U.elem0 = d_elem0.p;
             U.entry0 = d_ent.p;
             U.y = vb[(q + 1) % 3].p;
@@ -671,7 +653,7 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
         ftlm_status s1 = lzp_start_launch<VT, ST>(K, la, lz_grid, stream);
         if (s1 != FTLM_OK) return s1;
         count_launch();
-        lzp_finalize<<<fin_grid, kFinThreads, 0, stream>>>(0, 0, K, B, lz_grid, 0, lz_t0, lz_nt, lz_part.p, st, tol, kScaled);
+        lzp_finalize<<<fin_grid, kFinThreads, 0, stream>>>(0, 0, K, B, lz_grid, lz_t0, lz_nt, lz_part.p, st, tol, kScaled);
         FTLM_CUDA(cudaGetLastError());
         // ---- the step loop (captured once on a private stream, replayed once on the caller's)
         const bool prof = profiling_on();
@@ -694,20 +676,18 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
                     FTLM_CUDA(capture ? cudaEventRecordWithFlags(ev.back(), ss, cudaEventRecordExternal)
                                       : cudaEventRecord(ev.back(), ss));
                 count_launch();
-                lzp_finalize<<<fin_grid, kFinThreads, 0, ss>>>(1, j, K, B, hv_grid, 0, hv_t0, hv_nt, hv_part.p, st, tol,
-                                                          kScaled);
+                lzp_finalize<<<fin_grid, kFinThreads, 0, ss>>>(1, j, K, B, hv_grid, hv_t0, hv_nt, hv_part.p, st, tol, kScaled);
                 FTLM_CUDA(cudaGetLastError());
                 LzUpd<VT> U = ua[q];
                 U.has_prev = j > 0;
                 count_launch();
                 if (up_vec == 4)
-                    lzp_update<VT, ST, 4><<<up_grid, up_threads, 0, ss>>>(U);
+                    lzp_update<VT, ST, 4><<<(unsigned)up_runs, up_threads, 0, ss>>>(U);
                 else
-                    lzp_update<VT, ST, 1><<<up_grid, up_threads, 0, ss>>>(U);
+                    lzp_update<VT, ST, 1><<<(unsigned)up_runs, up_threads, 0, ss>>>(U);
                 FTLM_CUDA(cudaGetLastError());
                 count_launch();
-                lzp_finalize<<<fin_grid, kFinThreads, 0, ss>>>(2, j, K, B, up_grid, up_chunk, d_ut.p, d_ut.p + P, up_part.p,
-                                                          st, tol, kScaled);
+                lzp_finalize<<<fin_grid, kFinThreads, 0, ss>>>(2, j, K, B, 0, d_ut.p, d_ut.p + P, up_part.p, st, tol, kScaled);
                 FTLM_CUDA(cudaGetLastError());
             }
             return FTLM_OK;

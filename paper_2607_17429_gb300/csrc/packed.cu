@@ -409,14 +409,26 @@ std::mutex g_tune_mu;
 std::map<TuneKey, TuneVal> g_tuned;
 std::atomic<int> g_autotune{0};
 
+// Tiles of every part.  Large parts take the geometry's tiles (four representatives per warp: 1 to 3 %
+// over one per warp in FP64 and FP16 at 1.3e6 representatives).  Below eight such tiles per CTA the last
+// round counts: one representative per warp; below that a part is spread over all CTAs (18
+// representatives of the s = 1/2 icosahedron, FP64, on one SM's FP64 pipe before: 118 us a call, 39 us
+// spread; 1.7e3 of the s = 1 cuboctahedron, on 17 CTAs before: 186 us, 55 us).  The one-thread kernel takes
+// whole warps.  A part's tiles depend on the part alone, so its partial sums are the same in any mix.
 template <typename VT>
 void hvp_retile(HvpPlan<VT> &plan, std::vector<HvpPart<VT>> &parts) {
     uint64_t tiles = 0;
+    const uint64_t ctas = (uint64_t)std::max(1, plan.geo.grid);
     plan.tile0.clear();
     plan.ntile.clear();
     for (auto &p : parts) {
         p.tile0 = tiles;
-        const uint64_t nt = (p.n_reps + plan.geo.tile_reps - 1) / plan.geo.tile_reps;
+        uint64_t per = std::max<uint64_t>(1, (p.n_reps + ctas - 1) / ctas);
+        if (plan.ops->tile_fixed) per = (per + 31) / 32 * 32;
+        else if (per >= 32 * (uint64_t)plan.geo.warps) per = plan.geo.tile_reps;
+        else per = std::min<uint64_t>(plan.geo.warps, per);
+        p.tile_reps = (int)std::min<uint64_t>(plan.geo.tile_reps, per);
+        const uint64_t nt = (p.n_reps + p.tile_reps - 1) / p.tile_reps;
         plan.tile0.push_back(tiles);
         plan.ntile.push_back(nt);
         tiles += nt;
@@ -425,7 +437,6 @@ void hvp_retile(HvpPlan<VT> &plan, std::vector<HvpPart<VT>> &parts) {
     HvpArgs<VT> &a = plan.a;
     a.n_parts = (int)parts.size();
     a.n_tiles = tiles;
-    a.tile_reps = plan.geo.tile_reps;
     a.nbuf = plan.geo.nbuf;
     a.tma = plan.geo.tma;
     a.rho_smem = plan.geo.rho_smem;
