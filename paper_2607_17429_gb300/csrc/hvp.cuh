@@ -209,6 +209,14 @@ __device__ __forceinline__ int hvp_nth_set_bit(uint32_t m, int n) {
     return pos;
 }
 
+// warp minimum of a label (64 bits: the high words first, then the low words of the lanes that attain it)
+__device__ __forceinline__ uint32_t hvp_warp_min(uint32_t v) { return __reduce_min_sync(kFullMask, v); }
+__device__ __forceinline__ uint64_t hvp_warp_min(uint64_t v) {
+    const unsigned hi = __reduce_min_sync(kFullMask, (unsigned)(v >> 32));
+    const unsigned lo = __reduce_min_sync(kFullMask, (unsigned)(v >> 32) == hi ? (unsigned)v : ~0u);
+    return ((uint64_t)hi << 32) | lo;
+}
+
 // ---------------------------------------------------------------- exact-product dot accumulation
 
 // FP32 vectors: x*y exactly as (p, e) with p = fl(xy), e = fma(x, y, -p); the
@@ -613,50 +621,46 @@ __global__ void __launch_bounds__(hvp_max_threads<VT, SH>(), 1) hvp_kernel(const
                 }
                 LT my_rp = 0;
                 int my_g = 0;
-                // one flip's orbit minimum over the warp; FL: also the spin-flipped candidates
-                // (G x Z_2, elements (g, 1) after all of G: index 128 + g)
+                // One flip's orbit minimum over the warp, then the smallest element that attains it (a minimum
+                // and a few compares instead of a tracked index per candidate).  FL: also the spin-flipped
+                // candidates (G x Z_2, elements (g, 1) after all of G: index 128 + g).  The flip reverses the
+                // order of labels, so their minimum is the flip of the largest candidate; it wins only when
+                // strictly smaller, as (g, 1) comes after all of G.
                 auto search = [&](int j, auto FL) {
                     const int e = __shfl_sync(kFullMask, my_e, j);
                     const int sg = HALF ? 1 : __shfl_sync(kFullMask, my_sg, j);
-                    LT best = 0;
-                    int bg = 0;
                     LT cands[GPL];
 #pragma unroll
                     for (int c = 0; c < GPL; ++c) {
                         const int g = lane + 32 * c;
-                        LT cand;
                         if (HALF) {
-                            cand = I[c] ^ s_dtab[e * kMaxG + g];
+                            cands[c] = I[c] ^ s_dtab[e * kMaxG + g];
                         } else {
                             const LT dlt = s_dtab[e * kMaxG + g];
-                            cand = sg > 0 ? I[c] + dlt : I[c] - dlt;
-                        }
-                        cands[c] = cand;
-                        if (c == 0 || cand < best) {
-                            best = cand;
-                            bg = g;
+                            cands[c] = sg > 0 ? I[c] + dlt : I[c] - dlt;
                         }
                     }
-                    if constexpr (decltype(FL)::value) {  // after all of G, in index order: strict <
+                    LT lo = cands[0];
 #pragma unroll
-                        for (int c = 0; c < GPL; ++c) {
-                            const LT cf = HALF ? (cands[c] ^ (LT)a.flipc) : ((LT)a.flipc - cands[c]);
-                            if (cf < best) {
-                                best = cf;
-                                bg = (lane + 32 * c) | 128;
-                            }
+                    for (int c = 1; c < GPL; ++c) lo = min(lo, cands[c]);
+                    LT mn = hvp_warp_min(lo), hit = mn;
+                    int fl = 0;
+                    if constexpr (decltype(FL)::value) {
+                        LT hi = cands[0];
+#pragma unroll
+                        for (int c = 1; c < GPL; ++c) hi = max(hi, cands[c]);
+                        const LT mx = ~hvp_warp_min((LT)~hi);
+                        const LT mf = HALF ? (mx ^ (LT)a.flipc) : ((LT)a.flipc - mx);
+                        if (mf < mn) {
+                            mn = mf;
+                            hit = mx;
+                            fl = 128;
                         }
                     }
-                    LT mn;
-                    if (HALF) {
-                        mn = (LT)__reduce_min_sync(kFullMask, (unsigned)best);
-                    } else {
-                        const unsigned hi = __reduce_min_sync(kFullMask, (unsigned)((uint64_t)best >> 32));
-                        const unsigned lo = __reduce_min_sync(
-                            kFullMask, (unsigned)((uint64_t)best >> 32) == hi ? (unsigned)best : ~0u);
-                        mn = (LT)(((uint64_t)hi << 32) | (uint64_t)lo);
-                    }
-                    const int gs = (int)__reduce_min_sync(kFullMask, best == mn ? (unsigned)bg : 0xffffu);
+                    unsigned gi = 0xffffu;
+#pragma unroll
+                    for (int c = GPL - 1; c >= 0; --c) gi = cands[c] == hit ? (unsigned)(lane + 32 * c) : gi;
+                    const int gs = (int)__reduce_min_sync(kFullMask, gi) | fl;
                     if (lane == j) {
                         my_rp = mn;
                         my_g = gs;
