@@ -46,6 +46,26 @@ __global__ void index_records(const uint64_t *labels, const uint16_t *stab_id, u
 
 }  // namespace
 
+// Build-mode plan over parts whose entries go to fixed-stride slots (no count pass): launch it with
+// hvp_launch_plan, in the stream of the H·v that reads them.
+ftlm_status flips_build(const ftlm_sector *s, std::vector<HvpPart<float>> &parts, const HvpPart<float> *d_parts, int *err,
+                        HvpPlan<float> &plan) {
+    PackedSet ps;  // no blocks, no vectors
+    ps.K = 1;
+    ps.W = 1;
+    ps.dims[0] = 1;
+    plan.mode = 2;
+    hvp_fill_common<float>(s, &ps, 1, 4, plan.a);
+    plan.a.err = err;
+    plan.ops = hvp_ops_build(s->G <= 64 ? 2 : 4, s->half);
+    if (!plan.ops) return fail(FTLM_EUNSUPPORTED, "no build kernel for |G| = %d", s->G);
+    ftlm_status st = hvp_choose_geom<float>(plan.ops, plan.a, false, plan.geo);
+    if (st != FTLM_OK) return st;
+    hvp_retile<float>(plan, parts);
+    plan.a.parts = d_parts;
+    return FTLM_OK;
+}
+
 ftlm_status entry_table_build(ftlm_sector *s, cudaStream_t stream) {
     if (s->d_ent) return FTLM_OK;
     const uint64_t n = s->n_reps;
@@ -86,7 +106,7 @@ ftlm_status entry_table_build(ftlm_sector *s, cudaStream_t stream) {
         a.err = err.p;
         HvpPart<float> part;
         memset(&part, 0, sizeof(part));
-        part.n_reps = n;
+        part.n_reps = part.n_all = n;
         part.rec = rec.p;
         part.bucket = s->d_bucket;
         part.n_buckets = s->n_buckets;

@@ -97,7 +97,8 @@ __device__ __forceinline__ void static_for(F &&f) {
 
 template <typename VT>
 struct HvpPart {
-    uint64_t n_reps;
+    uint64_t n_reps;         // representatives of this part
+    uint64_t n_all;          // representatives of its sector (rows of x)
     uint64_t tile0;          // first tile of this part in the launch's tile order
     int tile_reps;           // representatives per tile of this part
     const HvRec *rec;        // [n_reps], ascending labels; rec.off = index * W
@@ -110,8 +111,11 @@ struct HvpPart {
     const VT *Pj[kPMaxK];    // block k: [n_sid][d_k][d_k] projector V V^T
     const void *x;           // lifted [n_reps * W][B] of the storage type (VT, or FP16 with VT = float)
     void *y;
+    uint64_t rep0;           // first representative of this part in rec and eoff (0: the whole sector)
     const uint64_t *eoff;    // entry table of the sector ([n_reps + 1]; table and build modes)
     HvEntry *ent;            // [n_entries] (read in table mode, written in build mode)
+    uint8_t *ecnt;           // instead of eoff: flips per representative of this part, whose entries
+    int estride;             // start at (index in the part) * estride
 };
 
 template <typename VT>
@@ -499,7 +503,7 @@ __global__ void __launch_bounds__(hvp_max_threads<VT, SH>(), 1) hvp_kernel(const
         const ST *__restrict__ x = static_cast<const ST *>(P.x);
         ST *__restrict__ y = static_cast<ST *>(P.y);
         for (uint64_t rep = r0 + wid; rep < r1 && !dead; rep += warps) {
-            const HvRec rr = rec[rep];
+            const HvRec rr = rec[P.rep0 + rep];
             const int sid = (int)rr.sid;
             const size_t seg = (size_t)rr.off * B;  // first element of r's W rows
             if (MODE != 2 && sid != 0 && __ldg(P.wtab + sid) == 0) {  // no block has rows for this orbit: y~(r) = 0
@@ -537,8 +541,8 @@ __global__ void __launch_bounds__(hvp_max_threads<VT, SH>(), 1) hvp_kernel(const
                 }
                 diag4 = __reduce_add_sync(kFullMask, diag4);
                 diag = a.J * (VT)diag4 * (VT)0.25;
-                const uint64_t e0 = __ldg(P.eoff + rep);
-                nf = (int)(__ldg(P.eoff + rep + 1) - e0);
+                const uint64_t e0 = P.ecnt ? rep * (uint64_t)P.estride : __ldg(P.eoff + P.rep0 + rep);
+                nf = P.ecnt ? (int)__ldg(P.ecnt + rep) : (int)(__ldg(P.eoff + P.rep0 + rep + 1) - e0);
                 n_flips += (unsigned long long)nf;
                 for (int base = lane; base < nf; base += 32) {
                     const uint2 raw = __ldg(reinterpret_cast<const uint2 *>(P.ent + e0 + base));
@@ -593,8 +597,12 @@ __global__ void __launch_bounds__(hvp_max_threads<VT, SH>(), 1) hvp_kernel(const
             diag = a.J * (VT)diag4 * (VT)0.25;
             nf = __popc(m[0]) + __popc(m[1]) + __popc(m[2]) + __popc(m[3]);
             n_flips += (unsigned long long)nf;
-            if (MODE == 2 && lane == 0 && (uint64_t)nf != P.eoff[rep + 1] - P.eoff[rep])
-                atomicOr(a.err, kErrMissingRep);  // the count pass and the kernel disagree
+            if (MODE == 2 && lane == 0) {
+                if (P.ecnt)
+                    P.ecnt[rep] = (uint8_t)nf;  // at most kMaxBonds * 2 = 128
+                else if ((uint64_t)nf != P.eoff[rep + 1] - P.eoff[rep])
+                    atomicOr(a.err, kErrMissingRep);  // the count pass and the kernel disagree
+            }
 
             // 3-4. search and lookup, 32 flips per round; records to shared memory
             for (int base = 0; base < nf; base += 32) {
@@ -704,8 +712,9 @@ __global__ void __launch_bounds__(hvp_max_threads<VT, SH>(), 1) hvp_kernel(const
                         my_c = (VT)0;
                     }
                     if constexpr (MODE == 2) {
-                        const uint64_t slot = P.eoff[rep] + (uint64_t)(base + lane);
-                        if (slot < P.eoff[rep + 1]) {
+                        const uint64_t first = P.ecnt ? rep * (uint64_t)P.estride : P.eoff[rep];
+                        const uint64_t slot = first + (uint64_t)(base + lane);
+                        if (P.ecnt ? base + lane < P.estride : slot < P.eoff[rep + 1]) {
                             HvEntry en;
                             en.tgt = idx_f;
                             en.g = (uint8_t)my_g;
@@ -881,30 +890,35 @@ size_t hvp_smem_t(const HvpArgs<VT> &a, int warps, int nbuf) {
         .total;
 }
 
-// CTAs per SM for the given geometry (0 if it does not fit); sets the shared-memory attribute.
-template <typename VT, typename ST, class SH, int GPL, bool HALF, int MODE>
-int hvp_occupancy_t(const HvpArgs<VT> &a, int warps, int nbuf) {
-    auto kern = hvp_kernel<VT, ST, SH, GPL, HALF, MODE>;
-    if (warps * 32 > hvp_max_threads<VT, SH>()) return 0;
-    const size_t smem = hvp_smem_t<VT, ST, SH, GPL, HALF, MODE>(a, warps, nbuf);
+// CTAs per SM of a kernel at the given warps and shared memory (0 if it does not fit).  The attribute is
+// only ever raised: a plan made on another thread never invalidates a launch.
+template <auto Kern>
+int hvp_fit_occupancy(int warps, size_t smem) {
     int dev = 0, max_smem = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (smem > (size_t)max_smem) return 0;
-    {  // the attribute is only ever raised: a plan made on another thread never invalidates a launch
+    {
         static std::mutex mu;
         static int raised[64] = {};
         std::lock_guard<std::mutex> lk(mu);
         const int d = dev & 63;
         if ((int)smem > raised[d]) {
-            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+            if (cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
                 return 0;
             raised[d] = (int)smem;
         }
     }
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, warps * 32, smem) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, Kern, warps * 32, smem) != cudaSuccess) return 0;
     return per_sm;
+}
+
+template <typename VT, typename ST, class SH, int GPL, bool HALF, int MODE>
+int hvp_occupancy_t(const HvpArgs<VT> &a, int warps, int nbuf) {
+    if (warps * 32 > hvp_max_threads<VT, SH>()) return 0;
+    return hvp_fit_occupancy<hvp_kernel<VT, ST, SH, GPL, HALF, MODE>>(
+        warps, hvp_smem_t<VT, ST, SH, GPL, HALF, MODE>(a, warps, nbuf));
 }
 
 template <typename VT, typename ST, class SH, int GPL, bool HALF, int MODE>

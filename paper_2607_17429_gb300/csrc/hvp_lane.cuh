@@ -125,9 +125,9 @@ __global__ void __launch_bounds__(kLaneThreads) hvp_lane_kernel(const __grid_con
         if (rep >= P.n_reps || (int)threadIdx.x >= P.tile_reps) continue;
         const ST *__restrict__ x = static_cast<const ST *>(P.x);
         ST *__restrict__ y = static_cast<ST *>(P.y);
-        const uint64_t n_elems = P.n_reps * (uint64_t)D;
+        const uint64_t n_elems = P.n_all * (uint64_t)D;
         const bool vec = (reinterpret_cast<uintptr_t>(x) & 15) == 0;
-        const HvRec rr = P.rec[rep];
+        const HvRec rr = P.rec[P.rep0 + rep];
         const int sid = (int)rr.sid;
         const size_t seg = rr.off;  // W = D rows, B = 1
         if (sid != 0 && __ldg(P.wtab + sid) == 0) {
@@ -141,7 +141,8 @@ __global__ void __launch_bounds__(kLaneThreads) hvp_lane_kernel(const __grid_con
             diag4 += (2 * (int)hvp_digit(lab, s_bond[2 * e], a.bits) - a.two_s) *
                      (2 * (int)hvp_digit(lab, s_bond[2 * e + 1], a.bits) - a.two_s);
         const VT diag = a.J * (VT)diag4 * (VT)0.25;
-        const uint64_t e0 = __ldg(P.eoff + rep), e1 = __ldg(P.eoff + rep + 1);
+        const uint64_t e0 = P.ecnt ? rep * (uint64_t)P.estride : __ldg(P.eoff + P.rep0 + rep);
+        const uint64_t e1 = P.ecnt ? e0 + __ldg(P.ecnt + rep) : __ldg(P.eoff + P.rep0 + rep + 1);
         n_flips += e1 - e0;
         VT z[D];
 #pragma unroll
@@ -204,7 +205,7 @@ __global__ void __launch_bounds__(kLaneThreads) hvp_lane_kernel(const __grid_con
             }
         }
         VT xo[D];
-        lane_row<VT, ST, D>(x, rep, n_elems, vec, xo);
+        lane_row<VT, ST, D>(x, P.rep0 + rep, n_elems, vec, xo);
 #pragma unroll
         for (int g = 0; g < D; ++g) {
             const VT xv = xo[g];
@@ -228,23 +229,7 @@ size_t hvp_lane_smem(const HvpArgs<VT> &a) {
 template <typename VT, typename ST, int D>
 int hvp_lane_occupancy_t(const HvpArgs<VT> &a, int warps, int) {
     if (warps * 32 != kLaneThreads) return 0;
-    auto kern = hvp_lane_kernel<VT, ST, D>;
-    const size_t smem = hvp_lane_smem<VT, ST, D>(a);
-    {  // raised only, as for the warp kernels
-        static std::mutex mu;
-        static int raised[64] = {};
-        int dev = 0;
-        cudaGetDevice(&dev);
-        std::lock_guard<std::mutex> lk(mu);
-        if ((int)smem > raised[dev & 63]) {
-            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-                return 0;
-            raised[dev & 63] = (int)smem;
-        }
-    }
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kLaneThreads, smem) != cudaSuccess) return 0;
-    return per_sm;
+    return hvp_fit_occupancy<hvp_lane_kernel<VT, ST, D>>(warps, hvp_lane_smem<VT, ST, D>(a));
 }
 
 template <typename VT, typename ST, int D>

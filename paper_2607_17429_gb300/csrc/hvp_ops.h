@@ -1,8 +1,11 @@
 // Compiled packed H·v kernels: one entry per (shape, elements per lane, label width).
 #pragma once
 
+#include <string.h>
+
 #include <vector>
 
+#include "hvp_flow.cuh"
 #include "hvp_lane.cuh"
 
 namespace ftlm {
@@ -37,6 +40,11 @@ struct HvpOps {
 // one thread per representative (table mode, one block, B = 1; hvp_lane.cuh)
 #define FTLM_HVP_LANE_OPS(VT, ST, D) \
     HvpOps<VT> { &hvp_lane_occupancy_t<VT, ST, D>, &hvp_lane_launch_t<VT, ST, D>, kLaneThreads, kLaneThreads }
+// table mode, multi-block shapes, FP32 arithmetic (hvp_flow.cuh)
+#define FTLM_HVP_FLOW_OPS(ST, SH, CL, BC)                                                      \
+    HvpOps<float> {                                                                             \
+        &hvp_flow_occupancy_t<ST, SH, CL, BC>, &hvp_flow_launch_t<ST, SH, CL, BC>, flow_threads<ST, SH, CL>(), 0 \
+    }
 #define FTLM_HVP_OPS(VT, ST, SH, GPL, HALF) FTLM_HVP_OPS_M(VT, ST, SH, GPL, HALF, 0)
 
 template <typename VT>
@@ -59,6 +67,22 @@ ftlm_status hvp_plan(const ftlm_sector *s, const PackedSet *ps, std::vector<HvpP
                      HvpPlan<VT> &plan, cudaStream_t tune_stream);
 template <typename VT>
 ftlm_status hvp_launch_plan(const HvpPlan<VT> &plan, double *dot_part, cudaStream_t stream, bool timed);
+// the part as the build kernel sees it (no vectors, no blocks)
+template <typename VT>
+void hvp_copy_flips(const HvpPart<VT> &p, HvpPart<float> &b) {
+    memset(&b, 0, sizeof(b));
+    b.n_reps = p.n_reps;
+    b.n_all = p.n_all;
+    b.rec = p.rec;
+    b.bucket = p.bucket;
+    b.n_buckets = p.n_buckets;
+    b.bucket_shift = p.bucket_shift;
+    b.n_sid = p.n_sid;
+    b.rep0 = p.rep0;
+    b.ent = p.ent;
+    b.ecnt = p.ecnt;
+    b.estride = p.estride;
+}
 // pieces of a plan (packed.cu): sector-wide arguments, geometry, tile order
 template <typename VT>
 void hvp_fill_common(const ftlm_sector *s, const PackedSet *ps, int B, int esize, HvpArgs<VT> &a);
@@ -66,6 +90,15 @@ template <typename VT>
 ftlm_status hvp_choose_geom(const HvpOps<VT> *ops, HvpArgs<VT> a, bool tma, HvpGeom &geo);
 template <typename VT>
 void hvp_retile(HvpPlan<VT> &plan, std::vector<HvpPart<VT>> &parts);
+// entries.cu: flips of the parts' representatives (rep0 .. rep0 + n_reps - 1) into ent, ecnt and estride of each part;
+// d_parts: device copy of the parts when there are several
+constexpr size_t kSplitBytes = 128u << 20;  // entry workspace of one H·v on the search path
+inline int flip_stride(const ftlm_sector *s) { return s->grp.n_bonds() * (s->two_s == 1 ? 1 : 2); }
+ftlm_status flips_build(const ftlm_sector *s, std::vector<HvpPart<float>> &parts, const HvpPart<float> *d_parts, int *err,
+                        HvpPlan<float> &plan);
+// scratch of one call, from a pool of at most kPoolBytes kept between calls (packed.cu)
+ftlm_status scratch_alloc(void **p, size_t bytes, cudaStream_t stream);
+void scratch_trim();
 // entries.cu: the sector's optional entry table
 ftlm_status entry_table_build(ftlm_sector *s, cudaStream_t stream);
 void entry_table_free(ftlm_sector *s);
@@ -86,6 +119,12 @@ const HvpOps<float> *hvp_ops_wide_f16(int shape, bool half, int kind);
 const HvpOps<double> *hvp_ops_table_f64(int shape);
 const HvpOps<float> *hvp_ops_table_f32(int shape);
 const HvpOps<float> *hvp_ops_table_f16(int shape);
+// table mode of the multi-block shapes for an even B in 6..32 (hvp_flow.cuh): lanes per flip and the ops
+constexpr int flow_lanes(int B) { return B <= 8 ? 4 : B <= 16 ? 8 : 16; }
+const HvpOps<float> *hvp_ops_flow_ih_f32(int B);
+const HvpOps<float> *hvp_ops_flow_ih_f16(int B);
+const HvpOps<float> *hvp_ops_flow_other_f32(int shape, int B);
+const HvpOps<float> *hvp_ops_flow_other_f16(int shape, int B);
 // table mode, one thread per representative: single blocks (shapes D1..D5) at B = 1
 const HvpOps<double> *hvp_ops_lane_f64(int shape);
 const HvpOps<float> *hvp_ops_lane_f32(int shape);

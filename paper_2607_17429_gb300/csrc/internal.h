@@ -111,8 +111,18 @@ struct ftlm_group {
     ftlm::GroupData d;
 };
 
+namespace ftlm {
+// Live sectors; the last one to go returns the scratch pool's memory (packed.cu).
+struct SectorCount {
+    SectorCount();
+    ~SectorCount();
+    static std::atomic<int> n;
+};
+}  // namespace ftlm
+
 // Packed-label sector on the device (basis.cu).
 struct ftlm_sector {
+    ftlm::SectorCount live;
     std::atomic<int> refs{1};
     // the group acting on the sector: G, or G x Z_2 with the spin flip at M = 0 (flip = 1), whose
     // element g + z |G| is stored as the signed permutation pi_g(k) + z N and whose irreps are

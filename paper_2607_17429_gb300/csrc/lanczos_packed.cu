@@ -417,6 +417,15 @@ __global__ void __launch_bounds__(32 * kFinSlices)
     }
 }
 
+// flips of a part in fixed-stride slots at `at`, counts behind them
+template <typename VT>
+void lz_use_flips(HvpPart<VT> &part, uint8_t *at, int stride) {
+    part.eoff = nullptr;
+    part.ent = reinterpret_cast<HvEntry *>(at);
+    part.ecnt = at + (size_t)part.n_reps * stride * sizeof(HvEntry);
+    part.estride = stride;
+}
+
 template <typename VT, typename ST>
 ftlm_status lzp_start_launch(int K, const LzArgs<VT> &a, int grid, cudaStream_t st) {
     count_launch();
@@ -432,6 +441,19 @@ ftlm_status lzp_start_launch(int K, const LzArgs<VT> &a, int grid, cudaStream_t 
 
 
 }  // namespace
+
+// Searching once and reading the flips in every step replaces a search per step (six s = 3/2
+// icosahedron sectors at 24 chains, 14 steps: 35.5 ms with a search in every H·v, 22.6 ms so; one block of
+// the 4x6 lattice at 4 chains: 2.0 and 1.4 ms).  The table has fixed-stride slots, eight bytes per possible
+// flip.  It is built where it takes at most twice the call's vectors, or 64 MB: single blocks of few
+// rows on large sectors (one chain of the s = 3/2 dodecahedron: 480 bytes a representative for 60 of
+// vectors) keep searching.
+size_t lanczos_flip_bytes(const ftlm_sector *sec, const PackedSet *ps, int B, int esize) {
+    if (sec->d_ent) return 0;
+    const size_t bytes = (size_t)sec->n_reps * ((size_t)flip_stride(sec) * sizeof(HvEntry) + 1);
+    const size_t vectors = 3 * (size_t)ps->rows * B * esize;
+    return bytes <= std::max<size_t>(64u << 20, 2 * vectors) ? (bytes + 255) / 256 * 256 : 0;
+}
 
 template <typename VT, typename ST>
 ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_steps, uint64_t seed, int rng,
@@ -495,6 +517,46 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
     DevBuf<int> derr;
     FTLM_CUDA(derr.alloc(1));
     FTLM_CUDA(cudaMemsetAsync(derr.p, 0, sizeof(int), stream));
+    // ---- flips of the sectors without an entry table, searched once for all steps
+    DevBuf<uint8_t> flips;
+    DevBuf<HvpPart<float>> d_fparts;
+    std::vector<size_t> flip_at(P, SIZE_MAX);  // a part's place in flips
+    {
+        size_t total = 0;
+        bool all = true;
+        std::vector<int> which;
+        for (int p = 0; p < P; ++p) {
+            if (sets[p].sec->d_ent || sets[p].sec->n_reps == 0) continue;
+            const size_t by = lanczos_flip_bytes(sets[p].sec, sets[p].ps, Bmax, (int)sizeof(ST));
+            all = all && by;
+            flip_at[p] = total;
+            total += by;
+            which.push_back(p);
+        }
+        if (!which.empty() && (!all || flips.alloc(total) != cudaSuccess)) {
+            cudaGetLastError();
+            flip_at.assign(P, SIZE_MAX);
+            which.clear();
+        }
+        if (!which.empty()) {
+            std::vector<HvpPart<float>> fparts;
+            for (int p : which) {
+                HvpPart<VT> part;
+                hvp_part_of<VT>(sets[p].sec, sets[p].ps, sets[p].blocks, nullptr, nullptr, part);
+                lz_use_flips(part, flips.p + flip_at[p], flip_stride(sets[p].sec));
+                fparts.emplace_back();
+                hvp_copy_flips(part, fparts.back());
+            }
+            if (fparts.size() > 1) FTLM_CUDA(d_fparts.alloc(fparts.size()));
+            HvpPlan<float> build;
+            ftlm_status sb = flips_build(sets[0].sec, fparts, d_fparts.p, derr.p, build);
+            if (sb != FTLM_OK) return sb;
+            if (fparts.size() > 1)
+                FTLM_CUDA(cudaMemcpyAsync(d_fparts.p, fparts.data(), fparts.size() * sizeof(HvpPart<float>),
+                                          cudaMemcpyHostToDevice, stream));
+            if ((sb = hvp_launch_plan<float>(build, nullptr, stream, false)) != FTLM_OK) return sb;
+        }
+    }
     int dev = 0, sms = kNumSMs;
     FTLM_CUDA(cudaGetDevice(&dev));
     FTLM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -513,9 +575,12 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
         DevBuf<HvpPart<VT>> d_hparts[3];
         for (int q = 0; q < 3; ++q) {
             hparts[q].resize(P);
-            for (int p = 0; p < P; ++p)
+            for (int p = 0; p < P; ++p) {
                 hvp_part_of<VT>(sets[p].sec, sets[p].ps, sets[p].blocks, vb[q].p + row0[p] * B,
                                 vb[(q + 1) % 3].p + row0[p] * B, hparts[q][p]);
+                if (flip_at[p] != SIZE_MAX)
+                    lz_use_flips(hparts[q][p], flips.p + flip_at[p], flip_stride(sets[p].sec));
+            }
             ftlm_status s0 = hvp_plan<VT>(sets[0].sec, ps0, hparts[q], B, (int)sizeof(ST), plan[q], stream);
             if (s0 != FTLM_OK) return s0;
             plan[q].a.err = derr.p;  // this call's own error word (launches on the same sector may run concurrently)

@@ -17,6 +17,10 @@ struct LzSetIn {
     int n_steps = 0;  // this set's step limit (0: the launch's n_steps; never above it)
 };
 
+// Bytes of the flip table a Lanczos call on the search path builds for one set and keeps for its
+// steps; 0 when the sector has a table or the call does without one.
+size_t lanczos_flip_bytes(const ftlm_sector *sec, const PackedSet *ps, int B, int esize);
+
 // R chains on every block of every set, n_steps steps (Section 2.2).  alpha,
 // beta: host [n_sets][K][R][n_steps]; steps_done: host [n_sets][K][R].  All
 // sets share the group, spin, block shape and irreps.  esize: bytes of a stored

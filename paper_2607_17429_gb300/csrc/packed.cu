@@ -314,7 +314,7 @@ template <typename VT>
 void hvp_part_of(const ftlm_sector *s, const PackedSet *ps, const ftlm_basis *const *blocks, const void *x, void *y,
                  HvpPart<VT> &p) {
     memset(&p, 0, sizeof(p));
-    p.n_reps = s->n_reps;
+    p.n_reps = p.n_all = s->n_reps;
     p.rec = ps->d_rec;
     p.bucket = s->d_bucket;
     p.n_buckets = s->n_buckets;
@@ -532,8 +532,8 @@ ftlm_status hvp_plan(const ftlm_sector *s, const PackedSet *ps, std::vector<HvpP
     HvpArgs<VT> &a = plan.a;
     hvp_fill_common<VT>(s, ps, B, esize, a);
     const int gpl = s->G <= 64 ? 2 : 4;
-    int mode = 1;  // the entry-table path when every part's sector has a table
-    for (auto &p : parts) mode = mode && p.eoff && p.ent;
+    int mode = 1;  // the entry-table path when every part has a table
+    for (auto &p : parts) mode = mode && p.ent && (p.eoff || p.ecnt);
     plan.mode = mode;
     plan.ops = hvp_ops<VT>(ps->shape, gpl, s->half, esize, mode);
     if (mode == 1 && ps->K == 1 && B == 1) {  // one thread per representative
@@ -550,6 +550,20 @@ ftlm_status hvp_plan(const ftlm_sector *s, const PackedSet *ps, std::vector<HvpP
     if (!plan.ops)
         return fail(FTLM_EUNSUPPORTED, "no compiled packed kernel for shape %d with |G| = %d", ps->shape, s->G);
     bool tma = (B * esize) % 16 == 0;
+    // Two right-hand sides per lane: an even B from 6 on (below, most of a warp's flips would be idle; odd
+    // B breaks the 8-byte row loads), segments that start on 16 bytes.
+    if constexpr (sizeof(VT) == 4) {
+        if (mode == 1 && ps->K > 1 && (ps->W * B * esize) % 16 == 0) {
+            const HvpOps<VT> *flow = ps->shape == kShapeIh ? (esize == 2 ? hvp_ops_flow_ih_f16(B) : hvp_ops_flow_ih_f32(B))
+                                     : esize == 2          ? hvp_ops_flow_other_f16(ps->shape, B)
+                                                           : hvp_ops_flow_other_f32(ps->shape, B);
+            if (flow) {
+                plan.ops = flow;
+                a.stage_elems = 32 / flow_lanes(B) * a.slot_elems;
+                tma = true;
+            }
+        }
+    }
     uint64_t n_reps_total = 0;
     for (auto &p : parts) {
         tma = tma && ((uintptr_t)p.x % 16) == 0;
@@ -633,22 +647,66 @@ ftlm_status lift_impl(const ftlm_sector *s, const PackedSet *ps, const ftlm_basi
     return FTLM_OK;
 }
 
+// ---------------------------------------------------------------- scratch pool
+//
+// Scratch of one call comes from a stream-ordered pool per device that keeps up to kPoolBytes between
+// calls (the default pool gives everything back at each synchronisation, and mapping it again cost
+// 1.1 ms for the 500 MB of an FP64 block's lift); scratch_trim returns it when the last sector goes.
+constexpr uint64_t kPoolBytes = 1ull << 30;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[64] = {};
+
+ftlm_status scratch_alloc(void **p, size_t bytes, cudaStream_t stream) {
+    int dev = 0;
+    FTLM_CUDA(cudaGetDevice(&dev));
+    cudaMemPool_t pool = nullptr;
+    {
+        std::lock_guard<std::mutex> lk(g_pool_mu);
+        cudaMemPool_t &slot = g_pool[dev & 63];
+        if (!slot) {
+            cudaMemPoolProps pr;
+            memset(&pr, 0, sizeof(pr));
+            pr.allocType = cudaMemAllocationTypePinned;
+            pr.location.type = cudaMemLocationTypeDevice;
+            pr.location.id = dev;
+            FTLM_CUDA(cudaMemPoolCreate(&slot, &pr));
+            uint64_t keep = kPoolBytes;
+            FTLM_CUDA(cudaMemPoolSetAttribute(slot, cudaMemPoolAttrReleaseThreshold, &keep));
+        }
+        pool = slot;
+    }
+    FTLM_CUDA(cudaMallocFromPoolAsync(p, bytes, pool, stream));
+    return FTLM_OK;
+}
+
+SectorCount::SectorCount() { n.fetch_add(1); }
+SectorCount::~SectorCount() {
+    if (n.fetch_sub(1) == 1) scratch_trim();
+}
+std::atomic<int> SectorCount::n{0};
+
+void scratch_trim() {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    for (cudaMemPool_t p : g_pool)
+        if (p) cudaMemPoolTrimTo(p, 0);
+}
+
 // One block through the packed kernel: lift x, H·v, lower y (stream-ordered scratch).
 template <typename VT>
 ftlm_status hv_block(const ftlm_basis *b, int B, const VT *x, VT *y, cudaStream_t stream) {
     const PackedSet *ps = b->ps;
     const size_t n = ps->rows * (size_t)B;
     VT *xl = nullptr, *yl = nullptr;
-    FTLM_CUDA(cudaMallocAsync((void **)&xl, std::max<size_t>(n, 1) * sizeof(VT), stream));
-    cudaError_t e = cudaMallocAsync((void **)&yl, std::max<size_t>(n, 1) * sizeof(VT), stream);
-    if (e != cudaSuccess) {
+    ftlm_status st = scratch_alloc((void **)&xl, std::max<size_t>(n, 1) * sizeof(VT), stream);
+    if (st != FTLM_OK) return st;
+    if ((st = scratch_alloc((void **)&yl, std::max<size_t>(n, 1) * sizeof(VT), stream)) != FTLM_OK) {
         cudaFreeAsync(xl, stream);
-        return fail(e == cudaErrorMemoryAllocation ? FTLM_ENOMEM : FTLM_ECUDA, "H·v scratch: %s", cudaGetErrorString(e));
+        return st;
     }
     const ftlm_basis *one[1] = {b};
     VT *xb[1] = {const_cast<VT *>(x)};
     VT *yb[1] = {y};
-    ftlm_status st = lift_impl<VT>(b->sec, ps, one, B, xb, xl, 1, stream);
+    st = lift_impl<VT>(b->sec, ps, one, B, xb, xl, 1, stream);
     if (st == FTLM_OK) {
         std::vector<HvpPart<VT>> parts(1);
         hvp_part_of<VT>(b->sec, ps, one, xl, yl, parts[0]);
@@ -663,11 +721,66 @@ ftlm_status hv_block(const ftlm_basis *b, int B, const VT *x, VT *y, cudaStream_
     return st;
 }
 
+// Search path of a multi-block set with FP32 arithmetic: the flips of a run of representatives are
+// searched into an entry workspace by the build kernel, then the table kernel reads them, run after
+// run.  (Search and contraction in one kernel share its 16 warps per SM and its instruction cache:
+// 15.7 ms a call for the ten icosidodecahedron irreps at B = 8, of which the search alone is 2.5 ms at the
+// build kernel's occupancy; 8.7 ms this way.)  Sums run in the table path's order, so both paths give
+// the same bits.  Single blocks and FP64 keep the search in the kernel: their contraction leaves the
+// integer pipes idle.  FTLM_ENOMEM (no workspace): the caller takes the one-kernel search.
+template <typename VT>
+ftlm_status hvp_run_split(const ftlm_sector *s, const PackedSet *ps, HvpPart<VT> part, int B, int esize, cudaStream_t stream) {
+    const int stride = flip_stride(s);
+    const uint64_t n = part.n_reps;
+    const uint64_t run = std::min<uint64_t>(n, std::max<uint64_t>(1, kSplitBytes / ((size_t)stride * sizeof(HvEntry))));
+    HvEntry *ent = nullptr;
+    const size_t ent_bytes = run * (size_t)stride * sizeof(HvEntry);
+    ftlm_status st = scratch_alloc((void **)&ent, ent_bytes + run, stream);
+    if (st != FTLM_OK) {
+        cudaGetLastError();
+        return st;
+    }
+    part.ent = ent;
+    part.eoff = nullptr;
+    part.ecnt = reinterpret_cast<uint8_t *>(ent) + ent_bytes;
+    part.estride = stride;
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    hv_timer_begin(stream, &e0, &e1);
+    HvpPlan<VT> plan;
+    HvpPlan<float> build;
+    for (uint64_t r = 0; r < n && st == FTLM_OK; r += run) {
+        part.rep0 = r;
+        part.n_reps = std::min<uint64_t>(run, n - r);
+        std::vector<HvpPart<VT>> parts{part};
+        std::vector<HvpPart<float>> bparts(1);
+        hvp_copy_flips(part, bparts[0]);
+        const bool fresh = r == 0 || part.n_reps != run;  // geometry and tiles of a full run, and of the last one
+        if (fresh)
+            st = flips_build(s, bparts, nullptr, s->d_err, build);
+        else
+            build.a.part0.rep0 = plan.a.part0.rep0 = r;
+        if (st == FTLM_OK) st = hvp_launch_plan<float>(build, nullptr, stream, false);
+        if (st == FTLM_OK && fresh) st = hvp_plan<VT>(s, ps, parts, B, esize, plan, stream);  // may time the kernel
+        if (st == FTLM_OK) st = hvp_launch_plan<VT>(plan, nullptr, stream, false);
+    }
+    hv_timer_end(stream, e0, e1, ps->rows * (uint64_t)B);
+    cudaFreeAsync(ent, stream);
+    return st;
+}
+
 template <typename VT>
 ftlm_status hvp_run_one(const ftlm_sector *s, const PackedSet *ps, const ftlm_basis *const *blocks, int B, int esize,
                         const void *x, void *y, cudaStream_t stream) {
     std::vector<HvpPart<VT>> parts(1);
     hvp_part_of<VT>(s, ps, blocks, x, y, parts[0]);
+    if constexpr (sizeof(VT) == 4) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;  // a graph holds one kernel and no scratch
+        if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) cudaGetLastError();
+        if (ps->K > 1 && ps->shape >= 0 && !s->d_ent && cap == cudaStreamCaptureStatusNone) {
+            const ftlm_status st = hvp_run_split<VT>(s, ps, parts[0], B, esize, stream);
+            if (st != FTLM_ENOMEM) return st;
+        }
+    }
     HvpPlan<VT> plan;
     ftlm_status st = hvp_plan<VT>(s, ps, parts, B, esize, plan, stream);
     if (st != FTLM_OK) return st;

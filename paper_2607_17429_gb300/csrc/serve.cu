@@ -187,13 +187,14 @@ void fail_job(ftlm_server *S, Job *J, ftlm_status st, const std::string &msg) {
     S->cv_done.notify_all();
 }
 
-// Bytes a job's Lanczos launch allocates: three packed vectors, the scale and
-// coefficient state, and the per-CTA dot partials.
+// Bytes a job's Lanczos launch allocates: three packed vectors, the flips it searches once for its
+// steps, the scale and coefficient state, and the per-CTA dot partials.
 size_t vector_bytes(const ftlm_basis *b, const ftlm_job &j) {
     const size_t e = j.dtype == FTLM_F64 ? 8 : (j.dtype == FTLM_F16 ? 2 : 4);
     const size_t B = (size_t)std::min(j.R, kMaxB);
     const size_t rows = b->ps ? b->ps->rows : b->dim;
-    return 3 * std::max<size_t>(rows, 1) * B * e + (2 * (size_t)j.n_steps + 16) * B * 8 + 4 * kNumSMs * B * 8 +
+    const size_t flips = b->ps ? lanczos_flip_bytes(b->sec, b->ps, (int)B, (int)e) : 0;
+    return 3 * std::max<size_t>(rows, 1) * B * e + flips + (2 * (size_t)j.n_steps + 16) * B * 8 + 4 * kNumSMs * B * 8 +
            (1u << 20);
 }
 
