@@ -557,6 +557,10 @@ ftlm_status build_block_impl(ftlm_sector *s, int irrep, cudaStream_t stream, ftl
     }
     b->h_ntab = ntab;
     std::vector<float> Vf(V.begin(), V.end()), sqf(sq.begin(), sq.end());
+    for (size_t t = 0; t < ns; ++t) {  // the inverses behind the roots
+        sq.push_back(1.0 / sq[t]);
+        sqf.push_back(1.0f / sqf[t]);
+    }
     b->rho_elems = rho_table_elems<double>(G, d);
     b->rho_elemsf = rho_table_elems<float>(G, d);
     std::vector<double> rhoT(b->rho_elems, 0.0);
@@ -570,17 +574,17 @@ ftlm_status build_block_impl(ftlm_sector *s, int irrep, cudaStream_t stream, ftl
                 rhoTf[((size_t)g * d + r) * RP + c] = (float)v;
             }
     FTLM_CUDA(cudaMalloc((void **)&b->d_ntab, ns));
-    FTLM_CUDA(cudaMalloc((void **)&b->d_sqrtS, ns * 8));
-    FTLM_CUDA(cudaMalloc((void **)&b->d_sqrtSf, ns * 4));
+    FTLM_CUDA(cudaMalloc((void **)&b->d_sqrtS, 2 * ns * 8));
+    FTLM_CUDA(cudaMalloc((void **)&b->d_sqrtSf, 2 * ns * 4));
     FTLM_CUDA(cudaMalloc((void **)&b->d_V, V.size() * 8));
     FTLM_CUDA(cudaMalloc((void **)&b->d_Vf, V.size() * 4));
     FTLM_CUDA(cudaMalloc((void **)&b->d_rhoT, rhoT.size() * 8));
     FTLM_CUDA(cudaMalloc((void **)&b->d_rhoTf, rhoTf.size() * 4));
     FTLM_CUDA(cudaMalloc((void **)&b->d_off, (s->n_reps + 1) * 8));
-    b->device_bytes = ns * 13 + V.size() * 12 + rhoT.size() * 8 + rhoTf.size() * 4 + (s->n_reps + 1) * 8;
+    b->device_bytes = ns * 25 + V.size() * 12 + rhoT.size() * 8 + rhoTf.size() * 4 + (s->n_reps + 1) * 8;
     FTLM_CUDA(cudaMemcpyAsync(b->d_ntab, ntab.data(), ns, cudaMemcpyHostToDevice, stream));
-    FTLM_CUDA(cudaMemcpyAsync(b->d_sqrtS, sq.data(), ns * 8, cudaMemcpyHostToDevice, stream));
-    FTLM_CUDA(cudaMemcpyAsync(b->d_sqrtSf, sqf.data(), ns * 4, cudaMemcpyHostToDevice, stream));
+    FTLM_CUDA(cudaMemcpyAsync(b->d_sqrtS, sq.data(), 2 * ns * 8, cudaMemcpyHostToDevice, stream));
+    FTLM_CUDA(cudaMemcpyAsync(b->d_sqrtSf, sqf.data(), 2 * ns * 4, cudaMemcpyHostToDevice, stream));
     FTLM_CUDA(cudaMemcpyAsync(b->d_V, V.data(), V.size() * 8, cudaMemcpyHostToDevice, stream));
     FTLM_CUDA(cudaMemcpyAsync(b->d_Vf, Vf.data(), Vf.size() * 4, cudaMemcpyHostToDevice, stream));
     FTLM_CUDA(cudaMemcpyAsync(b->d_rhoT, rhoT.data(), rhoT.size() * 8, cudaMemcpyHostToDevice, stream));

@@ -107,7 +107,7 @@ struct HvpPart {
     int bucket_shift;
     int n_sid;
     const uint8_t *wtab;     // [n_sid] sum over k of n_k(sid) (0: the orbit has no rows in the set)
-    const VT *sqrtS;         // [n_sid]
+    const VT *sqrtS;         // [n_sid], then the inverses [n_sid]
     const VT *Pj[kPMaxK];    // block k: [n_sid][d_k][d_k] projector V V^T
     const void *x;           // lifted [n_reps * W][B] of the storage type (VT, or FP16 with VT = float)
     void *y;
@@ -303,7 +303,9 @@ __device__ __forceinline__ unsigned long long f2_mul(unsigned long long a, unsig
     return d;
 }
 
-// z[beta] += cf * sum_gamma R[gamma * RP + beta] u[gamma] for beta < D.  FP32 with
+// z[beta] += cf * sum_gamma R[gamma * RP + beta] u[gamma] for beta < D.  FP64 (u scaled by the caller,
+// cf unused) adds every product to z: D^2 FP64 operations, and D less per flip than scaling the sums,
+// where the flip's factor is one (FP64 issue binds: 12 -> 9 operations per flip and column at D = 3).  FP32 with
 // D >= 2 runs pairs of output rows through fma.f32x2 (rows of R padded to RP,
 // an even count); otherwise scalar FMAs.  Same products and summation order
 // over gamma either way (the first product is a multiply, as a fused
@@ -338,19 +340,47 @@ __device__ __forceinline__ void hvp_rows(const VT *__restrict__ R, const VT (&u)
             z[D - 1] += cf * lo;
         }
     } else {
-        VT acc[D];
+        if constexpr (sizeof(VT) == 8) {
 #pragma unroll
-        for (int be = 0; be < D; ++be) acc[be] = (VT)0;
+            for (int ga = 0; ga < D; ++ga) {
+                VT row[RP];
+                load_row<VT, RP>(R + ga * RP, row);
 #pragma unroll
-        for (int ga = 0; ga < D; ++ga) {
-            VT row[RP];
-            load_row<VT, RP>(R + ga * RP, row);
+                for (int be = 0; be < D; ++be) z[be] += row[be] * u[ga];
+            }
+        } else {
+            VT acc[D];
 #pragma unroll
-            for (int be = 0; be < D; ++be) acc[be] += row[be] * u[ga];
+            for (int be = 0; be < D; ++be) acc[be] = (VT)0;
+#pragma unroll
+            for (int ga = 0; ga < D; ++ga) {
+                VT row[RP];
+                load_row<VT, RP>(R + ga * RP, row);
+#pragma unroll
+                for (int be = 0; be < D; ++be) acc[be] += row[be] * u[ga];
+            }
+#pragma unroll
+            for (int be = 0; be < D; ++be) z[be] += cf * acc[be];
         }
-#pragma unroll
-        for (int be = 0; be < D; ++be) z[be] += cf * acc[be];
     }
+}
+
+// FP64 factors of a flip: +-1 for s = 1/2 but for flips to symmetric orbits; signs are bit operations
+__device__ __forceinline__ bool hvp_unit64(double cf) {
+    return (__double2hiint(cf) & 0x7fffffff) == 0x3ff00000 && __double2loint(cf) == 0;
+}
+__device__ __forceinline__ double hvp_neg64(double v) {
+    return __hiloint2double(__double2hiint(v) ^ (int)0x80000000, __double2loint(v));
+}
+template <int D>
+__device__ __forceinline__ void hvp_sign64(double (&u)[D], bool neg) {
+#pragma unroll
+    for (int g = 0; g < D; ++g) u[g] = neg ? hvp_neg64(u[g]) : u[g];
+}
+template <int D>
+__device__ __forceinline__ void hvp_scale64(double (&u)[D], double cf) {
+#pragma unroll
+    for (int g = 0; g < D; ++g) u[g] *= cf;
 }
 
 // ---------------------------------------------------------------- storage conversions
@@ -440,7 +470,9 @@ __global__ void __launch_bounds__(hvp_max_threads<VT, SH>(), 1) hvp_kernel(const
     const int Q = 32 >> a.lgBT;        // flip groups per warp
     const int b = lane & (BT - 1);
     const int fg = lane >> a.lgBT;
-    const VT halfJ = a.J * (VT)0.5;
+    // J / 2 multiplies every flip's coefficient (FP32) or the sum over flips (FP64: factors of one stay free)
+    const VT halfJ = sizeof(VT) == 8 ? (VT)1 : a.J * (VT)0.5;
+    const VT zscale = sizeof(VT) == 8 ? a.J * (VT)0.5 : (VT)1;
     uint32_t parity = 0;               // bit i: phase parity of buffer i (bit kMaxBuf: own rows)
     uint32_t pending = 0;              // bit i: copies in flight into buffer i
     bool dead = false;                 // a wait ran out: no more work for this warp
@@ -786,18 +818,35 @@ __global__ void __launch_bounds__(hvp_max_threads<VT, SH>(), 1) hvp_kernel(const
                     const unsigned negj = (f_sg[j] & 128u) ? a.neg : 0u;  // (g*, 1) in a Gamma- block: -rho(g*)
                     const VT cf = f_c[j];
                     const ST *xs = stage + (size_t)buf * a.stage_elems + (size_t)fg * a.slot_elems + b;
-                    static_for<K>([&](auto kc) {
-                        constexpr int k = decltype(kc)::value;
-                        constexpr int D = SH::template D<k>;
-                        constexpr int Zk = SH::template Z<k>;
-                        constexpr int RP = rho_row(D);
-                        // R[gamma][beta] = rho_k(g*)[gamma][beta]; z_beta += cf sum_gamma R[gamma][beta] u_gamma
-                        const VT *R = rho_base + a.rho_off[k] + (size_t)g_j * D * RP;
-                        VT u[D];
+                    auto contract = [&](auto SC) {
+                        static_for<K>([&](auto kc) {
+                            constexpr int k = decltype(kc)::value;
+                            constexpr int D = SH::template D<k>;
+                            constexpr int Zk = SH::template Z<k>;
+                            constexpr int RP = rho_row(D);
+                            // R[gamma][beta] = rho_k(g*)[gamma][beta]; z_beta += cf sum_gamma R[gamma][beta] u_gamma
+                            const VT *R = rho_base + a.rho_off[k] + (size_t)g_j * D * RP;
+                            VT u[D];
 #pragma unroll
-                        for (int g2 = 0; g2 < D; ++g2) u[g2] = st_get<VT, ST>(xs[(Zk + g2) * B]);
-                        hvp_rows<VT, D, RP>(R, u, ((negj >> k) & 1u) ? -cf : cf, z + Zk);
-                    });
+                            for (int g2 = 0; g2 < D; ++g2) u[g2] = st_get<VT, ST>(xs[(Zk + g2) * B]);
+                            if constexpr (sizeof(VT) == 8) {
+                                const bool ng = (negj >> k) & 1u;
+                                if constexpr (decltype(SC)::value)
+                                    hvp_scale64<D>(u, ng ? hvp_neg64(cf) : cf);
+                                else
+                                    hvp_sign64<D>(u, ng != (__double2hiint(cf) < 0));
+                                hvp_rows<VT, D, RP>(R, u, cf, z + Zk);
+                            } else {
+                                hvp_rows<VT, D, RP>(R, u, ((negj >> k) & 1u) ? -cf : cf, z + Zk);
+                            }
+                        });
+                    };
+                    // FP64: two bodies, so that the common one issues no product by a factor of +-1 (predicated
+                    // products would occupy the FP64 pipe as well)
+                    if (sizeof(VT) == 8 && __ballot_sync(__activemask(), !hvp_unit64((double)cf)) == 0u)
+                        contract(std::false_type{});
+                    else
+                        contract(std::true_type{});
                 }
                 __syncwarp();
                 if (grp + nbuf < n_groups) fill(grp + nbuf);
@@ -846,7 +895,7 @@ __global__ void __launch_bounds__(hvp_max_threads<VT, SH>(), 1) hvp_kernel(const
             }
             __syncwarp();
             if (b < B) {
-                const VT inv_sq = sid == 0 ? (VT)1 : (VT)1 / __ldg(sqrtS + sid);
+                const VT inv_sq = sid == 0 ? (VT)1 : __ldg(sqrtS + P.n_sid + sid);
                 static_for<K>([&](auto kc) {
                     constexpr int k = decltype(kc)::value;
                     constexpr int D = SH::template D<k>;
@@ -855,12 +904,14 @@ __global__ void __launch_bounds__(hvp_max_threads<VT, SH>(), 1) hvp_kernel(const
                         VT val;
                         if (sid == 0) {
                             val = zs[(Zk + gam) * BT + b];
+                            if constexpr (sizeof(VT) == 8) val *= zscale;
                         } else {  // projector onto the range of V_k(r)
                             const VT *Pr = P.Pj[k] + ((size_t)sid * D + gam) * D;
                             val = (VT)0;
 #pragma unroll
                             for (int be = 0; be < D; ++be) val += __ldg(Pr + be) * zs[(Zk + be) * BT + b];
                             val *= inv_sq;
+                            if constexpr (sizeof(VT) == 8) val *= zscale;
                         }
                         const size_t e = seg + (size_t)(Zk + gam) * B + b;
                         const VT xv = st_get<VT, ST>(own_on ? own[(Zk + gam) * B + b] : __ldg(x + e));

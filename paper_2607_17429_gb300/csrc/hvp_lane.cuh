@@ -84,7 +84,8 @@ __global__ void __launch_bounds__(kLaneThreads) hvp_lane_kernel(const __grid_con
     for (int i = threadIdx.x; i < 2 * a.n_bonds; i += blockDim.x) s_bond[i] = a.bonds[i];
     __syncthreads();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const VT halfJ = a.J * (VT)0.5;
+    const VT halfJ = sizeof(VT) == 8 ? (VT)1 : a.J * (VT)0.5;  // as in hvp_kernel: FP64 scales the sums
+    const VT zscale = sizeof(VT) == 8 ? a.J * (VT)0.5 : (VT)1;
     const bool want_dot = a.dot_part != nullptr;
     DotAcc<VT> dacc;
     dacc.zero();
@@ -162,8 +163,18 @@ __global__ void __launch_bounds__(kLaneThreads) hvp_lane_kernel(const __grid_con
             if ((g8 & 128u) && (a.neg & 1u)) cf = -cf;  // (g*, 1) in a Gamma- block
             return cf;
         };
-        auto accumulate = [&](uint2 raw, VT cf, const VT(&u)[D]) {
+        auto accumulate = [&](uint2 raw, VT cf, VT(&u)[D]) {
             const VT *R = s_rho + (size_t)(raw.y & 127u) * D * RP;
+            if constexpr (sizeof(VT) == 8) {
+#pragma unroll
+                for (int g = 0; g < D; ++g) u[g] *= cf;
+#pragma unroll
+                for (int be = 0; be < D; ++be) {
+#pragma unroll
+                    for (int ga = 0; ga < D; ++ga) z[be] += R[ga * RP + be] * u[ga];
+                }
+                return;
+            }
 #pragma unroll
             for (int be = 0; be < D; ++be) {
                 VT acc = R[be] * u[0];
@@ -192,9 +203,9 @@ __global__ void __launch_bounds__(kLaneThreads) hvp_lane_kernel(const __grid_con
         VT val[D];
         if (sid == 0) {
 #pragma unroll
-            for (int g = 0; g < D; ++g) val[g] = z[g];
+            for (int g = 0; g < D; ++g) val[g] = sizeof(VT) == 8 ? z[g] * zscale : z[g];
         } else {  // projector onto the range of V(r), and 1/sqrt|Stab r|
-            const VT inv_sq = (VT)1 / __ldg(P.sqrtS + sid);
+            const VT inv_sq = zscale / __ldg(P.sqrtS + sid);
             const VT *Pr = P.Pj[0] + (size_t)sid * D * D;
 #pragma unroll
             for (int g = 0; g < D; ++g) {

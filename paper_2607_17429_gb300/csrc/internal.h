@@ -161,7 +161,7 @@ struct ftlm_basis {
     int irrep = 0, d = 0;
     uint64_t dim = 0;
     uint64_t *d_off = nullptr;      // [n_reps + 1]
-    // per stabilizer id: n_Gamma, sqrt|Stab|, V [d][d] (V[beta*d + k])
+    // per stabilizer id: n_Gamma, sqrt|Stab| (then 1 / sqrt|Stab| of every id), V [d][d] (V[beta*d + k])
     uint8_t *d_ntab = nullptr;
     double *d_sqrtS = nullptr;
     float *d_sqrtSf = nullptr;
