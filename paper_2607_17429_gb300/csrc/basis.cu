@@ -30,9 +30,9 @@ constexpr int kEnumThreads = 256;
 // Labels are enumerated under the prefixes (digits of the top sites) that can still be an orbit
 // minimum.  A prefix is dead when some element maps the state to a smaller label whatever the other
 // digits are; the labels under live prefixes are ranked consecutively, in ascending order.  The count
-// pass keeps its findings as one bit per label, so the write pass tests nothing.  Icosidodecahedron, M = 0 (1.55e8 labels, 1.3e6 representatives): 8.5 ms a sector with a
-// test of every label in both passes, 2.5 ms now; the dodecahedron's 1.65e9 labels at s = 3/2, M = 14:
-// 59 ms, 13.5 ms.
+// pass keeps its findings as one bit per label, so the write pass tests nothing.  Icosidodecahedron,
+// M = 0 (1.55e8 labels, 1.3e6 representatives): 8.5 ms a sector with a test of every label in both passes,
+// 2.5 ms now; the dodecahedron's 1.65e9 labels at s = 3/2, M = 14: 59 ms, 13.5 ms.
 struct EnumArgs {
     int N, bits, dmax, A, G;  // G: elements acting on the sector (2|G| with the spin flip)
     int pre;               // sites of a prefix
@@ -289,6 +289,17 @@ __global__ void build_buckets(const uint64_t *labels, uint64_t n_reps, int shift
     bucket[b] = (uint32_t)lo;
 }
 
+// {label, index, stabilizer id} of every representative: the lookup's last probe returns all three
+__global__ void fill_records(const uint64_t *labels, const uint16_t *stab_id, uint64_t n, HvRec *rec) {
+    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    HvRec r;
+    r.label = labels[i];
+    r.idx = (uint32_t)i;
+    r.sid = stab_id[i];
+    rec[i] = r;
+}
+
 struct NGammaOf {
     const uint16_t *stab_id;
     const uint8_t *ntab;
@@ -311,6 +322,7 @@ void free_sector(ftlm_sector *s) {
     cudaFree(s->d_labels);
     cudaFree(s->d_stab_id);
     cudaFree(s->d_bucket);
+    cudaFree(s->d_rec);
     cudaFree(s->d_lut);
     cudaFree(s->d_lut2);
     cudaFree(s->d_pos);
@@ -577,6 +589,11 @@ ftlm_status build_sector_impl(const GroupData &grp_in, int two_s, int two_M, int
         FTLM_CUDA(cudaGetLastError());
         FTLM_CUDA(cudaStreamSynchronize(stream));
     }
+    FTLM_CUDA(cudaMalloc((void **)&s->d_rec, n_reps * sizeof(HvRec)));
+    s->device_bytes += n_reps * sizeof(HvRec);
+    count_launch();
+    fill_records<<<(unsigned)((n_reps + 255) / 256), 256, 0, stream>>>(s->d_labels, s->d_stab_id, n_reps, s->d_rec);
+    FTLM_CUDA(cudaGetLastError());
     // bucket index on the high bits of the label
     uint64_t max_label = 0;
     FTLM_CUDA(cudaMemcpyAsync(&max_label, s->d_labels + (n_reps - 1), 8, cudaMemcpyDeviceToHost, stream));

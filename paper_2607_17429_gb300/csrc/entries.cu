@@ -33,17 +33,6 @@ struct FlipCount {
     }
 };
 
-// Records {label, index, stabilizer id}: the lookup of the build pass returns the index.
-__global__ void index_records(const uint64_t *labels, const uint16_t *stab_id, uint64_t n, HvRec *rec) {
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    HvRec r;
-    r.label = labels[i];
-    r.off = (uint32_t)i;
-    r.sid = stab_id[i];
-    rec[i] = r;
-}
-
 }  // namespace
 
 // Build-mode plan over parts whose entries go to fixed-stride slots (no count pass): launch it with
@@ -83,22 +72,16 @@ ftlm_status entry_table_build(ftlm_sector *s, cudaStream_t stream) {
         cudaGetLastError();
         return fail(FTLM_ENOMEM, "entry table of %llu entries: %s", (unsigned long long)total, cudaGetErrorString(e));
     }
-    DevBuf<HvRec> rec;
-    FTLM_CUDA(rec.alloc(std::max<uint64_t>(n, 1)));
     DevBuf<int> err;
     FTLM_CUDA(err.alloc(1));
     FTLM_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), stream));
     if (n) {
-        count_launch();
-        index_records<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(s->d_labels, s->d_stab_id, n, rec.p);
-        FTLM_CUDA(cudaGetLastError());
         // build-mode arguments: the search tables of the sector, no blocks, no vectors
         PackedSet ps;
         ps.K = 1;
         ps.W = 1;
         ps.dims[0] = 1;
         ps.rows = n;
-        ps.d_rec = rec.p;
         HvpPlan<float> plan;
         plan.mode = 2;
         HvpArgs<float> &a = plan.a;
@@ -107,7 +90,7 @@ ftlm_status entry_table_build(ftlm_sector *s, cudaStream_t stream) {
         HvpPart<float> part;
         memset(&part, 0, sizeof(part));
         part.n_reps = part.n_all = n;
-        part.rec = rec.p;
+        part.rec = s->d_rec;
         part.bucket = s->d_bucket;
         part.n_buckets = s->n_buckets;
         part.bucket_shift = s->bucket_shift;

@@ -101,7 +101,7 @@ struct HvpPart {
     uint64_t n_all;          // representatives of its sector (rows of x)
     uint64_t tile0;          // first tile of this part in the launch's tile order
     int tile_reps;           // representatives per tile of this part
-    const HvRec *rec;        // [n_reps], ascending labels; rec.off = index * W
+    const HvRec *rec;        // [n_all], ascending labels
     const uint32_t *bucket;  // [n_buckets + 1]
     uint64_t n_buckets;
     int bucket_shift;
@@ -537,7 +537,7 @@ __global__ void __launch_bounds__(hvp_max_threads<VT, SH>(), 1) hvp_kernel(const
         for (uint64_t rep = r0 + wid; rep < r1 && !dead; rep += warps) {
             const HvRec rr = rec[P.rep0 + rep];
             const int sid = (int)rr.sid;
-            const size_t seg = (size_t)rr.off * B;  // first element of r's W rows
+            const size_t seg = (size_t)rr.idx * W * B;  // first element of r's W rows
             if (MODE != 2 && sid != 0 && __ldg(P.wtab + sid) == 0) {  // no block has rows for this orbit: y~(r) = 0
                 for (int e = lane; e < W * B; e += 32) y[seg + e] = st_put<VT, ST>((VT)0);
                 continue;
@@ -715,7 +715,7 @@ __global__ void __launch_bounds__(hvp_max_threads<VT, SH>(), 1) hvp_kernel(const
                 if (lane < nround) {
                     const uint64_t key = (uint64_t)my_rp;
                     const uint64_t bk = key >> P.bucket_shift;
-                    uint32_t off_f = 0, sid_f = 0, idx_f = 0;
+                    uint32_t sid_f = 0, idx_f = 0;
                     bool found = false;
                     if (bk < P.n_buckets) {
                         uint32_t lo = __ldg(P.bucket + bk), hi = __ldg(P.bucket + bk + 1);
@@ -734,7 +734,6 @@ __global__ void __launch_bounds__(hvp_max_threads<VT, SH>(), 1) hvp_kernel(const
                         }
                         if (lo < hi0 && ((((uint64_t)hrec.y << 32) | hrec.x) == key)) {
                             found = true;
-                            off_f = hrec.z;
                             sid_f = hrec.w;
                             idx_f = lo;
                         }
@@ -755,7 +754,7 @@ __global__ void __launch_bounds__(hvp_max_threads<VT, SH>(), 1) hvp_kernel(const
                             P.ent[slot] = en;
                         }
                     } else {
-                        f_off[base + lane] = off_f;
+                        f_off[base + lane] = idx_f * (uint32_t)W;
                         f_sg[base + lane] = (sid_f << 8) | (uint32_t)my_g;  // g* < |G| <= 128, bit 7: spin flip
                         f_c[base + lane] = my_c * __ldg(sqrtS + sid_f);      // c_a sqrt|Stab r'|
                     }

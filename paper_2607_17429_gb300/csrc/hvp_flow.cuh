@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(flow_threads<ST, SH, CL>(), 1) hvp_flow_kernel
 
         struct Rep {  // one representative's record and its first 64 entries (lane j: flips j and 32 + j)
             uint64_t label, e0;
-            uint32_t off, sid;
+            uint32_t idx, sid;
             int nf, state;  // state: 0 none, 1 work, 2 no block has rows (y~ = 0)
             uint2 ea, eb;
         };
@@ -242,11 +242,11 @@ __global__ void __launch_bounds__(flow_threads<ST, SH, CL>(), 1) hvp_flow_kernel
             }
             q.nf = 0;
             q.label = q.e0 = 0;
-            q.off = q.sid = 0;
+            q.idx = q.sid = 0;
             if (!q.state) return;
             const uint4 v = __ldg(reinterpret_cast<const uint4 *>(rec + rep));
             q.label = ((uint64_t)v.y << 32) | v.x;
-            q.off = v.z;
+            q.idx = v.z;
             q.sid = v.w;
             if (P.ecnt) {
                 q.e0 = rep * (uint64_t)P.estride;
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(flow_threads<ST, SH, CL>(), 1) hvp_flow_kernel
             load_rec(nxt);
             nxt.ea = nxt.eb = make_uint2(0u, 0u);
             const int ng = (cur.nf + Q - 1) / Q;
-            const size_t seg = (size_t)cur.off * B;
+            const size_t seg = (size_t)cur.idx * W * B;
             int filled_n = 0;
             n_flips += (unsigned long long)cur.nf;
             const float cfa = coef(cur.label, cur.ea), cfb = coef(cur.label, cur.eb);

@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(kLaneThreads) hvp_lane_kernel(const __grid_con
         const bool vec = (reinterpret_cast<uintptr_t>(x) & 15) == 0;
         const HvRec rr = P.rec[P.rep0 + rep];
         const int sid = (int)rr.sid;
-        const size_t seg = rr.off;  // W = D rows, B = 1
+        const size_t seg = (size_t)rr.idx * D;  // W = D rows, B = 1
         if (sid != 0 && __ldg(P.wtab + sid) == 0) {
 #pragma unroll
             for (int g = 0; g < D; ++g) y[seg + g] = st_put<VT, ST>((VT)0);

@@ -20,11 +20,11 @@ constexpr int kMaxB = 32;       // right-hand sides per H·v launch
 constexpr int kPMaxK = 10;      // blocks per packed set (compile-time shapes)
 constexpr int kMaxSteps = 512;  // Lanczos steps per chain
 
-// Record of one representative in a packed set: label, first row of its
-// segment in the packed vector, stabilizer subgroup id.
+// Record of one representative: label, index in the sector (its segment of a packed vector starts at row
+// index * W), stabilizer subgroup id.
 struct alignas(16) HvRec {
     uint64_t label;
-    uint32_t off;
+    uint32_t idx;
     uint32_t sid;
 };
 
@@ -52,7 +52,6 @@ struct PackedSet {
     int shape = -1;     // compiled shape id (see packed.cu), -1 if none matches
     int dims[kPMaxK] = {};
     uint64_t rows = 0;  // packed rows = n_reps * W
-    HvRec *d_rec = nullptr;         // [n_reps]: label, off = index * W, stabilizer id
     uint8_t *d_ntab = nullptr;      // [n_sid][K] n_k(sid)
     uint8_t *d_wtab = nullptr;      // [n_sid] sum_k n_k(sid)
     double *d_P[kPMaxK] = {};       // block k: [n_sid][d_k][d_k] projector V V^T
@@ -137,6 +136,7 @@ struct ftlm_sector {
     uint16_t *d_stab_id = nullptr;  // [n_reps] stabilizer subgroup id (0 = trivial)
     std::vector<std::array<uint64_t, 4>> stab_masks;  // per id: bit g of the group acting on the sector
     std::vector<std::vector<int>> stab_elems;         // per id
+    ftlm::HvRec *d_rec = nullptr;   // [n_reps] label, index, stabilizer id (shared by every packed set)
     uint32_t *d_bucket = nullptr;                     // [n_buckets + 1] first rep index of each bucket
     uint64_t *d_eoff = nullptr;                       // entry table (optional): [n_reps + 1] first entry
     ftlm::HvEntry *d_ent = nullptr;                   // [n_entries] per representative, in flip order

@@ -57,7 +57,7 @@ struct LzArgs {
     uint64_t n_tiles;
     int tile_reps;
     int B, BT, lgBT;
-    int dims[kPMaxK], zoff[kPMaxK];
+    int W, dims[kPMaxK], zoff[kPMaxK];
     int rng;
     uint32_t chain0, key0;
     double *norm_part;     // [n_parts][gridDim.x][K][B]
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(kLzThreads) lzp_start(const __grid_constant__ 
             for (int k = 0; k < K; ++k) {
                 const int D = a.dims[k];
                 for (int gam = fg; gam < D; gam += Q) {
-                    const size_t e = ((size_t)rr.off + a.zoff[k] + gam) * B + b;
+                    const size_t e = ((size_t)rr.idx * a.W + a.zoff[k] + gam) * B + b;
                     const uint64_t row0 = __ldg(P.boff[k] + rep);
                     VT v;
                     if (sid == 0) {
@@ -620,7 +620,7 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
             memset(&lp, 0, sizeof(lp));
             lp.n_reps = sets[p].sec->n_reps;
             lp.tile0 = tinfo[2 * P + p];
-            lp.rec = sets[p].ps->d_rec;
+            lp.rec = sets[p].sec->d_rec;
             lp.ntab = sets[p].ps->d_ntab;
             for (int k = 0; k < K; ++k) {
                 lp.V[k] = sizeof(VT) == 8 ? reinterpret_cast<const VT *>(sets[p].blocks[k]->d_V)
@@ -641,6 +641,7 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
                                       stream));
             la.parts = d_lparts.p;
         }
+        la.W = ps0->W;
         la.n_tiles = lz_tiles;
         la.tile_reps = lz_tile;
         la.B = B;

@@ -2,9 +2,8 @@
 // in lifted coordinates) and the entry points of the packed H·v: ftlm_hv (one
 // block), ftlm_hv_packed, ftlm_multiblock_pack / _unpack, ftlm_set_wait_limit.
 //
-// Construction (Section 3's two phases): the irrep-independent records of the
-// sector (label, stabilizer id) get the segment offset r * W of every
-// representative; per stabilizer id the set keeps n_k (Section 2.3), their sum,
+// Construction (Section 3's two phases): the irrep-independent records belong to the
+// sector; representative r owns the rows from r * W; per stabilizer id the set keeps n_k (Section 2.3), their sum,
 // and the projector V_k V_k^T of every block (Eq. 11).  Lifting a block vector,
 // x~_k(r) = V_k(r) x_k(r), and lowering it back, x_k(r) = V_k(r)^T x~_k(r), are
 // the pack and unpack copies.
@@ -40,16 +39,6 @@ const ShapeDef kShapeDefs[kNumShapes] = {
 
 std::atomic<unsigned long long> g_wait_limit{kDrainCycles};
 
-__global__ void fill_records(const uint64_t *labels, const uint16_t *stab_id, uint64_t n, int W, HvRec *rec) {
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    HvRec r;
-    r.label = labels[i];
-    r.off = (uint32_t)(i * (uint64_t)W);
-    r.sid = stab_id[i];
-    rec[i] = r;
-}
-
 struct LiftArgs {
     uint64_t n_reps;
     int K, W, B, to_packed;
@@ -75,7 +64,7 @@ __global__ void lift_rows(const __grid_constant__ LiftArgs a, VT *packed) {
         const VT *V = reinterpret_cast<const VT *>(a.V[k]) + (size_t)r.sid * d * d;
         VT *blk = reinterpret_cast<VT *>(a.blk[k]);
         const uint64_t o = a.boff[k][rep];
-        VT *pk = packed + ((uint64_t)r.off + a.zoff[k]) * B + b;
+        VT *pk = packed + (rep * a.W + a.zoff[k]) * B + b;
         if (a.to_packed) {
             for (int gm = 0; gm < d; ++gm) {
                 VT v = (VT)0;
@@ -114,7 +103,6 @@ unsigned long long wait_limit_cycles() { return g_wait_limit.load(); }
 
 void packed_set_free(PackedSet *ps) {
     if (!ps) return;
-    cudaFree(ps->d_rec);
     cudaFree(ps->d_ntab);
     cudaFree(ps->d_wtab);
     for (int k = 0; k < kPMaxK; ++k) {
@@ -199,8 +187,7 @@ ftlm_status packed_set_build(ftlm_sector *s, int K, const ftlm_basis *const *blo
     FTLM_CUDA(cudaMalloc((void **)&ps->d_wtab, wtab.size() + 1));
     FTLM_CUDA(cudaMalloc((void **)&ps->d_rhoT, rho.size() * 8 + 16));
     FTLM_CUDA(cudaMalloc((void **)&ps->d_rhoTf, rhof.size() * 4 + 16));
-    FTLM_CUDA(cudaMalloc((void **)&ps->d_rec, s->n_reps * sizeof(HvRec) + sizeof(HvRec)));
-    ps->device_bytes += ntab.size() + wtab.size() + rho.size() * 8 + rhof.size() * 4 + s->n_reps * sizeof(HvRec);
+    ps->device_bytes += ntab.size() + wtab.size() + rho.size() * 8 + rhof.size() * 4;
     FTLM_CUDA(cudaMemcpyAsync(ps->d_ntab, ntab.data(), ntab.size(), cudaMemcpyHostToDevice, stream));
     FTLM_CUDA(cudaMemcpyAsync(ps->d_wtab, wtab.data(), wtab.size(), cudaMemcpyHostToDevice, stream));
     FTLM_CUDA(cudaMemcpyAsync(ps->d_rhoT, rho.data(), rho.size() * 8, cudaMemcpyHostToDevice, stream));
@@ -209,12 +196,6 @@ ftlm_status packed_set_build(ftlm_sector *s, int K, const ftlm_basis *const *blo
     if (rows >= 0xffffffffull)
         return fail(FTLM_EUNSUPPORTED, "packed set has %llu rows (limit 2^32 - 1)", (unsigned long long)rows);
     ps->rows = rows;
-    if (s->n_reps) {
-        count_launch();
-        fill_records<<<(unsigned)((s->n_reps + 255) / 256), 256, 0, stream>>>(s->d_labels, s->d_stab_id, s->n_reps,
-                                                                               ps->W, ps->d_rec);
-        FTLM_CUDA(cudaGetLastError());
-    }
     FTLM_CUDA(cudaStreamSynchronize(stream));
     guard.p = nullptr;
     *out = ps;
@@ -315,7 +296,7 @@ void hvp_part_of(const ftlm_sector *s, const PackedSet *ps, const ftlm_basis *co
                  HvpPart<VT> &p) {
     memset(&p, 0, sizeof(p));
     p.n_reps = p.n_all = s->n_reps;
-    p.rec = ps->d_rec;
+    p.rec = s->d_rec;
     p.bucket = s->d_bucket;
     p.n_buckets = s->n_buckets;
     p.bucket_shift = s->bucket_shift;
@@ -628,7 +609,7 @@ ftlm_status lift_impl(const ftlm_sector *s, const PackedSet *ps, const ftlm_basi
     la.B = B;
     la.to_packed = to_packed;
     la.ntab = ps->d_ntab;
-    la.rec = ps->d_rec;
+    la.rec = s->d_rec;
     int z = 0;
     for (int k = 0; k < ps->K; ++k) {
         la.dims[k] = ps->dims[k];

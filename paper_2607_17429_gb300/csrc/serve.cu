@@ -214,7 +214,7 @@ bool admit_head(ftlm_server *S, std::unique_lock<std::mutex> &lk, cudaStream_t b
     if (!se->sec) {
         const GroupData &g = js.group->d;
         const double dim = sector_dim_estimate(g.N, js.two_s, js.two_M);
-        const size_t est = (size_t)(dim / std::max(1, g.G) * 1.1 * 24.0) + (8u << 20);
+        const size_t est = (size_t)(dim / std::max(1, g.G) * 1.1 * 40.0) + (8u << 20);
         if (!make_room(S, est)) {
             if (!idle()) return false;
             if (se->blocks.empty() && se->pins == 0) S->sectors.erase(key);
@@ -259,7 +259,7 @@ bool admit_head(ftlm_server *S, std::unique_lock<std::mutex> &lk, cudaStream_t b
     be->last = ++S->tick;
     ++be->refs;  // pinned from here on; kept by the job once admitted
     if (!be->blk) {
-        const size_t est = (size_t)se->sec->n_reps * 40 + (4u << 20);
+        const size_t est = (size_t)se->sec->n_reps * 24 + (4u << 20);
         if (!make_room(S, est)) {
             --be->refs;
             if (!idle()) return false;
