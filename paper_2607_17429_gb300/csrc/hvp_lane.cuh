@@ -1,12 +1,16 @@
-// Table-mode H·v with one thread per output representative, for one block
-// (K = 1) and one right-hand side (B = 1): Eqs. 15-16 in the pull form with the
-// flips read from the sector's entry table (Section 3).  A warp of the search
-// or table kernel works on one representative at a time; with B = 1 most of its
-// lanes idle and each representative is a chain of dependent memory round trips
-// (record, entry offsets, entries, gathers).  Here every thread walks its own
-// representative's entries, so a warp keeps 32 such chains in flight.  The
-// contributions are summed in entry order (the warp kernels sum them per flip
+// Table-mode H·v of one block (K = 1) with a thread per output representative and CV right-hand sides:
+// Eqs. 15-16 in the pull form with the flips read from an entry table (Section 3).  A warp of the search
+// or table kernel works on one representative at a time; with d B small most of its lanes idle and
+// each representative is a chain of dependent memory round trips (record, entry offsets, entries,
+// gathers).  Here every thread walks its own representative's entries, so a warp keeps 32 / (B / CV) such
+// chains in flight.  CV is 1 for B = 1 and odd B, else 2 or 4 neighbouring right-hand sides, one vector
+// load per row.  The contributions are summed in entry order (the warp kernels sum them per flip
 // group and then across groups), so results agree with theirs to rounding.
+//
+// Blocks of dimension 1, 3, 4, 5 of the icosidodecahedron at M = 0, FP32, from the table: B = 1 0.19 to 0.43 ms;
+// B = 8 2.6 to 3.1 ms with a warp per representative, 0.29 to 1.25 ms here; B = 32 7.2 to 9.1 ms, 0.9 to 4.4 ms.
+// Bound by L1 sector look-ups of the gathers for rows of less than 32 bytes (B = 1: about one per cycle
+// and SM), by the entries' and gathers' latency above.
 #pragma once
 
 #include "hvp.cuh"
@@ -14,7 +18,10 @@
 namespace ftlm {
 
 constexpr int kLaneThreads = 256;
-constexpr int kLaneFlips = 2;  // flips whose entries and rows are loaded before the first is summed
+// flips whose entries and rows are loaded before the first is summed
+__host__ __device__ constexpr int lane_flips(int D, int CV) { return D * CV <= 4 ? 4 : D * CV <= 16 ? 2 : 1; }
+// right-hand sides per thread and threads per representative
+inline int lane_cols(int B) { return B % 4 == 0 ? 4 : B % 2 == 0 ? 2 : 1; }
 
 __host__ __device__ constexpr int lane_gcd(int a, int b) { return b == 0 ? a : lane_gcd(b, a % b); }
 
@@ -73,36 +80,65 @@ __device__ __forceinline__ void lane_row(const ST *__restrict__ x, uint64_t r, u
     }
 }
 
-template <typename VT, typename ST, int D>
+// CV neighbouring stored elements of row r, columns c .. c + CV - 1
+template <typename VT, typename ST, int CV>
+__device__ __forceinline__ void lane_cols_load(const ST *__restrict__ x, size_t e, bool vec, VT (&u)[CV]) {
+    if constexpr (CV > 1) {
+        constexpr int BYTES = CV * (int)sizeof(ST);
+        if (vec) {
+            alignas(16) ST s[CV];
+            if constexpr (BYTES == 4)
+                *reinterpret_cast<uint32_t *>(s) = __ldg(reinterpret_cast<const uint32_t *>(x + e));
+            else if constexpr (BYTES == 8)
+                *reinterpret_cast<uint2 *>(s) = __ldg(reinterpret_cast<const uint2 *>(x + e));
+            else
+                *reinterpret_cast<uint4 *>(s) = __ldg(reinterpret_cast<const uint4 *>(x + e));
+#pragma unroll
+            for (int v = 0; v < CV; ++v) u[v] = st_get<VT, ST>(s[v]);
+            return;
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < CV; ++v) u[v] = st_get<VT, ST>(__ldg(x + e + v));
+}
+
+// ONE: a single right-hand side (rows of D consecutive elements)
+template <typename VT, typename ST, int D, int CV, bool ONE>
 __global__ void __launch_bounds__(kLaneThreads) hvp_lane_kernel(const __grid_constant__ HvpArgs<VT> a) {
-    constexpr int RP = rho_row(D);
+    constexpr int RP = rho_row(D), FL = ONE ? 2 : lane_flips(D, CV);
     extern __shared__ __align__(128) uint8_t smem[];
     VT *s_rho = reinterpret_cast<VT *>(smem);  // rho(g) of the block, [G][D][RP]
     uint8_t *s_bond = smem + (((size_t)a.rho_total * sizeof(VT) + 15) & ~(size_t)15);
-    __shared__ double red[kLaneThreads / 32];
+    __shared__ double red[kLaneThreads];
     for (int i = threadIdx.x; i < a.rho_total; i += blockDim.x) s_rho[i] = a.rhoT[i];
     for (int i = threadIdx.x; i < 2 * a.n_bonds; i += blockDim.x) s_bond[i] = a.bonds[i];
     __syncthreads();
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+    const int B = ONE ? 1 : a.B, tpr = ONE ? 1 : B / CV, per_cta = kLaneThreads / tpr;  // threads per representative
+    const int lrep = (int)threadIdx.x / tpr, col = ((int)threadIdx.x - lrep * tpr) * CV;
     const VT halfJ = sizeof(VT) == 8 ? (VT)1 : a.J * (VT)0.5;  // as in hvp_kernel: FP64 scales the sums
     const VT zscale = sizeof(VT) == 8 ? a.J * (VT)0.5 : (VT)1;
     const bool want_dot = a.dot_part != nullptr;
-    DotAcc<VT> dacc;
-    dacc.zero();
+    DotAcc<VT> dacc[CV];
+#pragma unroll
+    for (int v = 0; v < CV; ++v) dacc[v].zero();
     int cur_part = -1;
     unsigned long long n_flips = 0;  // profiling: one atomic per warp at the end
-    auto flush = [&](int p) {  // CTA sum of the per-thread <x, y> in a fixed order
-        double v = dacc.value();
-        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(kFullMask, v, o);
-        __syncthreads();
-        if (lane == 0) red[wid] = v;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double t = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-            a.dot_part[(size_t)p * gridDim.x + blockIdx.x] = t;
+    auto flush = [&](int p) {        // CTA sums of the per-thread <x, y> per column, a fixed tree over representatives
+#pragma unroll
+        for (int v = 0; v < CV; ++v) {
+            __syncthreads();
+            red[threadIdx.x] = dacc[v].value();
+            int top = 1;
+            while (2 * top < per_cta) top *= 2;
+            for (int h = top; h; h >>= 1) {
+                __syncthreads();
+                if (lrep < h && lrep + h < min(per_cta, 2 * h)) red[threadIdx.x] += red[threadIdx.x + h * tpr];
+            }
+            __syncthreads();
+            if (lrep == 0) a.dot_part[((size_t)p * gridDim.x + blockIdx.x) * B + col + v] = red[threadIdx.x];
+            dacc[v].zero();
         }
-        dacc.zero();
     };
     for (uint64_t t = blockIdx.x; t < a.n_tiles; t += gridDim.x) {
         int p = 0;
@@ -122,34 +158,49 @@ __global__ void __launch_bounds__(kLaneThreads) hvp_lane_kernel(const __grid_con
             cur_part = p;
         }
         const HvpPart<VT> &P = a.n_parts == 1 ? a.part0 : a.parts[p];
-        const uint64_t rep = (t - P.tile0) * (uint64_t)P.tile_reps + threadIdx.x;
-        if (rep >= P.n_reps || (int)threadIdx.x >= P.tile_reps) continue;
+        const uint64_t rep = (t - P.tile0) * (uint64_t)P.tile_reps + lrep;
+        if (rep >= P.n_reps || lrep >= P.tile_reps) continue;
         const ST *__restrict__ x = static_cast<const ST *>(P.x);
         ST *__restrict__ y = static_cast<ST *>(P.y);
         const uint64_t n_elems = P.n_all * (uint64_t)D;
         const bool vec = (reinterpret_cast<uintptr_t>(x) & 15) == 0;
-        const HvRec rr = P.rec[P.rep0 + rep];
+        const uint64_t at = P.rep0 + rep;  // in the sector
+        const HvRec rr = P.rec[at];
         const int sid = (int)rr.sid;
-        const size_t seg = (size_t)rr.idx * D;  // W = D rows, B = 1
+        const size_t seg = at * D * B + col;
         if (sid != 0 && __ldg(P.wtab + sid) == 0) {
 #pragma unroll
-            for (int g = 0; g < D; ++g) y[seg + g] = st_put<VT, ST>((VT)0);
+            for (int g = 0; g < D; ++g)
+#pragma unroll
+                for (int v = 0; v < CV; ++v) y[seg + (size_t)g * B + v] = st_put<VT, ST>((VT)0);
             continue;
         }
         const uint64_t lab = rr.label;
+        uint64_t e0, e1;
+        if (P.ecnt) {
+            e0 = rep * (uint64_t)P.estride;
+            e1 = e0 + __ldg(P.ecnt + rep);
+        } else {
+            e0 = __ldg(P.eoff + at);
+            e1 = __ldg(P.eoff + at + 1);
+        }
         int diag4 = 0;
-        for (int e = 0; e < a.n_bonds; ++e)
-            diag4 += (2 * (int)hvp_digit(lab, s_bond[2 * e], a.bits) - a.two_s) *
-                     (2 * (int)hvp_digit(lab, s_bond[2 * e + 1], a.bits) - a.two_s);
+        if (a.two_s == 1) {  // every bond is +1/4 or, when it flips, -1/4
+            diag4 = a.n_bonds - 2 * (int)(e1 - e0);
+        } else {
+            for (int e = 0; e < a.n_bonds; ++e)
+                diag4 += (2 * (int)hvp_digit(lab, s_bond[2 * e], a.bits) - a.two_s) *
+                         (2 * (int)hvp_digit(lab, s_bond[2 * e + 1], a.bits) - a.two_s);
+        }
         const VT diag = a.J * (VT)diag4 * (VT)0.25;
-        const uint64_t e0 = P.ecnt ? rep * (uint64_t)P.estride : __ldg(P.eoff + P.rep0 + rep);
-        const uint64_t e1 = P.ecnt ? e0 + __ldg(P.ecnt + rep) : __ldg(P.eoff + P.rep0 + rep + 1);
-        n_flips += e1 - e0;
-        VT z[D];
+        if (col == 0) n_flips += e1 - e0;
+        VT z[D][CV];
 #pragma unroll
-        for (int g = 0; g < D; ++g) z[g] = (VT)0;
+        for (int g = 0; g < D; ++g)
+#pragma unroll
+            for (int v = 0; v < CV; ++v) z[g][v] = (VT)0;
         // one flip: coefficient of Eq. 3 times sqrt|Stab r'| (the 1/sqrt|Stab r| comes last), gather of
-        // the target's row, z += cf rho(g*)^T u; flips are summed in entry order
+        // the target's rows; flips are summed in entry order
         auto coef = [&](uint2 raw) {
             const uint32_t g8 = raw.y & 255u, es = (raw.y >> 8) & 255u, sidf = raw.y >> 16;
             VT c = halfJ;
@@ -163,66 +214,97 @@ __global__ void __launch_bounds__(kLaneThreads) hvp_lane_kernel(const __grid_con
             if ((g8 & 128u) && (a.neg & 1u)) cf = -cf;  // (g*, 1) in a Gamma- block
             return cf;
         };
-        auto accumulate = [&](uint2 raw, VT cf, VT(&u)[D]) {
-            const VT *R = s_rho + (size_t)(raw.y & 127u) * D * RP;
-            if constexpr (sizeof(VT) == 8) {
+        auto gather = [&](uint64_t r, VT(&u)[D][CV]) {
+            if constexpr (ONE) {
+                VT w[D];
+                lane_row<VT, ST, D>(x, r, n_elems, vec, w);
 #pragma unroll
-                for (int g = 0; g < D; ++g) u[g] *= cf;
+                for (int g = 0; g < D; ++g) u[g][0] = w[g];
+            } else {
 #pragma unroll
-                for (int be = 0; be < D; ++be) {
-#pragma unroll
-                    for (int ga = 0; ga < D; ++ga) z[be] += R[ga * RP + be] * u[ga];
-                }
-                return;
-            }
-#pragma unroll
-            for (int be = 0; be < D; ++be) {
-                VT acc = R[be] * u[0];
-#pragma unroll
-                for (int ga = 1; ga < D; ++ga) acc += R[ga * RP + be] * u[ga];
-                z[be] += cf * acc;
+                for (int g = 0; g < D; ++g) lane_cols_load<VT, ST, CV>(x, (r * D + g) * B + col, vec, u[g]);
             }
         };
+        // s = cf rho(g*)^T u of the first flip of a group, plus that of the others
+        auto contract = [&](uint2 raw, VT cf, const VT(&u)[D][CV], VT(&s)[D][CV], bool first) {
+            const VT *R = s_rho + (size_t)(raw.y & 127u) * D * RP;
+            VT acc[D][CV];
+#pragma unroll
+            for (int ga = 0; ga < D; ++ga) {
+                VT row[RP];
+                load_row<VT, RP>(R + ga * RP, row);
+#pragma unroll
+                for (int be = 0; be < D; ++be)
+#pragma unroll
+                    for (int v = 0; v < CV; ++v) acc[be][v] = ga == 0 ? row[be] * u[0][v] : acc[be][v] + row[be] * u[ga][v];
+            }
+#pragma unroll
+            for (int be = 0; be < D; ++be)
+#pragma unroll
+                for (int v = 0; v < CV; ++v) s[be][v] = first ? cf * acc[be][v] : s[be][v] + cf * acc[be][v];
+        };
+        const uint2 *ent = reinterpret_cast<const uint2 *>(P.ent);
         uint64_t e = e0;
-        for (; e + kLaneFlips <= e1; e += kLaneFlips) {  // kLaneFlips gathers in flight per thread
-            uint2 r[kLaneFlips];
-            VT u[kLaneFlips][D];
+        for (; e + FL <= e1; e += FL) {  // FL gathers in flight per thread, one addition to z for them all
+            uint2 r[FL];
+            VT u[FL][D][CV], s[D][CV];
 #pragma unroll
-            for (int q = 0; q < kLaneFlips; ++q) r[q] = __ldg(reinterpret_cast<const uint2 *>(P.ent + e + q));
+            for (int q = 0; q < FL; ++q) r[q] = __ldg(ent + e + q);
 #pragma unroll
-            for (int q = 0; q < kLaneFlips; ++q) lane_row<VT, ST, D>(x, r[q].x, n_elems, vec, u[q]);
+            for (int q = 0; q < FL; ++q) gather(r[q].x, u[q]);
 #pragma unroll
-            for (int q = 0; q < kLaneFlips; ++q) accumulate(r[q], coef(r[q]), u[q]);
+            for (int q = 0; q < FL; ++q) contract(r[q], coef(r[q]), u[q], s, q == 0);
+#pragma unroll
+            for (int g = 0; g < D; ++g)
+#pragma unroll
+                for (int v = 0; v < CV; ++v) z[g][v] += s[g][v];
         }
         for (; e < e1; ++e) {
-            const uint2 r0 = __ldg(reinterpret_cast<const uint2 *>(P.ent + e));
-            VT u0[D];
-            lane_row<VT, ST, D>(x, r0.x, n_elems, vec, u0);
-            accumulate(r0, coef(r0), u0);
+            const uint2 r0 = __ldg(ent + e);
+            VT u0[D][CV], s[D][CV];
+            gather(r0.x, u0);
+            contract(r0, coef(r0), u0, s, true);
+#pragma unroll
+            for (int g = 0; g < D; ++g)
+#pragma unroll
+                for (int v = 0; v < CV; ++v) z[g][v] += s[g][v];
         }
-        VT val[D];
-        if (sid == 0) {
+        VT xo[D][CV];
+        gather(at, xo);
 #pragma unroll
-            for (int g = 0; g < D; ++g) val[g] = sizeof(VT) == 8 ? z[g] * zscale : z[g];
-        } else {  // projector onto the range of V(r), and 1/sqrt|Stab r|
-            const VT inv_sq = zscale / __ldg(P.sqrtS + sid);
-            const VT *Pr = P.Pj[0] + (size_t)sid * D * D;
+        for (int v = 0; v < CV; ++v) {
+            VT val[D];
+            if (sid == 0) {
 #pragma unroll
-            for (int g = 0; g < D; ++g) {
-                VT v = (VT)0;
+                for (int g = 0; g < D; ++g) val[g] = sizeof(VT) == 8 ? z[g][v] * zscale : z[g][v];
+            } else {  // projector onto the range of V(r), and 1/sqrt|Stab r|
+                const VT inv_sq = zscale * __ldg(P.sqrtS + P.n_sid + sid);
+                const VT *Pr = P.Pj[0] + (size_t)sid * D * D;
 #pragma unroll
-                for (int be = 0; be < D; ++be) v += __ldg(Pr + g * D + be) * z[be];
-                val[g] = v * inv_sq;
+                for (int g = 0; g < D; ++g) {
+                    VT w = (VT)0;
+#pragma unroll
+                    for (int be = 0; be < D; ++be) w += __ldg(Pr + g * D + be) * z[be][v];
+                    val[g] = w * inv_sq;
+                }
             }
+#pragma unroll
+            for (int g = 0; g < D; ++g) z[g][v] = val[g] + diag * xo[g][v];
         }
-        VT xo[D];
-        lane_row<VT, ST, D>(x, P.rep0 + rep, n_elems, vec, xo);
 #pragma unroll
         for (int g = 0; g < D; ++g) {
-            const VT xv = xo[g];
-            const ST ys = st_put<VT, ST>(val[g] + diag * xv);
-            y[seg + g] = ys;
-            if (want_dot) dacc.add(xv, st_get<VT, ST>(ys));
+            alignas(16) ST ys[CV];
+#pragma unroll
+            for (int v = 0; v < CV; ++v) {
+                ys[v] = st_put<VT, ST>(z[g][v]);
+                if (want_dot) dacc[v].add(xo[g][v], st_get<VT, ST>(ys[v]));
+            }
+            if (CV * sizeof(ST) == 16 && vec && (reinterpret_cast<uintptr_t>(y) & 15) == 0) {
+                *reinterpret_cast<uint4 *>(y + seg + (size_t)g * B) = *reinterpret_cast<const uint4 *>(ys);
+            } else {
+#pragma unroll
+                for (int v = 0; v < CV; ++v) y[seg + (size_t)g * B + v] = ys[v];
+            }
         }
     }
     if (want_dot && cur_part >= 0) flush(cur_part);
@@ -237,15 +319,33 @@ size_t hvp_lane_smem(const HvpArgs<VT> &a) {
     return (((size_t)a.rho_total * sizeof(VT) + 15) & ~(size_t)15) + (size_t)2 * a.n_bonds + 16;
 }
 
+// CV for the plan's B (FP64: one right-hand side only)
+template <typename VT, typename ST, int D, class F>
+auto lane_dispatch(int B, F f) {
+    if constexpr (sizeof(VT) == 4) {
+        if (B > 1 && lane_cols(B) == 4) return f(std::integral_constant<int, 4>{}, std::false_type{});
+        if (B > 1 && lane_cols(B) == 2) return f(std::integral_constant<int, 2>{}, std::false_type{});
+        if (B > 1) return f(std::integral_constant<int, 1>{}, std::false_type{});
+    }
+    return f(std::integral_constant<int, 1>{}, std::true_type{});
+}
+
 template <typename VT, typename ST, int D>
 int hvp_lane_occupancy_t(const HvpArgs<VT> &a, int warps, int) {
     if (warps * 32 != kLaneThreads) return 0;
-    return hvp_fit_occupancy<hvp_lane_kernel<VT, ST, D>>(warps, hvp_lane_smem<VT, ST, D>(a));
+    return lane_dispatch<VT, ST, D>(a.B, [&](auto CV, auto ONE) {
+        return hvp_fit_occupancy<hvp_lane_kernel<VT, ST, D, decltype(CV)::value, decltype(ONE)::value>>(
+            warps, hvp_lane_smem<VT, ST, D>(a));
+    });
 }
 
 template <typename VT, typename ST, int D>
 ftlm_status hvp_lane_launch_t(HvpArgs<VT> a, const HvpGeom &geo, cudaStream_t stream) {
-    hvp_lane_kernel<VT, ST, D><<<(unsigned)geo.grid, kLaneThreads, hvp_lane_smem<VT, ST, D>(a), stream>>>(a);
+    lane_dispatch<VT, ST, D>(a.B, [&](auto CV, auto ONE) {
+        hvp_lane_kernel<VT, ST, D, decltype(CV)::value, decltype(ONE)::value>
+            <<<(unsigned)geo.grid, kLaneThreads, hvp_lane_smem<VT, ST, D>(a), stream>>>(a);
+        return 0;
+    });
     count_launch();
     FTLM_CUDA(cudaGetLastError());
     return FTLM_OK;

@@ -353,7 +353,7 @@ ftlm_status hvp_choose_geom(const HvpOps<VT> *ops, HvpArgs<VT> a, bool tma, HvpG
                     geo.tma = tma ? 1 : 0;
                     geo.rho_smem = rho;
                     geo.own = own;
-                    geo.tile_reps = ops->tile_fixed ? ops->tile_fixed : warps * 4;
+                    geo.tile_reps = ops->tile_fixed ? ops->tile_fixed / (a.B / lane_cols(a.B)) : warps * 4;
                     geo.grid = sms * per_sm;
                     return FTLM_OK;
                 }
@@ -405,7 +405,7 @@ void hvp_retile(HvpPlan<VT> &plan, std::vector<HvpPart<VT>> &parts) {
     for (auto &p : parts) {
         p.tile0 = tiles;
         uint64_t per = std::max<uint64_t>(1, (p.n_reps + ctas - 1) / ctas);
-        if (plan.ops->tile_fixed) per = (per + 31) / 32 * 32;
+        if (plan.ops->tile_fixed) per = plan.a.B > 1 ? per : (per + 31) / 32 * 32;
         else if (per >= 32 * (uint64_t)plan.geo.warps) per = plan.geo.tile_reps;
         else per = std::min<uint64_t>(plan.geo.warps, per);
         p.tile_reps = (int)std::min<uint64_t>(plan.geo.tile_reps, per);
@@ -517,7 +517,7 @@ ftlm_status hvp_plan(const ftlm_sector *s, const PackedSet *ps, std::vector<HvpP
     for (auto &p : parts) mode = mode && p.ent && (p.eoff || p.ecnt);
     plan.mode = mode;
     plan.ops = hvp_ops<VT>(ps->shape, gpl, s->half, esize, mode);
-    if (mode == 1 && ps->K == 1 && B == 1) {  // one thread per representative
+    if (mode == 1 && ps->K == 1 && (B == 1 || sizeof(VT) == 4)) {  // one thread per representative
         const HvpOps<VT> *lane = nullptr;
         if constexpr (sizeof(VT) == 8)
             lane = shape_is_wide(ps->shape) ? hvp_ops_wide_f64(ps->shape, s->half, 2) : hvp_ops_lane_f64(ps->shape);
@@ -757,7 +757,7 @@ ftlm_status hvp_run_one(const ftlm_sector *s, const PackedSet *ps, const ftlm_ba
     if constexpr (sizeof(VT) == 4) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;  // a graph holds one kernel and no scratch
         if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) cudaGetLastError();
-        if (ps->K > 1 && ps->shape >= 0 && !s->d_ent && cap == cudaStreamCaptureStatusNone) {
+        if (ps->shape >= 0 && !s->d_ent && cap == cudaStreamCaptureStatusNone) {
             const ftlm_status st = hvp_run_split<VT>(s, ps, parts[0], B, esize, stream);
             if (st != FTLM_ENOMEM) return st;
         }
