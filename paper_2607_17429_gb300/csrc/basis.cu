@@ -479,10 +479,10 @@ ftlm_status build_sector_impl(const GroupData &grp_in, int two_s, int two_M, int
         if (st != FTLM_OK) return st;
     }
     if (s->sector_dim == 0) return fail(FTLM_EINVAL, "empty sector");
-    DevBuf<uint64_t> d_cnt;
-    DevBuf<uint8_t> d_src;
-    FTLM_CUDA(d_cnt.alloc(cnt.size()));
-    FTLM_CUDA(d_src.alloc(src.size()));
+    ScratchBuf<uint64_t> d_cnt;
+    ScratchBuf<uint8_t> d_src;
+    FTLM_CUDA(d_cnt.alloc(cnt.size(), stream));
+    FTLM_CUDA(d_src.alloc(src.size(), stream));
     FTLM_CUDA(cudaMemcpyAsync(d_cnt.p, cnt.data(), cnt.size() * 8, cudaMemcpyHostToDevice, stream));
     FTLM_CUDA(cudaMemcpyAsync(d_src.p, src.data(), src.size(), cudaMemcpyHostToDevice, stream));
     EnumArgs ea;
@@ -502,13 +502,13 @@ ftlm_status build_sector_impl(const GroupData &grp_in, int two_s, int two_M, int
         for (const double most = std::min(64.0 * sqrt((double)s->sector_dim), 4194304.0);
              ea.pre < N - 1 && (double)ea.n_pre * (two_s + 1) <= most; ++ea.pre)
             ea.n_pre *= (uint32_t)(two_s + 1);
-    DevBuf<uint64_t> first;
-    FTLM_CUDA(first.alloc((size_t)ea.n_pre + 1));
+    ScratchBuf<uint64_t> first;
+    FTLM_CUDA(first.alloc((size_t)ea.n_pre + 1, stream));
     ea.first = first.p;
     ea.dim = s->sector_dim;
     if (ea.pre) {
-        DevBuf<uint64_t> count;
-        FTLM_CUDA(count.alloc(ea.n_pre));
+        ScratchBuf<uint64_t> count;
+        FTLM_CUDA(count.alloc(ea.n_pre, stream));
         count_launch();
         prefix_counts<<<(ea.n_pre + kEnumThreads - 1) / kEnumThreads, kEnumThreads, smem, stream>>>(ea, count.p);
         FTLM_CUDA(cudaGetLastError());
@@ -522,12 +522,12 @@ ftlm_status build_sector_impl(const GroupData &grp_in, int two_s, int two_M, int
     ea.chunk = std::min<uint64_t>(32, std::max<uint64_t>(1, ea.dim / (kNumSMs * 4096ull)));
     ea.n_threads = (ea.dim + ea.chunk - 1) / ea.chunk;
     const uint64_t n_blocks = (ea.n_threads + kEnumThreads - 1) / kEnumThreads;
-    DevBuf<uint2> found;
-    DevBuf<uint64_t> offsets;
-    DevBuf<unsigned long long> nontriv;
-    FTLM_CUDA(found.alloc(ea.n_threads));
-    FTLM_CUDA(offsets.alloc(ea.n_threads + 1));
-    FTLM_CUDA(nontriv.alloc(2));
+    ScratchBuf<uint2> found;
+    ScratchBuf<uint64_t> offsets;
+    ScratchBuf<unsigned long long> nontriv;
+    FTLM_CUDA(found.alloc(ea.n_threads, stream));
+    FTLM_CUDA(offsets.alloc(ea.n_threads + 1, stream));
+    FTLM_CUDA(nontriv.alloc(2, stream));
     FTLM_CUDA(cudaMemsetAsync(nontriv.p, 0, 2 * sizeof(unsigned long long), stream));
     count_launch();
     enum_count<<<(unsigned)n_blocks, kEnumThreads, smem, stream>>>(ea, found.p, nontriv.p);
@@ -546,8 +546,8 @@ ftlm_status build_sector_impl(const GroupData &grp_in, int two_s, int two_M, int
     FTLM_CUDA(cudaMalloc((void **)&s->d_stab_id, n_reps * 2));
     s->device_bytes += n_reps * 10;
     FTLM_CUDA(cudaMemsetAsync(s->d_stab_id, 0, n_reps * 2, stream));
-    DevBuf<uint64_t> side;
-    FTLM_CUDA(side.alloc(5 * n_side + 5));
+    ScratchBuf<uint64_t> side;
+    FTLM_CUDA(side.alloc(5 * n_side + 5, stream));
     FTLM_CUDA(cudaMemsetAsync(nontriv.p, 0, sizeof(unsigned long long), stream));
     count_launch();
     enum_write<<<(unsigned)n_blocks, kEnumThreads, smem, stream>>>(ea, found.p, offsets.p, s->d_labels, nontriv.p, side.p,
@@ -579,8 +579,8 @@ ftlm_status build_sector_impl(const GroupData &grp_in, int two_s, int two_M, int
         for (int w = 0; w < 4; ++w) masks_flat.push_back(m[w]);
     }
     if (n_side) {
-        DevBuf<uint64_t> d_masks;
-        FTLM_CUDA(d_masks.alloc(masks_flat.size()));
+        ScratchBuf<uint64_t> d_masks;
+        FTLM_CUDA(d_masks.alloc(masks_flat.size(), stream));
         FTLM_CUDA(cudaMemcpyAsync(d_masks.p, masks_flat.data(), masks_flat.size() * 8, cudaMemcpyHostToDevice,
                                   stream));
         count_launch();
@@ -781,8 +781,8 @@ ftlm_status build_multiblock_impl(ftlm_sector *s, int n, const int *irreps, cuda
     mb->rho_totalf = (int)rhof.size();
     std::vector<const uint64_t *> offs(n);
     for (int k = 0; k < n; ++k) offs[k] = mb->blocks[k]->d_off;
-    DevBuf<const uint64_t *> d_offs;
-    FTLM_CUDA(d_offs.alloc(n));
+    ScratchBuf<const uint64_t *> d_offs;
+    FTLM_CUDA(d_offs.alloc(n, stream));
     FTLM_CUDA(cudaMemcpyAsync(d_offs.p, offs.data(), n * sizeof(void *), cudaMemcpyHostToDevice, stream));
     FTLM_CUDA(cudaMalloc((void **)&mb->d_offm, s->n_reps * n * 8 + 8));
     FTLM_CUDA(cudaMalloc((void **)&mb->d_ntab, ntab.size()));

@@ -44,6 +44,33 @@ struct DevBuf {
     }
 };
 
+// Device scratch of one call, stream-ordered on its stream: up to kScratchPooled bytes come from the
+// library's pool (packed.cu), which keeps them for the next call, larger buffers from cudaMalloc.  (A
+// Lanczos call of 14 steps on a small block made 15 allocations and frees: 1.02 ms a call, 0.82 ms so.)
+constexpr size_t kScratchPooled = 64u << 20;
+cudaError_t scratch_malloc(void **p, size_t bytes, cudaStream_t stream);
+template <typename T>
+struct ScratchBuf {
+    T *p = nullptr;
+    cudaStream_t st = nullptr;
+    bool pooled = false;
+    ScratchBuf() = default;
+    ScratchBuf(const ScratchBuf &) = delete;
+    ScratchBuf &operator=(const ScratchBuf &) = delete;
+    ~ScratchBuf() { reset(); }
+    void reset() {
+        if (p) pooled ? cudaFreeAsync(p, st) : cudaFree(p);
+        p = nullptr;
+    }
+    cudaError_t alloc(size_t n, cudaStream_t stream) {
+        reset();
+        const size_t bytes = (n ? n : 1) * sizeof(T);
+        st = stream;
+        pooled = bytes <= kScratchPooled;
+        return pooled ? scratch_malloc((void **)&p, bytes, stream) : cudaMalloc((void **)&p, bytes);
+    }
+};
+
 // Exclusive prefix sum (uint64) of n values given by a functor v(i); out[0..n], out[n] = total.
 // Three passes: tile sums, scan of tile sums in one block, tile-local scan with carry-in.
 constexpr int kScanThreads = 512;
@@ -131,8 +158,8 @@ ftlm_status exclusive_scan(F v, uint64_t n, uint64_t *out, cudaStream_t stream, 
         *total = 0;
         return FTLM_OK;
     }
-    DevBuf<uint64_t> tiles;
-    FTLM_CUDA(tiles.alloc(n_tiles + 1));
+    ScratchBuf<uint64_t> tiles;
+    FTLM_CUDA(tiles.alloc(n_tiles + 1, stream));
     count_launch(3);
     scan_tile_sums<<<(unsigned)n_tiles, kScanThreads, 0, stream>>>(v, n, tiles.p);
     FTLM_CUDA(cudaGetLastError());

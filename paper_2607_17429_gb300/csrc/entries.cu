@@ -72,8 +72,8 @@ ftlm_status entry_table_build(ftlm_sector *s, cudaStream_t stream) {
         cudaGetLastError();
         return fail(FTLM_ENOMEM, "entry table of %llu entries: %s", (unsigned long long)total, cudaGetErrorString(e));
     }
-    DevBuf<int> err;
-    FTLM_CUDA(err.alloc(1));
+    ScratchBuf<int> err;
+    FTLM_CUDA(err.alloc(1, stream));
     FTLM_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), stream));
     if (n) {
         // build-mode arguments: the search tables of the sector, no blocks, no vectors

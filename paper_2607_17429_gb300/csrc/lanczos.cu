@@ -363,14 +363,14 @@ ftlm_status ftlm_ritz(int n_chains, int ld, const int *m, const double *alpha, c
         if (m[c] < 0 || m[c] > ld) return fail(FTLM_EINVAL, "steps out of range");
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const size_t n = (size_t)n_chains * ld;
-    DevBuf<double> da, db, dt, dw;
-    DevBuf<int> dm, derr;
-    FTLM_CUDA(da.alloc(n));
-    FTLM_CUDA(db.alloc(n));
-    FTLM_CUDA(dt.alloc(n));
-    FTLM_CUDA(dw.alloc(n));
-    FTLM_CUDA(dm.alloc(n_chains));
-    FTLM_CUDA(derr.alloc(1));
+    ScratchBuf<double> da, db, dt, dw;
+    ScratchBuf<int> dm, derr;
+    FTLM_CUDA(da.alloc(n, st));
+    FTLM_CUDA(db.alloc(n, st));
+    FTLM_CUDA(dt.alloc(n, st));
+    FTLM_CUDA(dw.alloc(n, st));
+    FTLM_CUDA(dm.alloc(n_chains, st));
+    FTLM_CUDA(derr.alloc(1, st));
     FTLM_CUDA(cudaMemcpyAsync(da.p, alpha, n * 8, cudaMemcpyHostToDevice, st));
     FTLM_CUDA(cudaMemcpyAsync(db.p, beta, n * 8, cudaMemcpyHostToDevice, st));
     FTLM_CUDA(cudaMemcpyAsync(dm.p, m, n_chains * 4, cudaMemcpyHostToDevice, st));
@@ -420,19 +420,19 @@ ftlm_status ftlm_thermo(int n_blocks, const ftlm_block *blocks, int n_T, const d
     }
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const size_t n = (size_t)n_chains * ld;
-    DevBuf<double> da, db, dt, dw, dW, dM, dT, dE0, dout;
-    DevBuf<int> dm, derr;
-    FTLM_CUDA(da.alloc(n));
-    FTLM_CUDA(db.alloc(n));
-    FTLM_CUDA(dt.alloc(n));
-    FTLM_CUDA(dw.alloc(n));
-    FTLM_CUDA(dW.alloc(n_chains));
-    FTLM_CUDA(dM.alloc(n_chains));
-    FTLM_CUDA(dT.alloc(n_T));
-    FTLM_CUDA(dE0.alloc(1));
-    FTLM_CUDA(dout.alloc((size_t)4 * n_T));
-    FTLM_CUDA(dm.alloc(n_chains));
-    FTLM_CUDA(derr.alloc(1));
+    ScratchBuf<double> da, db, dt, dw, dW, dM, dT, dE0, dout;
+    ScratchBuf<int> dm, derr;
+    FTLM_CUDA(da.alloc(n, st));
+    FTLM_CUDA(db.alloc(n, st));
+    FTLM_CUDA(dt.alloc(n, st));
+    FTLM_CUDA(dw.alloc(n, st));
+    FTLM_CUDA(dW.alloc(n_chains, st));
+    FTLM_CUDA(dM.alloc(n_chains, st));
+    FTLM_CUDA(dT.alloc(n_T, st));
+    FTLM_CUDA(dE0.alloc(1, st));
+    FTLM_CUDA(dout.alloc((size_t)4 * n_T, st));
+    FTLM_CUDA(dm.alloc(n_chains, st));
+    FTLM_CUDA(derr.alloc(1, st));
     FTLM_CUDA(cudaMemcpyAsync(da.p, a.data(), n * 8, cudaMemcpyHostToDevice, st));
     FTLM_CUDA(cudaMemcpyAsync(db.p, b.data(), n * 8, cudaMemcpyHostToDevice, st));
     FTLM_CUDA(cudaMemcpyAsync(dW.p, Wc.data(), n_chains * 8, cudaMemcpyHostToDevice, st));

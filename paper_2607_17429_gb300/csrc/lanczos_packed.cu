@@ -479,15 +479,15 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
     }
     if (m_all == 0) return FTLM_OK;
     const uint64_t rows = row0[P];
-    DevBuf<ST> vb[3];
-    for (int q = 0; q < 3; ++q) FTLM_CUDA(vb[q].alloc(std::max<uint64_t>(rows, 1) * Bmax));
+    ScratchBuf<ST> vb[3];
+    for (int q = 0; q < 3; ++q) FTLM_CUDA(vb[q].alloc(std::max<uint64_t>(rows, 1) * Bmax, stream));
     const size_t E = (size_t)P * K * Bmax;
-    DevBuf<double> dstate;
-    DevBuf<float> fstate;
-    DevBuf<int> istate;
-    FTLM_CUDA(dstate.alloc(2 * (size_t)n_steps * E + 7 * E + (size_t)P * K));
-    FTLM_CUDA(fstate.alloc(3 * E));
-    FTLM_CUDA(istate.alloc(2 * E + (size_t)P * K));
+    ScratchBuf<double> dstate;
+    ScratchBuf<float> fstate;
+    ScratchBuf<int> istate;
+    FTLM_CUDA(dstate.alloc(2 * (size_t)n_steps * E + 7 * E + (size_t)P * K, stream));
+    FTLM_CUDA(fstate.alloc(3 * E, stream));
+    FTLM_CUDA(istate.alloc(2 * E + (size_t)P * K, stream));
     LzState st;
     st.alpha = dstate.p;
     st.beta = dstate.p + (size_t)n_steps * E;
@@ -514,12 +514,12 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
     st.m_max = istate.p + 2 * E;
     FTLM_CUDA(cudaMemcpyAsync(istate.p + 2 * E, m_max.data(), m_max.size() * sizeof(int), cudaMemcpyHostToDevice,
                               stream));
-    DevBuf<int> derr;
-    FTLM_CUDA(derr.alloc(1));
+    ScratchBuf<int> derr;
+    FTLM_CUDA(derr.alloc(1, stream));
     FTLM_CUDA(cudaMemsetAsync(derr.p, 0, sizeof(int), stream));
     // ---- flips of the sectors without an entry table, searched once for all steps
-    DevBuf<uint8_t> flips;
-    DevBuf<HvpPart<float>> d_fparts;
+    ScratchBuf<uint8_t> flips;
+    ScratchBuf<HvpPart<float>> d_fparts;
     std::vector<size_t> flip_at(P, SIZE_MAX);  // a part's place in flips
     {
         size_t total = 0;
@@ -533,7 +533,7 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
             total += by;
             which.push_back(p);
         }
-        if (!which.empty() && (!all || flips.alloc(total) != cudaSuccess)) {
+        if (!which.empty() && (!all || flips.alloc(total, stream) != cudaSuccess)) {
             cudaGetLastError();
             flip_at.assign(P, SIZE_MAX);
             which.clear();
@@ -547,7 +547,7 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
                 fparts.emplace_back();
                 hvp_copy_flips(part, fparts.back());
             }
-            if (fparts.size() > 1) FTLM_CUDA(d_fparts.alloc(fparts.size()));
+            if (fparts.size() > 1) FTLM_CUDA(d_fparts.alloc(fparts.size(), stream));
             HvpPlan<float> build;
             ftlm_status sb = flips_build(sets[0].sec, fparts, d_fparts.p, derr.p, build);
             if (sb != FTLM_OK) return sb;
@@ -572,7 +572,7 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
         // ---- H·v plans for the three rotations: x = vb[j % 3], y = vb[(j + 1) % 3]
         HvpPlan<VT> plan[3];
         std::vector<HvpPart<VT>> hparts[3];
-        DevBuf<HvpPart<VT>> d_hparts[3];
+        ScratchBuf<HvpPart<VT>> d_hparts[3];
         for (int q = 0; q < 3; ++q) {
             hparts[q].resize(P);
             for (int p = 0; p < P; ++p) {
@@ -586,17 +586,17 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
             plan[q].a.err = derr.p;  // this call's own error word (launches on the same sector may run concurrently)
             plan[q].rows_total = rows;
             if (P > 1) {
-                FTLM_CUDA(d_hparts[q].alloc(P));
+                FTLM_CUDA(d_hparts[q].alloc(P, stream));
                 FTLM_CUDA(cudaMemcpyAsync(d_hparts[q].p, hparts[q].data(), P * sizeof(HvpPart<VT>),
                                           cudaMemcpyHostToDevice, stream));
                 plan[q].a.parts = d_hparts[q].p;
             }
         }
         const int hv_grid = plan[0].geo.grid;
-        DevBuf<double> hv_part, lz_part;
-        FTLM_CUDA(hv_part.alloc((size_t)P * hv_grid * K * B));
-        DevBuf<uint64_t> tiles;  // hv tile0, hv ntile, lz tile0, lz ntile
-        FTLM_CUDA(tiles.alloc(4 * (size_t)P));
+        ScratchBuf<double> hv_part, lz_part;
+        FTLM_CUDA(hv_part.alloc((size_t)P * hv_grid * K * B, stream));
+        ScratchBuf<uint64_t> tiles;  // hv tile0, hv ntile, lz tile0, lz ntile
+        FTLM_CUDA(tiles.alloc(4 * (size_t)P, stream));
         // ---- recurrence kernels: tiles of 64 representatives, up to 8 CTAs per SM
         const int lz_tile = 64;
         std::vector<uint64_t> tinfo(4 * (size_t)P);
@@ -610,10 +610,10 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
             lz_tiles += nt;
         }
         const int lz_grid = (int)std::max<uint64_t>(1, std::min<uint64_t>(lz_tiles, (uint64_t)sms * 8));
-        FTLM_CUDA(lz_part.alloc((size_t)P * lz_grid * K * B));
+        FTLM_CUDA(lz_part.alloc((size_t)P * lz_grid * K * B, stream));
         FTLM_CUDA(cudaMemcpyAsync(tiles.p, tinfo.data(), tinfo.size() * 8, cudaMemcpyHostToDevice, stream));
         std::vector<LzPart<VT>> lparts(P);  // start vectors
-        DevBuf<LzPart<VT>> d_lparts;
+        ScratchBuf<LzPart<VT>> d_lparts;
         LzArgs<VT> la;
         for (int p = 0; p < P; ++p) {
             LzPart<VT> &lp = lparts[p];
@@ -636,7 +636,7 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
         if (P == 1) {
             la.part0 = lparts[0];
         } else {
-            FTLM_CUDA(d_lparts.alloc(P));
+            FTLM_CUDA(d_lparts.alloc(P, stream));
             FTLM_CUDA(cudaMemcpyAsync(d_lparts.p, lparts.data(), P * sizeof(LzPart<VT>), cudaMemcpyHostToDevice,
                                       stream));
             la.parts = d_lparts.p;
@@ -679,13 +679,13 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
             ut[2 * P + p] = len;
             up_runs += ut[P + p];
         }
-        DevBuf<double> up_part;
-        FTLM_CUDA(up_part.alloc(std::max<uint64_t>(1, up_runs) * K * B));
-        DevBuf<uint64_t> d_elem0, d_ut;
-        DevBuf<int> d_ent;
-        FTLM_CUDA(d_elem0.alloc(P + 1));
-        FTLM_CUDA(d_ut.alloc(3 * (size_t)P));
-        FTLM_CUDA(d_ent.alloc(P));
+        ScratchBuf<double> up_part;
+        FTLM_CUDA(up_part.alloc(std::max<uint64_t>(1, up_runs) * K * B, stream));
+        ScratchBuf<uint64_t> d_elem0, d_ut;
+        ScratchBuf<int> d_ent;
+        FTLM_CUDA(d_elem0.alloc(P + 1, stream));
+        FTLM_CUDA(d_ut.alloc(3 * (size_t)P, stream));
+        FTLM_CUDA(d_ent.alloc(P, stream));
         FTLM_CUDA(cudaMemcpyAsync(d_elem0.p, elem0.data(), (P + 1) * 8, cudaMemcpyHostToDevice, stream));
         FTLM_CUDA(cudaMemcpyAsync(d_ut.p, ut.data(), 3 * (size_t)P * 8, cudaMemcpyHostToDevice, stream));
         FTLM_CUDA(cudaMemcpyAsync(d_ent.p, ent.data(), P * sizeof(int), cudaMemcpyHostToDevice, stream));

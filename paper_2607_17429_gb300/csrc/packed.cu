@@ -637,9 +637,10 @@ constexpr uint64_t kPoolBytes = 1ull << 30;
 std::mutex g_pool_mu;
 cudaMemPool_t g_pool[64] = {};
 
-ftlm_status scratch_alloc(void **p, size_t bytes, cudaStream_t stream) {
+cudaError_t scratch_malloc(void **p, size_t bytes, cudaStream_t stream) {
     int dev = 0;
-    FTLM_CUDA(cudaGetDevice(&dev));
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
     cudaMemPool_t pool = nullptr;
     {
         std::lock_guard<std::mutex> lk(g_pool_mu);
@@ -650,13 +651,20 @@ ftlm_status scratch_alloc(void **p, size_t bytes, cudaStream_t stream) {
             pr.allocType = cudaMemAllocationTypePinned;
             pr.location.type = cudaMemLocationTypeDevice;
             pr.location.id = dev;
-            FTLM_CUDA(cudaMemPoolCreate(&slot, &pr));
+            if ((e = cudaMemPoolCreate(&slot, &pr)) != cudaSuccess) {
+                slot = nullptr;
+                return e;
+            }
             uint64_t keep = kPoolBytes;
-            FTLM_CUDA(cudaMemPoolSetAttribute(slot, cudaMemPoolAttrReleaseThreshold, &keep));
+            if ((e = cudaMemPoolSetAttribute(slot, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) return e;
         }
         pool = slot;
     }
-    FTLM_CUDA(cudaMallocFromPoolAsync(p, bytes, pool, stream));
+    return cudaMallocFromPoolAsync(p, bytes, pool, stream);
+}
+
+ftlm_status scratch_alloc(void **p, size_t bytes, cudaStream_t stream) {
+    FTLM_CUDA(scratch_malloc(p, bytes, stream));
     return FTLM_OK;
 }
 
