@@ -109,6 +109,7 @@ struct HvpPart {
     const uint8_t *wtab;     // [n_sid] sum over k of n_k(sid) (0: the orbit has no rows in the set)
     const VT *sqrtS;         // [n_sid], then the inverses [n_sid]
     const VT *Pj[kPMaxK];    // block k: [n_sid][d_k][d_k] projector V V^T
+    const void *xpad;        // padded copy of x's rows (one-thread kernel, B = 1), or null
     const void *x;           // lifted [n_reps * W][B] of the storage type (VT, or FP16 with VT = float)
     void *y;
     uint64_t rep0;           // first representative of this part in rec and eoff (0: the whole sector)
@@ -145,6 +146,9 @@ struct HvpArgs {
     int own;                 // bulk-copy path: prefetch the representative's own rows into shared memory
     unsigned long long wait_limit;
     int *err;
+    const void *pad_x;       // rows of every part, one after another: copied to pad_out before the launch
+    void *pad_out;
+    uint64_t pad_n;          // rows to copy (0: no padded copy)
     double *dot_part;        // [n_parts][gridDim.x][K][B] partial <x_k, y_k>, or null
     unsigned long long *flips;  // profiling: ladder flips processed (one atomic per representative), or null
 };

@@ -80,6 +80,79 @@ __device__ __forceinline__ void lane_row(const ST *__restrict__ x, uint64_t r, u
     }
 }
 
+// Rows whose size is no power of two straddle sectors: a copy of x with rows padded to the next one (PB bytes, 32
+// at most) is made before the launch, and a row then is one aligned load (256 bits for PB = 32) and one
+// sector (s = 3/2 dodecahedron, M = 14, d = 5: 3.84 -> 3.56 ms in FP32, 3.71 -> 3.1 in FP16; what remains is the
+// rate of random sectors, 1.1e11 a second here).  0: the rows are aligned already or too long, or FP64,
+// whose operations bind.
+template <typename ST, int D>
+__host__ __device__ constexpr int lane_pad_bytes() {
+    int pb = 1;
+    while (pb < D * (int)sizeof(ST)) pb *= 2;
+    return pb == D * (int)sizeof(ST) || pb > 32 || sizeof(ST) == 8 ? 0 : pb;
+}
+template <int PB>
+struct PadRow {
+    uint32_t w[PB / 4];
+};
+template <typename ST, int D, int PB>
+__device__ __forceinline__ PadRow<PB> pad_row(const ST *v) {
+    PadRow<PB> r;
+#pragma unroll
+    for (int i = 0; i < PB / 4; ++i) r.w[i] = 0u;
+#pragma unroll
+    for (int g = 0; g < D; ++g) {
+        if constexpr (sizeof(ST) == 2) {
+            r.w[g >> 1] |= (uint32_t)__half_as_ushort(v[g]) << (16 * (g & 1));
+        } else if constexpr (sizeof(ST) == 4) {
+            r.w[g] = __float_as_uint(v[g]);
+        } else {
+            r.w[2 * g] = (uint32_t)__double2loint(v[g]);
+            r.w[2 * g + 1] = (uint32_t)__double2hiint(v[g]);
+        }
+    }
+    return r;
+}
+
+// one thread per row: D elements in, PB bytes out (bandwidth of both)
+template <typename ST, int D, int PB>
+__global__ void __launch_bounds__(256) lane_pad_kernel(const ST *__restrict__ x, uint64_t n, void *out) {
+    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    ST v[D];
+#pragma unroll
+    for (int g = 0; g < D; ++g) v[g] = __ldg(x + i * D + g);
+    const PadRow<PB> r = pad_row<ST, D, PB>(v);
+    uint32_t *o = reinterpret_cast<uint32_t *>(static_cast<char *>(out) + i * PB);
+    if constexpr (PB == 8) {
+        *reinterpret_cast<uint2 *>(o) = make_uint2(r.w[0], r.w[1]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < PB / 16; ++k)
+            reinterpret_cast<uint4 *>(o)[k] = make_uint4(r.w[4 * k], r.w[4 * k + 1], r.w[4 * k + 2], r.w[4 * k + 3]);
+    }
+}
+
+// row r of the padded copy
+template <typename VT, typename ST, int D, int PB>
+__device__ __forceinline__ void padded_row(const void *xpad, uint64_t r, VT (&u)[D]) {
+    const char *p = static_cast<const char *>(xpad) + r * PB;
+    uint32_t w[PB / 4];
+    if constexpr (PB == 8) {
+        const uint2 v = __ldg(reinterpret_cast<const uint2 *>(p));
+        w[0] = v.x, w[1] = v.y;
+    } else if constexpr (PB == 16) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p));
+        w[0] = v.x, w[1] = v.y, w[2] = v.z, w[3] = v.w;
+    } else {
+        asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
+            : "l"(p));
+    }
+#pragma unroll
+    for (int g = 0; g < D; ++g) u[g] = st_get<VT, ST>(span_elem<ST>(w, g));
+}
+
 // CV neighbouring stored elements of row r, columns c .. c + CV - 1
 template <typename VT, typename ST, int CV>
 __device__ __forceinline__ void lane_cols_load(const ST *__restrict__ x, size_t e, bool vec, VT (&u)[CV]) {
@@ -102,8 +175,8 @@ __device__ __forceinline__ void lane_cols_load(const ST *__restrict__ x, size_t 
     for (int v = 0; v < CV; ++v) u[v] = st_get<VT, ST>(__ldg(x + e + v));
 }
 
-// ONE: a single right-hand side (rows of D consecutive elements)
-template <typename VT, typename ST, int D, int CV, bool ONE>
+// ONE: a single right-hand side (rows of D consecutive elements); PB: bytes of the padded copy's rows, 0 for none
+template <typename VT, typename ST, int D, int CV, bool ONE, int PB>
 __global__ void __launch_bounds__(kLaneThreads) hvp_lane_kernel(const __grid_constant__ HvpArgs<VT> a) {
     constexpr int RP = rho_row(D), FL = ONE ? 2 : lane_flips(D, CV);
     extern __shared__ __align__(128) uint8_t smem[];
@@ -217,7 +290,10 @@ __global__ void __launch_bounds__(kLaneThreads) hvp_lane_kernel(const __grid_con
         auto gather = [&](uint64_t r, VT(&u)[D][CV]) {
             if constexpr (ONE) {
                 VT w[D];
-                lane_row<VT, ST, D>(x, r, n_elems, vec, w);
+                if constexpr (PB > 0)
+                    padded_row<VT, ST, D, PB>(P.xpad, r, w);
+                else
+                    lane_row<VT, ST, D>(x, r, n_elems, vec, w);
 #pragma unroll
                 for (int g = 0; g < D; ++g) u[g][0] = w[g];
             } else {
@@ -253,21 +329,32 @@ __global__ void __launch_bounds__(kLaneThreads) hvp_lane_kernel(const __grid_con
 #pragma unroll
             for (int q = 0; q < FL; ++q) gather(r[q].x, u[q]);
 #pragma unroll
-            for (int q = 0; q < FL; ++q) contract(r[q], coef(r[q]), u[q], s, q == 0);
+            for (int q = 0; q < FL; ++q) {
+                if constexpr (sizeof(VT) == 8)  // FP64 operations bind: none for the group's sum
+                    contract(r[q], coef(r[q]), u[q], z, false);
+                else
+                    contract(r[q], coef(r[q]), u[q], s, q == 0);
+            }
+            if constexpr (sizeof(VT) == 4) {
 #pragma unroll
-            for (int g = 0; g < D; ++g)
+                for (int g = 0; g < D; ++g)
 #pragma unroll
-                for (int v = 0; v < CV; ++v) z[g][v] += s[g][v];
+                    for (int v = 0; v < CV; ++v) z[g][v] += s[g][v];
+            }
         }
         for (; e < e1; ++e) {
             const uint2 r0 = __ldg(ent + e);
             VT u0[D][CV], s[D][CV];
             gather(r0.x, u0);
-            contract(r0, coef(r0), u0, s, true);
+            if constexpr (sizeof(VT) == 8) {
+                contract(r0, coef(r0), u0, z, false);
+            } else {
+                contract(r0, coef(r0), u0, s, true);
 #pragma unroll
-            for (int g = 0; g < D; ++g)
+                for (int g = 0; g < D; ++g)
 #pragma unroll
-                for (int v = 0; v < CV; ++v) z[g][v] += s[g][v];
+                    for (int v = 0; v < CV; ++v) z[g][v] += s[g][v];
+            }
         }
         VT xo[D][CV];
         gather(at, xo);
@@ -319,30 +406,48 @@ size_t hvp_lane_smem(const HvpArgs<VT> &a) {
     return (((size_t)a.rho_total * sizeof(VT) + 15) & ~(size_t)15) + (size_t)2 * a.n_bonds + 16;
 }
 
-// CV for the plan's B (FP64: one right-hand side only)
+// CV for the plan's B (FP64: one right-hand side only), PB with a padded copy
 template <typename VT, typename ST, int D, class F>
-auto lane_dispatch(int B, F f) {
+auto lane_dispatch(const HvpArgs<VT> &a, F f) {
+    using std::false_type;
+    using std::true_type;
+    constexpr int PB = lane_pad_bytes<ST, D>();
     if constexpr (sizeof(VT) == 4) {
-        if (B > 1 && lane_cols(B) == 4) return f(std::integral_constant<int, 4>{}, std::false_type{});
-        if (B > 1 && lane_cols(B) == 2) return f(std::integral_constant<int, 2>{}, std::false_type{});
-        if (B > 1) return f(std::integral_constant<int, 1>{}, std::false_type{});
+        if (a.B > 1 && lane_cols(a.B) == 4)
+            return f(std::integral_constant<int, 4>{}, false_type{}, std::integral_constant<int, 0>{});
+        if (a.B > 1 && lane_cols(a.B) == 2)
+            return f(std::integral_constant<int, 2>{}, false_type{}, std::integral_constant<int, 0>{});
+        if (a.B > 1) return f(std::integral_constant<int, 1>{}, false_type{}, std::integral_constant<int, 0>{});
     }
-    return f(std::integral_constant<int, 1>{}, std::true_type{});
+    if (PB > 0 && a.pad_n) return f(std::integral_constant<int, 1>{}, true_type{}, std::integral_constant<int, PB>{});
+    return f(std::integral_constant<int, 1>{}, true_type{}, std::integral_constant<int, 0>{});
 }
 
 template <typename VT, typename ST, int D>
 int hvp_lane_occupancy_t(const HvpArgs<VT> &a, int warps, int) {
     if (warps * 32 != kLaneThreads) return 0;
-    return lane_dispatch<VT, ST, D>(a.B, [&](auto CV, auto ONE) {
-        return hvp_fit_occupancy<hvp_lane_kernel<VT, ST, D, decltype(CV)::value, decltype(ONE)::value>>(
+    return lane_dispatch<VT, ST, D>(a, [&](auto CV, auto ONE, auto PB) {
+        return hvp_fit_occupancy<
+            hvp_lane_kernel<VT, ST, D, decltype(CV)::value, decltype(ONE)::value, decltype(PB)::value>>(
             warps, hvp_lane_smem<VT, ST, D>(a));
     });
 }
 
 template <typename VT, typename ST, int D>
 ftlm_status hvp_lane_launch_t(HvpArgs<VT> a, const HvpGeom &geo, cudaStream_t stream) {
-    lane_dispatch<VT, ST, D>(a.B, [&](auto CV, auto ONE) {
-        hvp_lane_kernel<VT, ST, D, decltype(CV)::value, decltype(ONE)::value>
+    constexpr int PB = lane_pad_bytes<ST, D>();
+    if constexpr (PB > 0) {
+        if (a.pad_n) {
+            lane_pad_kernel<ST, D, PB><<<(unsigned)((a.pad_n + 255) / 256), 256, 0, stream>>>(
+                static_cast<const ST *>(a.pad_x), a.pad_n, a.pad_out);
+            count_launch();
+            FTLM_CUDA(cudaGetLastError());
+        }
+    }
+    if (hvp_lane_smem<VT, ST, D>(a) > 48 * 1024 && hvp_lane_occupancy_t<VT, ST, D>(a, kLaneThreads / 32, 1) < 1)
+        return fail(FTLM_EUNSUPPORTED, "rho table does not fit in shared memory");  // raises the padded kernel's limit
+    lane_dispatch<VT, ST, D>(a, [&](auto CV, auto ONE, auto PBC) {
+        hvp_lane_kernel<VT, ST, D, decltype(CV)::value, decltype(ONE)::value, decltype(PBC)::value>
             <<<(unsigned)geo.grid, kLaneThreads, hvp_lane_smem<VT, ST, D>(a), stream>>>(a);
         return 0;
     });

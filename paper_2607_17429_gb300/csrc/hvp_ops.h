@@ -30,20 +30,24 @@ struct HvpOps {
     ftlm_status (*launch)(HvpArgs<VT>, const HvpGeom &, cudaStream_t);
     int max_threads;
     int tile_fixed;  // one thread per representative: the CTA's threads, the most a tile takes (0: warp kernels)
+    int pad_bytes;   // one thread per representative, B = 1: bytes of a padded row (0: rows stay as they are)
 };
 
 #define FTLM_HVP_OPS_M(VT, ST, SH, GPL, HALF, MODE)                                              \
     HvpOps<VT> {                                                                                   \
         &hvp_occupancy_t<VT, ST, SH, GPL, HALF, MODE>, &hvp_launch_t<VT, ST, SH, GPL, HALF, MODE>, \
-            hvp_max_threads<VT, SH>(), 0                                                           \
+            hvp_max_threads<VT, SH>(), 0, 0                                                        \
     }
 // one thread per representative (table mode, one block, B = 1; hvp_lane.cuh)
 #define FTLM_HVP_LANE_OPS(VT, ST, D) \
-    HvpOps<VT> { &hvp_lane_occupancy_t<VT, ST, D>, &hvp_lane_launch_t<VT, ST, D>, kLaneThreads, kLaneThreads }
+    HvpOps<VT> {                                                                                                   \
+        &hvp_lane_occupancy_t<VT, ST, D>, &hvp_lane_launch_t<VT, ST, D>, kLaneThreads, kLaneThreads,               \
+            lane_pad_bytes<ST, D>()                                                                               \
+    }
 // table mode, multi-block shapes, FP32 arithmetic (hvp_flow.cuh)
 #define FTLM_HVP_FLOW_OPS(ST, SH, CL, BC)                                                      \
     HvpOps<float> {                                                                             \
-        &hvp_flow_occupancy_t<ST, SH, CL, BC>, &hvp_flow_launch_t<ST, SH, CL, BC>, flow_threads<ST, SH, CL>(), 0 \
+        &hvp_flow_occupancy_t<ST, SH, CL, BC>, &hvp_flow_launch_t<ST, SH, CL, BC>, flow_threads<ST, SH, CL>(), 0, 0 \
     }
 #define FTLM_HVP_OPS(VT, ST, SH, GPL, HALF) FTLM_HVP_OPS_M(VT, ST, SH, GPL, HALF, 0)
 
@@ -65,6 +69,13 @@ void hvp_part_of(const ftlm_sector *s, const PackedSet *ps, const ftlm_basis *co
 template <typename VT>
 ftlm_status hvp_plan(const ftlm_sector *s, const PackedSet *ps, std::vector<HvpPart<VT>> &parts, int B, int esize,
                      HvpPlan<VT> &plan, cudaStream_t tune_stream);
+// padded copy of the parts' rows for a plan on the one-thread kernel at B = 1: bytes it needs (0: none), and its
+// use (x: the first part's rows, the others' following; out: that many bytes).  Below 2^18 rows the vector sits in
+// L2 and the copy's launch costs what it saves (2.5e5 rows of five: 91 us without, 88 with).
+template <typename VT>
+size_t hvp_pad_bytes(const HvpPlan<VT> &plan, uint64_t n_rows) {
+    return plan.a.B == 1 && n_rows >= (1u << 18) ? (size_t)n_rows * plan.ops->pad_bytes : 0;
+}
 template <typename VT>
 ftlm_status hvp_launch_plan(const HvpPlan<VT> &plan, double *dot_part, cudaStream_t stream, bool timed);
 // the part as the build kernel sees it (no vectors, no blocks)

@@ -571,6 +571,8 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
         const size_t EB = (size_t)P * K * B;  // entries of this batch
         // ---- H·v plans for the three rotations: x = vb[j % 3], y = vb[(j + 1) % 3]
         HvpPlan<VT> plan[3];
+        ScratchBuf<uint8_t> pad;  // padded rows of the vector an H·v gathers from (B = 1)
+        bool no_pad = false;
         std::vector<HvpPart<VT>> hparts[3];
         ScratchBuf<HvpPart<VT>> d_hparts[3];
         for (int q = 0; q < 3; ++q) {
@@ -583,6 +585,19 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
             }
             ftlm_status s0 = hvp_plan<VT>(sets[0].sec, ps0, hparts[q], B, (int)sizeof(ST), plan[q], stream);
             if (s0 != FTLM_OK) return s0;
+            const size_t pb = hvp_pad_bytes(plan[q], rows / ps0->W);
+            if (pb && !pad.p && !no_pad && pad.alloc(pb, stream) != cudaSuccess) {
+                cudaGetLastError();
+                no_pad = true;
+            }
+            if (pb && !no_pad) {  // the parts' rows follow one another in the vector
+                plan[q].a.pad_x = vb[q].p;
+                plan[q].a.pad_out = pad.p;
+                plan[q].a.pad_n = rows / ps0->W;
+                for (int p = 0; p < P; ++p)
+                    hparts[q][p].xpad = pad.p + row0[p] / ps0->W * (size_t)plan[q].ops->pad_bytes;
+                if (P == 1) plan[q].a.part0.xpad = hparts[q][0].xpad;
+            }
             plan[q].a.err = derr.p;  // this call's own error word (launches on the same sector may run concurrently)
             plan[q].rows_total = rows;
             if (P > 1) {

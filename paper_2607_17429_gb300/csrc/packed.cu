@@ -757,15 +757,20 @@ ftlm_status hvp_run_split(const ftlm_sector *s, const PackedSet *ps, HvpPart<VT>
     return st;
 }
 
+// a call in a stream capture is one kernel without scratch, as a graph keeps it
+static bool capturing(cudaStream_t stream) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) cudaGetLastError();
+    return cap != cudaStreamCaptureStatusNone;
+}
+
 template <typename VT>
 ftlm_status hvp_run_one(const ftlm_sector *s, const PackedSet *ps, const ftlm_basis *const *blocks, int B, int esize,
                         const void *x, void *y, cudaStream_t stream) {
     std::vector<HvpPart<VT>> parts(1);
     hvp_part_of<VT>(s, ps, blocks, x, y, parts[0]);
     if constexpr (sizeof(VT) == 4) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;  // a graph holds one kernel and no scratch
-        if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) cudaGetLastError();
-        if (ps->shape >= 0 && !s->d_ent && cap == cudaStreamCaptureStatusNone) {
+        if (ps->shape >= 0 && !s->d_ent && !capturing(stream)) {
             const ftlm_status st = hvp_run_split<VT>(s, ps, parts[0], B, esize, stream);
             if (st != FTLM_ENOMEM) return st;
         }
@@ -774,7 +779,22 @@ ftlm_status hvp_run_one(const ftlm_sector *s, const PackedSet *ps, const ftlm_ba
     ftlm_status st = hvp_plan<VT>(s, ps, parts, B, esize, plan, stream);
     if (st != FTLM_OK) return st;
     plan.rows_total = ps->rows;
-    return hvp_launch_plan<VT>(plan, nullptr, stream, true);
+    void *pad = nullptr;
+    const size_t pad_bytes = hvp_pad_bytes(plan, s->n_reps);
+    if (pad_bytes && pad_bytes <= kPoolBytes && !capturing(stream)) {
+        if (scratch_malloc(&pad, pad_bytes, stream) == cudaSuccess) {
+            plan.a.pad_x = x;
+            plan.a.pad_out = pad;
+            plan.a.pad_n = s->n_reps;
+            plan.a.part0.xpad = pad;
+        } else {
+            cudaGetLastError();
+            pad = nullptr;
+        }
+    }
+    st = hvp_launch_plan<VT>(plan, nullptr, stream, true);
+    if (pad) cudaFreeAsync(pad, stream);
+    return st;
 }
 
 template ftlm_status hvp_plan<float>(const ftlm_sector *, const PackedSet *, std::vector<HvpPart<float>> &, int,
