@@ -38,7 +38,7 @@ struct HvpOps {
         &hvp_occupancy_t<VT, ST, SH, GPL, HALF, MODE>, &hvp_launch_t<VT, ST, SH, GPL, HALF, MODE>, \
             hvp_max_threads<VT, SH>(), 0, 0                                                        \
     }
-// one thread per representative (table mode, one block, B = 1; hvp_lane.cuh)
+// one thread per representative (table mode, one block; hvp_lane.cuh)
 #define FTLM_HVP_LANE_OPS(VT, ST, D) \
     HvpOps<VT> {                                                                                                   \
         &hvp_lane_occupancy_t<VT, ST, D>, &hvp_lane_launch_t<VT, ST, D>, kLaneThreads, kLaneThreads,               \
@@ -122,11 +122,11 @@ const HvpOps<double> *hvp_ops_multi_f64(int shape, int gpl, bool half);
 const HvpOps<float> *hvp_ops_single_f16(int shape, int gpl, bool half);  // FP16 storage, FP32 arithmetic
 const HvpOps<float> *hvp_ops_multi_f16(int shape, int gpl, bool half);
 // one block of dimension 6..12 (label search with 4 elements per lane, any |G| <= 128):
-// kind 0 search, 1 table, 2 table with one thread per representative (B = 1)
+// kind 0 search, 1 table (FP64), 2 table with one thread per representative (FP64: B = 1)
 const HvpOps<float> *hvp_ops_wide_f32(int shape, bool half, int kind);
 const HvpOps<double> *hvp_ops_wide_f64(int shape, bool half, int kind);
 const HvpOps<float> *hvp_ops_wide_f16(int shape, bool half, int kind);
-// table mode (flips from the sector's entry table), shapes D1..D5, I_h, O_h, T_d; esize 8, 4 or 2
+// table mode (flips from an entry table), shapes D1..D5 (FP64), I_h, O_h, T_d; esize 8, 4 or 2
 const HvpOps<double> *hvp_ops_table_f64(int shape);
 const HvpOps<float> *hvp_ops_table_f32(int shape);
 const HvpOps<float> *hvp_ops_table_f16(int shape);
@@ -136,7 +136,7 @@ const HvpOps<float> *hvp_ops_flow_ih_f32(int B);
 const HvpOps<float> *hvp_ops_flow_ih_f16(int B);
 const HvpOps<float> *hvp_ops_flow_other_f32(int shape, int B);
 const HvpOps<float> *hvp_ops_flow_other_f16(int shape, int B);
-// table mode, one thread per representative: single blocks (shapes D1..D5) at B = 1
+// table mode, one thread per representative: single blocks (shapes D1..D5), FP64 at B = 1
 const HvpOps<double> *hvp_ops_lane_f64(int shape);
 const HvpOps<float> *hvp_ops_lane_f32(int shape);
 const HvpOps<float> *hvp_ops_lane_f16(int shape);

@@ -517,7 +517,9 @@ ftlm_status hvp_plan(const ftlm_sector *s, const PackedSet *ps, std::vector<HvpP
     for (auto &p : parts) mode = mode && p.ent && (p.eoff || p.ecnt);
     plan.mode = mode;
     plan.ops = hvp_ops<VT>(ps->shape, gpl, s->half, esize, mode);
-    if (mode == 1 && ps->K == 1 && (B == 1 || sizeof(VT) == 4)) {  // one thread per representative
+    if (mode == 1 && ps->K == 1 && (B == 1 || sizeof(VT) == 4)) {
+        // one thread per representative: every B in FP32 arithmetic (2 to 9 times the warp kernel's
+        // rate); FP64 operations bind either kernel, so FP64 keeps the warp kernel above B = 1
         const HvpOps<VT> *lane = nullptr;
         if constexpr (sizeof(VT) == 8)
             lane = shape_is_wide(ps->shape) ? hvp_ops_wide_f64(ps->shape, s->half, 2) : hvp_ops_lane_f64(ps->shape);
@@ -680,43 +682,13 @@ void scratch_trim() {
         if (p) cudaMemPoolTrimTo(p, 0);
 }
 
-// One block through the packed kernel: lift x, H·v, lower y (stream-ordered scratch).
-template <typename VT>
-ftlm_status hv_block(const ftlm_basis *b, int B, const VT *x, VT *y, cudaStream_t stream) {
-    const PackedSet *ps = b->ps;
-    const size_t n = ps->rows * (size_t)B;
-    VT *xl = nullptr, *yl = nullptr;
-    ftlm_status st = scratch_alloc((void **)&xl, std::max<size_t>(n, 1) * sizeof(VT), stream);
-    if (st != FTLM_OK) return st;
-    if ((st = scratch_alloc((void **)&yl, std::max<size_t>(n, 1) * sizeof(VT), stream)) != FTLM_OK) {
-        cudaFreeAsync(xl, stream);
-        return st;
-    }
-    const ftlm_basis *one[1] = {b};
-    VT *xb[1] = {const_cast<VT *>(x)};
-    VT *yb[1] = {y};
-    st = lift_impl<VT>(b->sec, ps, one, B, xb, xl, 1, stream);
-    if (st == FTLM_OK) {
-        std::vector<HvpPart<VT>> parts(1);
-        hvp_part_of<VT>(b->sec, ps, one, xl, yl, parts[0]);
-        HvpPlan<VT> plan;
-        st = hvp_plan<VT>(b->sec, ps, parts, B, (int)sizeof(VT), plan, stream);
-        plan.rows_total = ps->rows;
-        if (st == FTLM_OK) st = hvp_launch_plan<VT>(plan, nullptr, stream, true);
-    }
-    if (st == FTLM_OK) st = lift_impl<VT>(b->sec, ps, one, B, yb, yl, 0, stream);
-    cudaFreeAsync(xl, stream);
-    cudaFreeAsync(yl, stream);
-    return st;
-}
-
-// Search path of a multi-block set with FP32 arithmetic: the flips of a run of representatives are
-// searched into an entry workspace by the build kernel, then the table kernel reads them, run after
-// run.  (Search and contraction in one kernel share its 16 warps per SM and its instruction cache:
+// Search path with FP32 arithmetic: the flips of a run of representatives are searched into an entry
+// workspace by the build kernel, then the table kernel reads them, run after run.  (Search and
+// contraction in one kernel share its 16 warps per SM and its instruction cache:
 // 15.7 ms a call for the ten icosidodecahedron irreps at B = 8, of which the search alone is 2.5 ms at the
 // build kernel's occupancy; 8.7 ms this way.)  Sums run in the table path's order, so both paths give
-// the same bits.  Single blocks and FP64 keep the search in the kernel: their contraction leaves the
-// integer pipes idle.  FTLM_ENOMEM (no workspace): the caller takes the one-kernel search.
+// the same bits.  FP64 keeps the search in the kernel: its contraction leaves the integer pipes
+// idle.  FTLM_ENOMEM (no workspace): the caller takes the one-kernel search.
 template <typename VT>
 ftlm_status hvp_run_split(const ftlm_sector *s, const PackedSet *ps, HvpPart<VT> part, int B, int esize, cudaStream_t stream) {
     const int stride = flip_stride(s);
@@ -794,6 +766,29 @@ ftlm_status hvp_run_one(const ftlm_sector *s, const PackedSet *ps, const ftlm_ba
     }
     st = hvp_launch_plan<VT>(plan, nullptr, stream, true);
     if (pad) cudaFreeAsync(pad, stream);
+    return st;
+}
+
+// One block through the packed kernel: lift x, H·v, lower y (stream-ordered scratch).
+template <typename VT>
+ftlm_status hv_block(const ftlm_basis *b, int B, const VT *x, VT *y, cudaStream_t stream) {
+    const PackedSet *ps = b->ps;
+    const size_t n = ps->rows * (size_t)B;
+    VT *xl = nullptr, *yl = nullptr;
+    ftlm_status st = scratch_alloc((void **)&xl, std::max<size_t>(n, 1) * sizeof(VT), stream);
+    if (st != FTLM_OK) return st;
+    if ((st = scratch_alloc((void **)&yl, std::max<size_t>(n, 1) * sizeof(VT), stream)) != FTLM_OK) {
+        cudaFreeAsync(xl, stream);
+        return st;
+    }
+    const ftlm_basis *one[1] = {b};
+    VT *xb[1] = {const_cast<VT *>(x)};
+    VT *yb[1] = {y};
+    st = lift_impl<VT>(b->sec, ps, one, B, xb, xl, 1, stream);
+    if (st == FTLM_OK) st = hvp_run_one<VT>(b->sec, ps, one, B, (int)sizeof(VT), xl, yl, stream);
+    if (st == FTLM_OK) st = lift_impl<VT>(b->sec, ps, one, B, yb, yl, 0, stream);
+    cudaFreeAsync(xl, stream);
+    cudaFreeAsync(yl, stream);
     return st;
 }
 
