@@ -24,9 +24,11 @@ constexpr int kThermoThreads = 256;
 //  - comparisons look at exponents with integer instructions;
 //  - d, e and z live in shared memory, [row][chain], and the next row is loaded ahead of its use;
 //  - every lane walks its own sequence of sweeps, so lanes wait for the longest total sequence of
-//    their warp and not for the longest one of every eigenvalue;
+//    their warp and not for the longest one of every eigenvalue; the warp starts each sweep together and
+//    counts the longest one's rotations, since lanes that the compiler lets run apart pay for
+//    every rotation again (eight chains of a warp: 6.0 ms apart, 4.5 together, one chain 3.9);
 //  - a CTA is one warp and takes ceil(chains / (4 SMs)) chains: every scheduler gets one warp first.
-// 4560 chains of 60 steps: 9.0 ms with one thread per chain in global memory, 6.0 ms now.
+// 4560 chains of 60 steps: 9.0 ms with one thread per chain in global memory, 4.5 ms now.
 
 // 1 / sqrt(h) for normal h: the hardware's approximation and one step of Householder's third-order
 // iteration, y (1 + e / 2 + 3 e^2 / 8) with e = 1 - h y^2 (five FP64 operations).
@@ -48,31 +50,46 @@ static __device__ __forceinline__ bool ql_maybe_small(double e, double d0, doubl
 // e[i] between i and i+1) and the first row z of its orthonormal eigenvector
 // matrix, element i of each array at i * ST.  Implicit QL sweeps with the shift
 // taken from the leading 2x2 block; each Givens rotation is also applied to z.
-// Returns false if an eigenvalue does not converge within 60 sweeps.
+// Called by the whole warp, lanes without a chain with n = 0.  Returns false if an
+// eigenvalue does not converge within 60 sweeps.
 static __device__ bool tridiag_ql(int n, double *d, double *e, double *z, int ST) {
     for (int i = 0; i < n; ++i) z[i * ST] = (i == 0) ? 1.0 : 0.0;
     if (n > 0) e[(n - 1) * ST] = 0.0;
     int l = 0, sweep = 0;
+    bool live = n > 0, ok = true;
     for (;;) {
         int m = l;
-        for (; l < n; m = ++l, sweep = 0) {  // the next eigenvalue that needs a sweep, and its block's end
-            for (; m < n - 1; ++m) {
-                const double em = e[m * ST], d0 = d[m * ST], d1 = d[(m + 1) * ST];
-                if (ql_maybe_small(em, d0, d1) && fabs(em) <= DBL_EPSILON * (fabs(d0) + fabs(d1))) break;
+        if (live) {
+            for (; l < n; m = ++l, sweep = 0) {  // the next eigenvalue that needs a sweep, and its block's end
+                for (; m < n - 1; ++m) {
+                    const double em = e[m * ST], d0 = d[m * ST], d1 = d[(m + 1) * ST];
+                    if (ql_maybe_small(em, d0, d1) && fabs(em) <= DBL_EPSILON * (fabs(d0) + fabs(d1))) break;
+                }
+                if (m != l) break;
             }
-            if (m != l) break;
+            live = l < n;
+            if (live && sweep++ == 60) live = ok = false;
         }
-        if (l >= n) return true;
-        if (sweep++ == 60) return false;
-        const double dl = d[l * ST], el = e[l * ST];
-        double g = (d[(l + 1) * ST] - dl) / (2.0 * el);
-        const double r0 = hypot(g, 1.0);
-        double dhi = d[m * ST], zhi = z[m * ST];
-        g = dhi - dl + el / (g + (g >= 0 ? r0 : -r0));
+        const int longest = __reduce_max_sync(kFull, live ? m - l : 0);
+        if (longest == 0) return ok;
+        double g = 0.0, dhi = 0.0, zhi = 0.0, ei = 0.0, di = 0.0, zi = 0.0;
+        if (live) {
+            const double dl = d[l * ST], el = e[l * ST];
+            g = (d[(l + 1) * ST] - dl) / (2.0 * el);
+            const double r0 = hypot(g, 1.0);
+            dhi = d[m * ST];
+            zhi = z[m * ST];
+            g = dhi - dl + el / (g + (g >= 0 ? r0 : -r0));
+            ei = e[(m - 1) * ST];
+            di = d[(m - 1) * ST];
+            zi = z[(m - 1) * ST];
+        }
         double s = 1.0, c = 1.0, p = 0.0;
-        double ei = e[(m - 1) * ST], di = d[(m - 1) * ST], zi = z[(m - 1) * ST];
-        bool deflated = false;
-        for (int i = m - 1; i >= l; --i) {
+        bool run = live;
+        int i = m - 1;
+        for (int step = 0; step < longest; ++step, --i) {  // the same count in every lane
+            __syncwarp();
+            if (!run || i < l) continue;
             const int nx = (i > l ? i - 1 : i) * ST;
             const double en = e[nx], dn = d[nx], zn = z[nx];
             const double f = s * ei, bb = c * ei;
@@ -90,8 +107,8 @@ static __device__ bool tridiag_ql(int n, double *d, double *e, double *z, int ST
                     d[(i + 1) * ST] = dhi - p;
                     z[(i + 1) * ST] = zhi;
                     e[m * ST] = 0.0;
-                    deflated = true;
-                    break;
+                    run = false;
+                    continue;
                 }
                 s = f / r;
                 c = g / r;
@@ -109,11 +126,12 @@ static __device__ bool tridiag_ql(int n, double *d, double *e, double *z, int ST
             di = dn;
             zi = zn;
         }
-        if (deflated) continue;
-        d[l * ST] = dhi - p;
-        z[l * ST] = zhi;
-        e[l * ST] = g;
-        e[m * ST] = 0.0;
+        if (run) {
+            d[l * ST] = dhi - p;
+            z[l * ST] = zhi;
+            e[l * ST] = g;
+            e[m * ST] = 0.0;
+        }
     }
 }
 
@@ -136,21 +154,19 @@ static __global__ void __launch_bounds__(32) ritz_kernel(int n_chains, int ld, i
     const bool bad = n_raw > ld || n_raw > kMaxSteps;
     if (bad) atomicOr(err, 2);
     const int n = bad || n_raw < 0 ? 0 : n_raw;
-    if (n > 0) {
-        double *d = sd + lane, *e = se + lane, *z = sz + lane;
-        double big = 0.0;
-        for (int i = 0; i < n; ++i) big = fmax(big, fmax(fabs(d[i * per]), i + 1 < n ? fabs(e[i * per]) : 0.0));
-        const int k = big > 0.0 && big < INFINITY ? ilogb(big) : 0;
-        if (k != 0)
-            for (int i = 0; i < n; ++i) {
-                d[i * per] = ldexp(d[i * per], -k);
-                e[i * per] = ldexp(e[i * per], -k);
-            }
-        if (!tridiag_ql(n, d, e, z, per)) atomicOr(err, 1);
+    double *d = sd + lane, *e = se + lane, *z = sz + lane;  // read and written below n only
+    double big = 0.0;
+    for (int i = 0; i < n; ++i) big = fmax(big, fmax(fabs(d[i * per]), i + 1 < n ? fabs(e[i * per]) : 0.0));
+    const int k = big > 0.0 && big < INFINITY ? ilogb(big) : 0;
+    if (k != 0)
         for (int i = 0; i < n; ++i) {
-            if (k != 0) d[i * per] = ldexp(d[i * per], k);
-            z[i * per] *= z[i * per];
+            d[i * per] = ldexp(d[i * per], -k);
+            e[i * per] = ldexp(e[i * per], -k);
         }
+    if (!tridiag_ql(n, d, e, z, per)) atomicOr(err, 1);
+    for (int i = 0; i < n; ++i) {
+        if (k != 0) d[i * per] = ldexp(d[i * per], k);
+        z[i * per] *= z[i * per];
     }
     __syncwarp();
     for (int q = 0; q < nc; ++q) {  // the warp ranks one chain's values at a time (ties in row order)
