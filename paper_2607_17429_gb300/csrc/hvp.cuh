@@ -146,12 +146,48 @@ struct HvpArgs {
     int own;                 // bulk-copy path: prefetch the representative's own rows into shared memory
     unsigned long long wait_limit;
     int *err;
+    int overlap;             // host: the kernel before in the stream may still run at the launch
     const void *pad_x;       // rows of every part, one after another: copied to pad_out before the launch
     void *pad_out;
     uint64_t pad_n;          // rows to copy (0: no padded copy)
     double *dot_part;        // [n_parts][gridDim.x][K][B] partial <x_k, y_k>, or null
     unsigned long long *flips;  // profiling: ladder flips processed (one atomic per representative), or null
 };
+
+// ---------------------------------------------------------------- overlapped launches
+//
+// A kernel whose predecessor in the stream is a kernel of the same call can be launched while that one
+// runs (programmatic stream serialization): the launch and the prologue, rho(g) to shared memory, hide
+// behind it, and prior_done() then waits until the predecessor has ended and its stores are visible (it
+// returns at once in any other launch).  Every thread calls it before it touches what an earlier
+// kernel writes, so the end of a kernel still means the end of all before it.  The 0 that it returns goes
+// into the addresses of the loads that follow, so none of them is moved before the wait.
+// A table kernel behind the build of its entries: 18 representatives of the s = 1/2 icosahedron at B = 8
+// 34.9 -> 28.7 us a call, 1.7e3 of the s = 1 cuboctahedron at B = 24 47.1 -> 44.6, the benchmark sector's five
+// runs of the workspace 8.68 -> 8.51 ms.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ unsigned prior_done() {
+    unsigned zero;
+    asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(zero)::"memory");
+    return zero;
+}
+template <class... P, class... A>
+cudaError_t launch_overlapped(bool overlap, void (*kern)(P...), dim3 grid, int threads, size_t smem,
+                              cudaStream_t stream, const A &...args) {
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = overlap ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kern, args...);
+    return cudaGetLastError();
+}
 
 // ---------------------------------------------------------------- shared-memory layout
 
@@ -431,6 +467,7 @@ __global__ void __launch_bounds__(hvp_max_threads<VT, SH>(), 1) hvp_kernel(const
                                              a.nbuf, a.stage_elems, MODE != 2 && a.tma && a.own, (int)sizeof(ST),
                                              MODE != 1);
     const bool own_on = MODE != 2 && a.tma && a.own;
+    if (MODE == 2) let_next_start();  // the table kernel of these flips may start its prologue
     if (MODE != 1) {
         const size_t n_tab = HALF ? (size_t)a.n_chunks * 4 * kMaxG * 4 : (size_t)kMaxG * 64;
         const uint4 *src0 = reinterpret_cast<const uint4 *>(HALF ? (const void *)a.lut2 : (const void *)a.pos);

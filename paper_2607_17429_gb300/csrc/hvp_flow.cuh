@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(flow_threads<ST, SH, CL>(), 1) hvp_flow_kernel
         for (int i = 0; i < R; ++i) dacc[i][0].zero(), dacc[i][1].zero();
     };
 
-    for (uint64_t t = blockIdx.x; t < a.n_tiles;) {
+    for (uint64_t t = blockIdx.x + prior_done(); t < a.n_tiles;) {
         int p = 0;
         if (a.n_parts > 1) {  // last part whose first tile is <= t
             int lo = 0, hi = a.n_parts - 1;
@@ -533,10 +533,9 @@ template <typename ST, class SH, int CL, int BC>
 ftlm_status hvp_flow_launch_t(HvpArgs<float> a, const HvpGeom &geo, cudaStream_t stream) {
     a.nbuf = geo.nbuf;
     a.tma = geo.tma;
-    hvp_flow_kernel<ST, SH, CL, BC>
-        <<<(unsigned)geo.grid, geo.warps * 32, flow_smem<ST, SH, CL, BC>(a, geo.warps, geo.nbuf), stream>>>(a);
     count_launch();
-    FTLM_CUDA(cudaGetLastError());
+    FTLM_CUDA(launch_overlapped(a.overlap, hvp_flow_kernel<ST, SH, CL, BC>, (unsigned)geo.grid, geo.warps * 32,
+                                flow_smem<ST, SH, CL, BC>(a, geo.warps, geo.nbuf), stream, a));
     return FTLM_OK;
 }
 

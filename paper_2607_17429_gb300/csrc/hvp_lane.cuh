@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kLaneThreads) hvp_lane_kernel(const __grid_con
             dacc[v].zero();
         }
     };
-    for (uint64_t t = blockIdx.x; t < a.n_tiles; t += gridDim.x) {
+    for (uint64_t t = blockIdx.x + prior_done(); t < a.n_tiles; t += gridDim.x) {
         int p = 0;
         if (a.n_parts > 1) {
             int lo = 0, hi = a.n_parts - 1;
@@ -446,13 +446,13 @@ ftlm_status hvp_lane_launch_t(HvpArgs<VT> a, const HvpGeom &geo, cudaStream_t st
     }
     if (hvp_lane_smem<VT, ST, D>(a) > 48 * 1024 && hvp_lane_occupancy_t<VT, ST, D>(a, kLaneThreads / 32, 1) < 1)
         return fail(FTLM_EUNSUPPORTED, "rho table does not fit in shared memory");  // raises the padded kernel's limit
-    lane_dispatch<VT, ST, D>(a, [&](auto CV, auto ONE, auto PBC) {
-        hvp_lane_kernel<VT, ST, D, decltype(CV)::value, decltype(ONE)::value, decltype(PBC)::value>
-            <<<(unsigned)geo.grid, kLaneThreads, hvp_lane_smem<VT, ST, D>(a), stream>>>(a);
-        return 0;
-    });
     count_launch();
-    FTLM_CUDA(cudaGetLastError());
+    const cudaError_t e = lane_dispatch<VT, ST, D>(a, [&](auto CV, auto ONE, auto PBC) {
+        return launch_overlapped(
+            a.overlap, hvp_lane_kernel<VT, ST, D, decltype(CV)::value, decltype(ONE)::value, decltype(PBC)::value>,
+            (unsigned)geo.grid, kLaneThreads, hvp_lane_smem<VT, ST, D>(a), stream, a);
+    });
+    FTLM_CUDA(e);
     return FTLM_OK;
 }
 

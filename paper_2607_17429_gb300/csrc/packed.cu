@@ -722,6 +722,7 @@ ftlm_status hvp_run_split(const ftlm_sector *s, const PackedSet *ps, HvpPart<VT>
             build.a.part0.rep0 = plan.a.part0.rep0 = r;
         if (st == FTLM_OK) st = hvp_launch_plan<float>(build, nullptr, stream, false);
         if (st == FTLM_OK && fresh) st = hvp_plan<VT>(s, ps, parts, B, esize, plan, stream);  // may time the kernel
+        plan.a.overlap = 1;
         if (st == FTLM_OK) st = hvp_launch_plan<VT>(plan, nullptr, stream, false);
     }
     hv_timer_end(stream, e0, e1, ps->rows * (uint64_t)B);
