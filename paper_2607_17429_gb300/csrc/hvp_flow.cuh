@@ -122,6 +122,7 @@ __global__ void __launch_bounds__(flow_threads<ST, SH, CL>(), 1) hvp_flow_kernel
     const int nbuf = a.nbuf;
     const size_t stage_bytes = (size_t)a.stage_elems * sizeof(ST);
     const FlowLayout L = flow_layout(a.G, S, a.n_bonds, K, B, warps, nbuf, stage_bytes);
+    let_next_start();
     float *s_rho = reinterpret_cast<float *>(smem);
     uint8_t *s_bond = smem + L.o_bond;
     double *red = reinterpret_cast<double *>(smem + L.o_red);

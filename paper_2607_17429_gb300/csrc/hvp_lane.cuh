@@ -183,6 +183,7 @@ __global__ void __launch_bounds__(kLaneThreads) hvp_lane_kernel(const __grid_con
     VT *s_rho = reinterpret_cast<VT *>(smem);  // rho(g) of the block, [G][D][RP]
     uint8_t *s_bond = smem + (((size_t)a.rho_total * sizeof(VT) + 15) & ~(size_t)15);
     __shared__ double red[kLaneThreads];
+    let_next_start();
     for (int i = threadIdx.x; i < a.rho_total; i += blockDim.x) s_rho[i] = a.rhoT[i];
     for (int i = threadIdx.x; i < 2 * a.n_bonds; i += blockDim.x) s_bond[i] = a.bonds[i];
     __syncthreads();

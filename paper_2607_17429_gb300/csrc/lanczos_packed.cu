@@ -1,6 +1,6 @@
 // FTLM Lanczos chains on packed sets (Section 2.2 of arXiv 2607.17429), batched
-// through one packed H·v launch per step, with the step loop captured in a
-// CUDA graph.
+// through one packed H·v launch per step, every launch of the step loop overlapping
+// the end of the one before (while profiling, captured in a CUDA graph).
 //
 // The vectors are kept unnormalised: u_j with v_j = s_j u_j.  One step j is
 //   A  y = H u_j (packed H·v) with <u_j, y> per (block, chain) fused into
@@ -220,7 +220,8 @@ __global__ void __launch_bounds__(VEC == 1 ? kUpdElems : kUpdElems / VEC) lzp_up
     __shared__ double red[kUpdElems];
     const int B = a.B, WB = a.W * a.B, K = a.K, tid = threadIdx.x;
     const int tb = tid * VEC % WB, k = a.blk_of_row[tb / B], b = tb % B;
-    const uint64_t run = blockIdx.x, T = (uint64_t)blockDim.x * VEC;
+    let_next_start();
+    const uint64_t run = blockIdx.x + prior_done(), T = (uint64_t)blockDim.x * VEC;
     int p = 0;
     for (int hi = a.n_parts - 1; p < hi;) {  // last part whose first run is <= run (parts without runs come before it)
         const int mid = (p + hi + 1) >> 1;
@@ -324,7 +325,8 @@ constexpr int kFinSlices = 8;
 __global__ void __launch_bounds__(32 * kFinSlices)
     lzp_finalize(int mode, int j, int K, int B, int grid, const uint64_t *tile0, const uint64_t *ntile, const double *part,
                  LzState st, double tol, int scaled) {
-    const int p = blockIdx.x, KB = K * B;
+    let_next_start();
+    const int p = blockIdx.x + (int)prior_done(), KB = K * B;
     const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5, t = blockIdx.y * 32 + lane;
     __shared__ double sl_sum[kFinSlices][32];
     const int k = t / B, b = t % B;
@@ -736,8 +738,12 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
         count_launch();
         lzp_finalize<<<fin_grid, kFinThreads, 0, stream>>>(0, 0, K, B, lz_grid, lz_t0, lz_nt, lz_part.p, st, tol, kScaled);
         FTLM_CUDA(cudaGetLastError());
-        // ---- the step loop (captured once on a private stream, replayed once on the caller's)
-        const bool prof = profiling_on();
+        // ---- the step loop (while profiling: captured once on a private stream, replayed once on the caller's)
+        // Each launch overlaps the end of the one before: jobs of 8 to 14 steps on small sectors take 533, 745 and
+        // 801 us a call, 583, 813 and 821 with the steps in a graph that is built for one replay, 627, 856
+        // and 906 in a graph with overlap (its construction costs more), 22.3 ms in the large batch either way.
+        // Profiling events between the launches keep them apart, and there the graph is the faster form.
+        const bool prof = profiling_on(), overlap = !prof;
         std::vector<cudaEvent_t> ev;
         auto steps = [&](cudaStream_t ss, bool capture) -> ftlm_status {
             for (int j = 0; j < m_all; ++j) {
@@ -751,30 +757,28 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
                     FTLM_CUDA(capture ? cudaEventRecordWithFlags(e0, ss, cudaEventRecordExternal)
                                       : cudaEventRecord(e0, ss));
                 }
+                plan[q].a.overlap = overlap && j > 0;
                 ftlm_status s2 = hvp_launch_plan<VT>(plan[q], hv_part.p, ss, false);
                 if (s2 != FTLM_OK) return s2;
                 if (prof)
                     FTLM_CUDA(capture ? cudaEventRecordWithFlags(ev.back(), ss, cudaEventRecordExternal)
                                       : cudaEventRecord(ev.back(), ss));
                 count_launch();
-                lzp_finalize<<<fin_grid, kFinThreads, 0, ss>>>(1, j, K, B, hv_grid, hv_t0, hv_nt, hv_part.p, st, tol, kScaled);
-                FTLM_CUDA(cudaGetLastError());
+                FTLM_CUDA(launch_overlapped(overlap, lzp_finalize, fin_grid, kFinThreads, 0, ss, 1, j, K, B, hv_grid, hv_t0,
+                                            hv_nt, hv_part.p, st, tol, kScaled));
                 LzUpd<VT> U = ua[q];
                 U.has_prev = j > 0;
                 count_launch();
-                if (up_vec == 4)
-                    lzp_update<VT, ST, 4><<<(unsigned)up_runs, up_threads, 0, ss>>>(U);
-                else
-                    lzp_update<VT, ST, 1><<<(unsigned)up_runs, up_threads, 0, ss>>>(U);
-                FTLM_CUDA(cudaGetLastError());
+                FTLM_CUDA(launch_overlapped(overlap, up_vec == 4 ? lzp_update<VT, ST, 4> : lzp_update<VT, ST, 1>,
+                                            (unsigned)up_runs, up_threads, 0, ss, U));
                 count_launch();
-                lzp_finalize<<<fin_grid, kFinThreads, 0, ss>>>(2, j, K, B, 0, d_ut.p, d_ut.p + P, up_part.p, st, tol, kScaled);
-                FTLM_CUDA(cudaGetLastError());
+                FTLM_CUDA(launch_overlapped(overlap, lzp_finalize, fin_grid, kFinThreads, 0, ss, 2, j, K, B, 0, d_ut.p,
+                                            d_ut.p + P, up_part.p, st, tol, kScaled));
             }
             return FTLM_OK;
         };
         if (prof) profile_flip_counter();  // allocated before the capture (no allocation while capturing)
-        if (use_graph) {
+        if (prof && use_graph) {
             cudaStream_t cap = nullptr;
             FTLM_CUDA(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
             cudaGraph_t graph = nullptr;
