@@ -278,7 +278,7 @@ def _kernel_sha():
     import hashlib
 
     h = hashlib.sha256()
-    for name in ("hvp.cuh", "hvp_lane.cuh", "ptx.cuh", "contract.cuh"):
+    for name in ("hvp.cuh", "hvp_flow.cuh", "hvp_lane.cuh", "ptx.cuh", "contract.cuh"):
         with open(os.path.join(ROOT, "paper_2607_17429_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -615,8 +615,8 @@ CONFIG3 = [("cuboctahedron", 1), ("cuboctahedron", 2), ("icosahedron", 3)]
 def config3(args):
     """Batched SpMM across uneven blocks: s=1/2 and s=1 cuboctahedron (O_h), s=3/2 icosahedron (I_h); every
     M >= 0 sector x every irrep; R = 24 Rademacher vectors (seed 2), 60 steps, FP32 vectors with FP64
-    reductions.  Batched form: per cluster, all sectors as the parts of one launch per kernel, the step loop
-    in one CUDA graph, geometry from the autotuner.  Plain form: FP64, one block at a time."""
+    reductions.  Batched form: per cluster, all sectors as the parts of one launch per kernel,
+    geometry from the autotuner.  Plain form: FP64, one block at a time."""
     import torch
 
     from paper_2607_17429_gb300 import build as pb

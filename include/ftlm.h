@@ -182,11 +182,14 @@ void ftlm_sector_free(ftlm_sector *s);
  * and keeps the table on the device with the sector: 8 bytes per flip plus 8
  * per representative, counted in ftlm_sector_info's device_bytes; n_entries
  * (may be NULL) receives the flip count.  From then on every packed H·v and
- * Lanczos call on blocks of this sector reads the table (the same flips in
- * the same order as the search, so the results are bitwise those of the
- * search path; a single block at one right-hand side runs one thread per
- * representative and sums its flips in entry order, equal to the search path
- * to rounding).  Synchronises cuda_stream; FTLM_ENOMEM if the table does not
+ * Lanczos call on blocks of this sector reads the table.  The flips and their
+ * order are those of the search, and with FP32 arithmetic (FTLM_F32, FTLM_F16)
+ * the search path hands its flips to the same kernels, so the results are
+ * bitwise those of the search path; in FP64 they are too, but for a single
+ * block at one right-hand side (one thread per representative, flips summed in
+ * entry order: equal to rounding).  A search-path call inside a stream capture,
+ * or without room for its scratch, runs search and contraction in one kernel
+ * (equal to rounding).  Synchronises cuda_stream; FTLM_ENOMEM if the table does not
  * fit.  ftlm_sector_free_entries drops the table (back to the search).
  * Neither may run while another call uses the sector.
  */
@@ -230,8 +233,9 @@ void ftlm_basis_free(ftlm_basis *b);
  * looked up in the sorted representative table.
  *   x, y  device [dim][B] of double (FTLM_F64) or float (FTLM_F32), not aliased.
  * The call lifts x into the block's one-block packed layout, runs the packed
- * kernel (see ftlm_hv_packed) and lowers the result into y, with scratch from
- * the stream-ordered allocator (cudaMallocAsync) on cuda_stream.
+ * kernel (see ftlm_hv_packed) and lowers the result into y, with scratch on
+ * cuda_stream from the library's stream-ordered pool (one per device; it keeps
+ * up to 1 GB between calls and returns it when the last sector is freed).
  * Errors: FTLM_EINVAL (null pointers, B out of range), FTLM_ECUDA (launch).
  * A representative missing from the table (impossible for a consistent basis)
  * sets a device flag reported as FTLM_EINTERNAL by ftlm_basis_check; a
@@ -302,11 +306,12 @@ ftlm_status ftlm_multiblock_unpack(const ftlm_multiblock *mb, ftlm_dtype dtype, 
  * same arithmetic as ftlm_hv per block, in lifted coordinates):
  *   y~_k(r) = P_k(r) z_k(r) / sqrt|Stab r| + diag(r) x~_k(r),
  *   z_k(r)  = sum_{bond, sign} c_a sqrt|Stab r'| rho_k(g_e) x~_k(r'),
- * with P_k(r) = V_k(r) V_k(r)^T.  One warp per representative searches and
- * looks up every flipped state once, gathers r''s whole segment (bulk copies
- * into shared memory when B * element size is a multiple of 16 bytes and x is
- * 16-byte aligned, lane loads otherwise) and contracts it with every block's
- * rho(g*)^T.  x, y: device [rows][B], not aliased, 1 <= B <= 32.  Asynchronous
+ * with P_k(r) = V_k(r) V_k(r)^T.  Every flipped state is searched and looked up
+ * once (FP32 arithmetic: into an entry workspace of at most 128 MB from the
+ * stream-ordered scratch pool, run of representatives after run), then r''s
+ * whole segment is gathered (bulk copies into shared memory where segments start on 16
+ * bytes, lane loads otherwise) and contracted with every block's rho(g*)^T.
+ * x, y: device [rows][B], not aliased, 1 <= B <= 32.  Asynchronous
  * on cuda_stream.  Errors: FTLM_EINVAL, FTLM_EUNSUPPORTED (no packed layout),
  * FTLM_ECUDA.  Device-side failures (a representative missing from the table,
  * a bounded wait that gave up) are reported by ftlm_basis_check on any block of
@@ -374,14 +379,18 @@ ftlm_status ftlm_basis_rows(const ftlm_basis *b, int n, const uint64_t *labels, 
  * stored vector is u_j = v_j / s_j and alpha_j = s_j^2 <u_j, H u_j>.  Dot
  * products and norms use exact products of the stored values (FP32 vectors in
  * FTLM_F32), double-float sums per representative and lane, FP64 beyond; the
- * order is fixed, so repeated runs give identical coefficients.  The N_L-step
- * loop is captured in a CUDA graph (FTLM_NO_GRAPH=1 launches it directly).
+ * order is fixed, so repeated runs give identical coefficients.  While
+ * profiling is on the N_L-step loop is captured in a CUDA graph
+ * (FTLM_NO_GRAPH=1 launches it directly).
  * A chain stops after step j when beta_{j+1} <= tol (|alpha_j| + beta_j)
  * (tol = 1e-12 for FP64, 1e-6 for FP32) or when j + 1 = min(n_steps, dim).
  *   alpha, beta   host [R][n_steps]; beta[r][j] = beta_{j+1} (beta[r][m-1] is
  *                 the final residual norm); entries past steps_done are 0.
  *   steps_done    host [R].
- * Device work memory (3 packed [rows][B] vectors and reduction scratch) is
+ * On a sector without an entry table the call searches every flip once and
+ * keeps the result for its steps, if that table (8 bytes per possible flip of
+ * a representative) takes at most twice the call's vectors or 64 MB.  Device work
+ * memory (3 packed [rows][B] vectors, that table and reduction scratch) is
  * allocated and freed by the call.  Synchronises cuda_stream before returning.
  * FTLM_ETIMEOUT / FTLM_EINTERNAL report device-side failures of the H·v.
  */
@@ -392,7 +401,7 @@ ftlm_status ftlm_lanczos(const ftlm_basis *b, ftlm_dtype dtype, int R, int n_ste
 /*
  * ftlm_lanczos on every block of a multi-block set in lockstep.  Sets with a
  * packed layout run the packed path of ftlm_lanczos_sets (one H·v launch and
- * one update launch per step for all blocks, captured in a CUDA graph);
+ * one update launch per step for all blocks);
  * others take one ftlm_hv_multi launch plus per-block recurrence kernels per
  * step.  Block k
  * draws its start vectors with block_ids[k]; results equal ftlm_lanczos per
@@ -409,8 +418,8 @@ ftlm_status ftlm_lanczos_multi(const ftlm_multiblock *mb, ftlm_dtype dtype, int 
  * come from the same group (same permutations, bonds, J and irreps), the same
  * spin and the same irreps in the same order, and have a packed layout.  Each
  * kernel of a step is one launch over the representatives of every set (the
- * sets are the parts of a persistent tile walk), and the step loop is one
- * CUDA graph.  block_ids: host [n_sets][K]; alpha, beta: host
+ * sets are the parts of a persistent tile walk).
+ * block_ids: host [n_sets][K]; alpha, beta: host
  * [n_sets][K][R][n_steps]; steps_done: host [n_sets][K][R].
  */
 ftlm_status ftlm_lanczos_sets(int n_sets, const ftlm_multiblock *const *sets, ftlm_dtype dtype, int R, int n_steps,
@@ -500,8 +509,8 @@ ftlm_status ftlm_thermo_noalloc(int n_chains, int ld, const int *m, const double
  *    charged stay within cap_bytes.  Charged are the resident sector tables
  *    (one per group, 2s, 2M; shared by every job on them), the resident
  *    block tables (one per sector and irrep) and each admitted job's Lanczos
- *    vectors and state (3 packed vectors of rows x min(R, 32) elements plus a
- *    few MB).  A sector is estimated from its dimension before it is built and
+ *    vectors and state (3 packed vectors of rows x min(R, 32) elements, the
+ *    flip table of ftlm_lanczos where it builds one, and a few MB).  A sector is estimated from its dimension before it is built and
  *    charged its actual size after.  Tables that no admitted job references
  *    are evicted least recently used first when room is needed.  A job that
  *    does not fit even with nothing else admitted fails with FTLM_ENOMEM; a
