@@ -311,7 +311,9 @@ ftlm_status ftlm_multiblock_unpack(const ftlm_multiblock *mb, ftlm_dtype dtype, 
  * stream-ordered scratch pool, run of representatives after run), then r''s
  * whole segment is gathered (bulk copies into shared memory where segments start on 16
  * bytes, lane loads otherwise) and contracted with every block's rho(g*)^T.
- * x, y: device [rows][B], not aliased, 1 <= B <= 32.  Asynchronous
+ * x, y: device [rows][B], not aliased, 1 <= B <= 32, each starting on any element
+ * (FP32 arithmetic: an x or y off a pair of elements takes another kernel,
+ * whose sums run in another order: equal to rounding).  Asynchronous
  * on cuda_stream.  Errors: FTLM_EINVAL, FTLM_EUNSUPPORTED (no packed layout),
  * FTLM_ECUDA.  Device-side failures (a representative missing from the table,
  * a bounded wait that gave up) are reported by ftlm_basis_check on any block of

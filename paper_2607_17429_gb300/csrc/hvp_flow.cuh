@@ -21,6 +21,8 @@
 // Icosidodecahedron, M = 0, ten irreps, FP32: B = 8 9.16 -> 5.9 ms, B = 16 16.7 -> 10.5, B = 24 29.9 -> 16.9 (with
 // the contraction left out 4.5, 9.6 and 16.2 ms: at B = 24 the 25 GB of gathers that miss L2 bind, at
 // B = 8 gathers and contraction take 4.5 and 4.4 ms and overlap in part).
+//
+// x and y start on a pair of elements (own rows and outputs move as pairs); hvp_plan takes the kernel of hvp.cuh otherwise.
 #pragma once
 
 #include "hvp.cuh"

@@ -365,7 +365,7 @@ ftlm_status hvp_choose_geom(const HvpOps<VT> *ops, HvpArgs<VT> a, bool tma, HvpG
 // ---------------------------------------------------------------- autotuner
 //
 // With autotuning on, the first plan of every (shape, elements per lane, label
-// width, element type, B, gather path, log2 of the representative count) key
+// width, element type, B, gather path, log2 of the representative count, kernel) key
 // times the candidate geometries on the plan's own buffers and keeps the
 // fastest for the rest of the process: warps per CTA (the kernel's bound down
 // to 4), staging buffers in flight (1..4 on the bulk-copy path), rho tables in
@@ -376,9 +376,10 @@ ftlm_status hvp_choose_geom(const HvpOps<VT> *ops, HvpArgs<VT> a, bool tma, HvpG
 
 struct TuneKey {
     int shape, gpl, half, vt, B, tma, lg, mode;
+    const void *ops;  // the kernel: one shape and B may run in two (x and y on pairs of elements or not)
     bool operator<(const TuneKey &o) const {
-        return std::tie(shape, gpl, half, vt, B, tma, lg, mode) <
-               std::tie(o.shape, o.gpl, o.half, o.vt, o.B, o.tma, o.lg, o.mode);
+        return std::tie(shape, gpl, half, vt, B, tma, lg, mode, ops) <
+               std::tie(o.shape, o.gpl, o.half, o.vt, o.B, o.tma, o.lg, o.mode, o.ops);
     }
 };
 struct TuneVal {
@@ -534,9 +535,13 @@ ftlm_status hvp_plan(const ftlm_sector *s, const PackedSet *ps, std::vector<HvpP
         return fail(FTLM_EUNSUPPORTED, "no compiled packed kernel for shape %d with |G| = %d", ps->shape, s->G);
     bool tma = (B * esize) % 16 == 0;
     // Two right-hand sides per lane: an even B from 6 on (below, most of a warp's flips would be idle; odd
-    // B breaks the 8-byte row loads), segments that start on 16 bytes.
+    // B breaks the 8-byte row loads), segments that start on 16 bytes.  Rows are read and written in pairs of
+    // elements, so x and y have to start on one; views from an odd element on take the warp kernel, whose lane
+    // loads and stores are single elements.
     if constexpr (sizeof(VT) == 4) {
-        if (mode == 1 && ps->K > 1 && (ps->W * B * esize) % 16 == 0) {
+        bool pairs = true;
+        for (auto &p : parts) pairs = pairs && ((uintptr_t)p.x | (uintptr_t)p.y) % (2 * (uintptr_t)esize) == 0;
+        if (mode == 1 && ps->K > 1 && pairs && (ps->W * B * esize) % 16 == 0) {
             const HvpOps<VT> *flow = ps->shape == kShapeIh ? (esize == 2 ? hvp_ops_flow_ih_f16(B) : hvp_ops_flow_ih_f32(B))
                                      : esize == 2          ? hvp_ops_flow_other_f16(ps->shape, B)
                                                            : hvp_ops_flow_other_f32(ps->shape, B);
@@ -560,7 +565,7 @@ ftlm_status hvp_plan(const ftlm_sector *s, const PackedSet *ps, std::vector<HvpP
     if (g_autotune.load() && !plan.ops->tile_fixed && !getenv("FTLM_HV_WARPS") && !getenv("FTLM_HV_NBUF")) {
         int lg = 0;
         while ((1ull << lg) < n_reps_total) ++lg;
-        const TuneKey key{ps->shape, gpl, s->half ? 1 : 0, esize, B, tma ? 1 : 0, lg, mode};
+        const TuneKey key{ps->shape, gpl, s->half ? 1 : 0, esize, B, tma ? 1 : 0, lg, mode, plan.ops};
         std::unique_lock<std::mutex> lk(g_tune_mu);
         auto it = g_tuned.find(key);
         if (it != g_tuned.end()) {
