@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(32 * kFinSlices)
     if (grid) {
         wrap = (uint64_t)grid;
         n = min(nt, wrap);
-        c0 = nt >= wrap ? 0 : t0 % wrap;
+        c0 = t0 % wrap;  // the CTA of the part's first tile: the order is that of its own tiles, whatever came before
         base = (uint64_t)p * wrap;
     }
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
