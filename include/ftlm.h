@@ -188,8 +188,9 @@ void ftlm_sector_free(ftlm_sector *s);
  * bitwise those of the search path; in FP64 they are too, but for a single
  * block at one right-hand side (one thread per representative, flips summed in
  * entry order: equal to rounding).  A search-path call inside a stream capture,
- * or without room for its scratch, runs search and contraction in one kernel
- * (equal to rounding).  Synchronises cuda_stream; FTLM_ENOMEM if the table does not
+ * or without room for its scratch, and the steps of a Lanczos call whose flip
+ * table is too large to build (ftlm_lanczos), run search and contraction in one
+ * kernel (equal to rounding).  Synchronises cuda_stream; FTLM_ENOMEM if the table does not
  * fit.  ftlm_sector_free_entries drops the table (back to the search).
  * Neither may run while another call uses the sector.
  */
@@ -391,9 +392,10 @@ ftlm_status ftlm_basis_rows(const ftlm_basis *b, int n, const uint64_t *labels, 
  *   steps_done    host [R].
  * On a sector without an entry table the call searches every flip once and
  * keeps the result for its steps, if that table (8 bytes per possible flip of
- * a representative) takes at most twice the call's vectors or 64 MB.  Device work
- * memory (3 packed [rows][B] vectors, that table and reduction scratch) is
- * allocated and freed by the call.  Synchronises cuda_stream before returning.
+ * a representative) takes at most twice the block's vectors or 64 MB; a larger
+ * one is not built, and every step searches.  With several sets the bound is
+ * that of each set.  Device work memory (3 packed [rows][B] vectors, those
+ * tables and reduction scratch) is allocated and freed by the call.  Synchronises cuda_stream before returning.
  * FTLM_ETIMEOUT / FTLM_EINTERNAL report device-side failures of the H·v.
  */
 ftlm_status ftlm_lanczos(const ftlm_basis *b, ftlm_dtype dtype, int R, int n_steps, uint64_t seed,
@@ -420,7 +422,9 @@ ftlm_status ftlm_lanczos_multi(const ftlm_multiblock *mb, ftlm_dtype dtype, int 
  * come from the same group (same permutations, bonds, J and irreps), the same
  * spin and the same irreps in the same order, and have a packed layout.  Each
  * kernel of a step is one launch over the representatives of every set (the
- * sets are the parts of a persistent tile walk).
+ * sets are the parts of a persistent tile walk); the H·v is two launches when
+ * some sets read a flip table (ftlm_lanczos) and others search.  With the
+ * autotuner off a set's coefficients are bitwise those it has alone.
  * block_ids: host [n_sets][K]; alpha, beta: host
  * [n_sets][K][R][n_steps]; steps_done: host [n_sets][K][R].
  */

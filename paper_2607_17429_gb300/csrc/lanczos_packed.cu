@@ -16,7 +16,8 @@
 // 1e-6 for FP32 vectors) or when j + 1 = min(n_steps, dim).
 //
 // Several packed sets of the same group and shape (for instance every S^z
-// sector of a cluster) run as the parts of one launch per kernel.
+// sector of a cluster) run as the parts of one launch per kernel (two for the
+// H·v when only some of them have a flip table).
 #include <string.h>
 
 #include <algorithm>
@@ -306,10 +307,14 @@ struct LzState {
     float *coef32;              // [entries][3]
 };
 
+// The partials of a part: n rows of [K][B], the i-th in row base + (first + i) mod wrap.  `first` is the CTA of
+// the part's first tile, so the order is that of its own tiles, whatever part came before.
+struct LzFin {
+    uint64_t base, wrap, first, n;
+};
+
 // One CTA per part and 32 (block, chain) entries: a lane per entry, eight warps over slices of the
-// per-CTA partials of the CTAs that processed tiles of the part (fixed association: it depends on the
-// partial count only).  grid = 0: one partial per tile (or run); else CTA t mod grid took tile t and wrote
-// [p][CTA].
+// part's partials (fixed association: it depends on their count only).
 // mode 0: start-vector norms; 1: alpha_j and the update coefficients; 2: beta_{j+1}.
 // With `scaled` (FP16 storage) the update writes sigma w instead of w, sigma the
 // per-block power of two 2^floor(log2(sqrt(rows) / (16 Hmax))) with Hmax = |J|
@@ -323,30 +328,23 @@ struct LzState {
 constexpr int kFinSlices = 8;
 
 __global__ void __launch_bounds__(32 * kFinSlices)
-    lzp_finalize(int mode, int j, int K, int B, int grid, const uint64_t *tile0, const uint64_t *ntile, const double *part,
-                 LzState st, double tol, int scaled) {
+    lzp_finalize(int mode, int j, int K, int B, const LzFin *fin, const double *part, LzState st, double tol, int scaled) {
     let_next_start();
     const int p = blockIdx.x + (int)prior_done(), KB = K * B;
     const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5, t = blockIdx.y * 32 + lane;
     __shared__ double sl_sum[kFinSlices][32];
     const int k = t / B, b = t % B;
     const size_t e = ((size_t)p * K + k) * B + b;
-    const uint64_t nt = ntile[p], t0 = tile0[p];
-    uint64_t n = nt, c0 = 0, base = t0, wrap = nt;  // partial i sits in row base + (c0 + i) mod wrap
-    if (grid) {
-        wrap = (uint64_t)grid;
-        n = min(nt, wrap);
-        c0 = t0 % wrap;  // the CTA of the part's first tile: the order is that of its own tiles, whatever came before
-        base = (uint64_t)p * wrap;
-    }
+    const LzFin fp = fin[p];
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
     if (t < KB) {
         auto at = [&](uint64_t i) {
-            uint64_t c = c0 + i;
-            if (c >= wrap) c -= wrap;
-            return part[(base + c) * KB + t];
+            uint64_t c = fp.first + i;
+            if (c >= fp.wrap) c -= fp.wrap;
+            return part[(fp.base + c) * KB + t];
         };
         constexpr uint64_t S = kFinSlices;
+        const uint64_t n = fp.n;
         uint64_t i = (uint64_t)sl;
         for (; i + 3 * S < n; i += 4 * S) {  // four interleaved running sums: loads in flight
             const double v0 = at(i), v1 = at(i + S), v2 = at(i + 2 * S), v3 = at(i + 3 * S);
@@ -457,32 +455,75 @@ size_t lanczos_flip_bytes(const ftlm_sector *sec, const PackedSet *ps, int B, in
     return bytes <= std::max<size_t>(64u << 20, 2 * vectors) ? (bytes + 255) / 256 * 256 : 0;
 }
 
+// A launch over the parts with flip tables and one over those without run in turn in every step: a large
+// sector that keeps searching leaves the others their tables (and their sums: the kernel of a part, and so its
+// bits, do not depend on what runs with it).  Five icosidodecahedron sectors at four chains of dimension 3,
+// one of them above the bound, 14 steps: 31.1 ms with a search in every part, 24.4 so.
+template <typename VT>
+struct LzHv {
+    int p0 = 0, n = 0;           // parts
+    HvpPlan<VT> plan[3];         // of the three rotations: x = vb[j % 3], y = vb[(j + 1) % 3]
+    std::vector<HvpPart<VT>> parts[3];
+    ScratchBuf<HvpPart<VT>> d_parts[3];
+    size_t row = 0;              // first row of its dot partials
+};
+
 template <typename VT, typename ST>
-ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_steps, uint64_t seed, int rng,
+ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets_in, int R, int n_steps, uint64_t seed, int rng,
                               cudaStream_t stream, double *alpha, double *beta, int *steps_done) {
     constexpr bool kScaled = sizeof(ST) < sizeof(VT);
-    const int P = (int)sets.size();
-    const PackedSet *ps0 = sets[0].ps;
+    const int P = (int)sets_in.size();
+    const PackedSet *ps0 = sets_in[0].ps;
     const int K = ps0->K;
     const size_t out_n = (size_t)P * K * R;
     for (size_t i = 0; i < out_n; ++i) steps_done[i] = 0;
     for (size_t i = 0; i < out_n * n_steps; ++i) alpha[i] = beta[i] = 0.0;
     const int Bmax = std::min(R, kMaxB);
-    std::vector<uint64_t> row0(P + 1, 0);
-    std::vector<int> m_max((size_t)P * K);
+    auto limit = [&](const LzSetIn &in, int k) {
+        const int lim = in.n_steps > 0 ? std::min(in.n_steps, n_steps) : n_steps;
+        return (int)std::min<uint64_t>((uint64_t)lim, in.blocks[k]->dim);
+    };
     int m_all = 0;
-    for (int p = 0; p < P; ++p) {
-        row0[p + 1] = row0[p] + sets[p].ps->rows;
-        for (int k = 0; k < K; ++k) {
-            const int lim = sets[p].n_steps > 0 ? std::min(sets[p].n_steps, n_steps) : n_steps;
-            m_max[(size_t)p * K + k] = (int)std::min<uint64_t>((uint64_t)lim, sets[p].blocks[k]->dim);
-            m_all = std::max(m_all, m_max[(size_t)p * K + k]);
-        }
+    uint64_t rows = 0;
+    for (const LzSetIn &in : sets_in) {
+        rows += in.ps->rows;
+        for (int k = 0; k < K; ++k) m_all = std::max(m_all, limit(in, k));
     }
     if (m_all == 0) return FTLM_OK;
-    const uint64_t rows = row0[P];
     ScratchBuf<ST> vb[3];
     for (int q = 0; q < 3; ++q) FTLM_CUDA(vb[q].alloc(std::max<uint64_t>(rows, 1) * Bmax, stream));
+    // ---- flips of the sectors without an entry table, searched once for all steps; parts with tables first
+    ScratchBuf<uint8_t> flips;
+    std::vector<LzSetIn> sets;
+    std::vector<int> orig;        // place of each part in sets_in
+    std::vector<size_t> flip_at;  // a part's place in flips
+    int n_table = 0;
+    {
+        std::vector<size_t> by(P);
+        size_t total = 0;
+        for (int i = 0; i < P; ++i)
+            total += by[i] = lanczos_flip_bytes(sets_in[i].sec, sets_in[i].ps, Bmax, (int)sizeof(ST));
+        if (total && flips.alloc(total, stream) != cudaSuccess) {
+            cudaGetLastError();
+            by.assign(P, 0);
+        }
+        size_t at = 0;
+        for (bool table : {true, false})
+            for (int i = 0; i < P; ++i) {
+                if ((sets_in[i].sec->d_ent || by[i]) != table) continue;
+                sets.push_back(sets_in[i]);
+                orig.push_back(i);
+                flip_at.push_back(by[i] ? at : SIZE_MAX);
+                at += by[i];
+                n_table += table;
+            }
+    }
+    std::vector<uint64_t> row0(P + 1, 0);
+    std::vector<int> m_max((size_t)P * K);
+    for (int p = 0; p < P; ++p) {
+        row0[p + 1] = row0[p] + sets[p].ps->rows;
+        for (int k = 0; k < K; ++k) m_max[(size_t)p * K + k] = limit(sets[p], k);
+    }
     const size_t E = (size_t)P * K * Bmax;
     ScratchBuf<double> dstate;
     ScratchBuf<float> fstate;
@@ -519,45 +560,25 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
     ScratchBuf<int> derr;
     FTLM_CUDA(derr.alloc(1, stream));
     FTLM_CUDA(cudaMemsetAsync(derr.p, 0, sizeof(int), stream));
-    // ---- flips of the sectors without an entry table, searched once for all steps
-    ScratchBuf<uint8_t> flips;
     ScratchBuf<HvpPart<float>> d_fparts;
-    std::vector<size_t> flip_at(P, SIZE_MAX);  // a part's place in flips
-    {
-        size_t total = 0;
-        bool all = true;
-        std::vector<int> which;
-        for (int p = 0; p < P; ++p) {
-            if (sets[p].sec->d_ent || sets[p].sec->n_reps == 0) continue;
-            const size_t by = lanczos_flip_bytes(sets[p].sec, sets[p].ps, Bmax, (int)sizeof(ST));
-            all = all && by;
-            flip_at[p] = total;
-            total += by;
-            which.push_back(p);
+    if (flips.p) {
+        std::vector<HvpPart<float>> fparts;
+        for (int p = 0; p < n_table; ++p) {
+            if (flip_at[p] == SIZE_MAX) continue;
+            HvpPart<VT> part;
+            hvp_part_of<VT>(sets[p].sec, sets[p].ps, sets[p].blocks, nullptr, nullptr, part);
+            lz_use_flips(part, flips.p + flip_at[p], flip_stride(sets[p].sec));
+            fparts.emplace_back();
+            hvp_copy_flips(part, fparts.back());
         }
-        if (!which.empty() && (!all || flips.alloc(total, stream) != cudaSuccess)) {
-            cudaGetLastError();
-            flip_at.assign(P, SIZE_MAX);
-            which.clear();
-        }
-        if (!which.empty()) {
-            std::vector<HvpPart<float>> fparts;
-            for (int p : which) {
-                HvpPart<VT> part;
-                hvp_part_of<VT>(sets[p].sec, sets[p].ps, sets[p].blocks, nullptr, nullptr, part);
-                lz_use_flips(part, flips.p + flip_at[p], flip_stride(sets[p].sec));
-                fparts.emplace_back();
-                hvp_copy_flips(part, fparts.back());
-            }
-            if (fparts.size() > 1) FTLM_CUDA(d_fparts.alloc(fparts.size(), stream));
-            HvpPlan<float> build;
-            ftlm_status sb = flips_build(sets[0].sec, fparts, d_fparts.p, derr.p, build);
-            if (sb != FTLM_OK) return sb;
-            if (fparts.size() > 1)
-                FTLM_CUDA(cudaMemcpyAsync(d_fparts.p, fparts.data(), fparts.size() * sizeof(HvpPart<float>),
-                                          cudaMemcpyHostToDevice, stream));
-            if ((sb = hvp_launch_plan<float>(build, nullptr, stream, false)) != FTLM_OK) return sb;
-        }
+        if (fparts.size() > 1) FTLM_CUDA(d_fparts.alloc(fparts.size(), stream));
+        HvpPlan<float> build;
+        ftlm_status sb = flips_build(sets[0].sec, fparts, d_fparts.p, derr.p, build);
+        if (sb != FTLM_OK) return sb;
+        if (fparts.size() > 1)
+            FTLM_CUDA(cudaMemcpyAsync(d_fparts.p, fparts.data(), fparts.size() * sizeof(HvpPart<float>),
+                                      cudaMemcpyHostToDevice, stream));
+        if ((sb = hvp_launch_plan<float>(build, nullptr, stream, false)) != FTLM_OK) return sb;
     }
     int dev = 0, sms = kNumSMs;
     FTLM_CUDA(cudaGetDevice(&dev));
@@ -571,64 +592,73 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
     for (int chain0 = 0; chain0 < R; chain0 += Bmax) {
         const int B = std::min(Bmax, R - chain0);
         const size_t EB = (size_t)P * K * B;  // entries of this batch
-        // ---- H·v plans for the three rotations: x = vb[j % 3], y = vb[(j + 1) % 3]
-        HvpPlan<VT> plan[3];
+        LzHv<VT> hv[2];
+        hv[0].n = hv[1].p0 = n_table;
+        hv[1].n = P - n_table;
         ScratchBuf<uint8_t> pad;  // padded rows of the vector an H·v gathers from (B = 1)
         bool no_pad = false;
-        std::vector<HvpPart<VT>> hparts[3];
-        ScratchBuf<HvpPart<VT>> d_hparts[3];
-        for (int q = 0; q < 3; ++q) {
-            hparts[q].resize(P);
-            for (int p = 0; p < P; ++p) {
-                hvp_part_of<VT>(sets[p].sec, sets[p].ps, sets[p].blocks, vb[q].p + row0[p] * B,
-                                vb[(q + 1) % 3].p + row0[p] * B, hparts[q][p]);
-                if (flip_at[p] != SIZE_MAX)
-                    lz_use_flips(hparts[q][p], flips.p + flip_at[p], flip_stride(sets[p].sec));
+        size_t hv_rows = 0;  // rows of dot partials
+        for (LzHv<VT> &h : hv) {
+            if (h.n == 0) continue;
+            const uint64_t reps0 = row0[h.p0] / ps0->W, reps = row0[h.p0 + h.n] / ps0->W - reps0;
+            for (int q = 0; q < 3; ++q) {
+                HvpPlan<VT> &plan = h.plan[q];
+                h.parts[q].resize(h.n);
+                for (int i = 0; i < h.n; ++i) {
+                    const int p = h.p0 + i;
+                    hvp_part_of<VT>(sets[p].sec, sets[p].ps, sets[p].blocks, vb[q].p + row0[p] * B,
+                                    vb[(q + 1) % 3].p + row0[p] * B, h.parts[q][i]);
+                    if (flip_at[p] != SIZE_MAX)
+                        lz_use_flips(h.parts[q][i], flips.p + flip_at[p], flip_stride(sets[p].sec));
+                }
+                ftlm_status s0 = hvp_plan<VT>(sets[h.p0].sec, ps0, h.parts[q], B, (int)sizeof(ST), plan, stream);
+                if (s0 != FTLM_OK) return s0;
+                const size_t pb = hvp_pad_bytes(plan, reps);
+                if (pb && !pad.p && !no_pad && pad.alloc(pb, stream) != cudaSuccess) {
+                    cudaGetLastError();
+                    no_pad = true;
+                }
+                if (pb && !no_pad) {  // the parts' rows follow one another in the vector
+                    plan.a.pad_x = vb[q].p + row0[h.p0] * B;
+                    plan.a.pad_out = pad.p;
+                    plan.a.pad_n = reps;
+                    for (int i = 0; i < h.n; ++i)
+                        h.parts[q][i].xpad = pad.p + (row0[h.p0 + i] / ps0->W - reps0) * (size_t)plan.ops->pad_bytes;
+                    if (h.n == 1) plan.a.part0.xpad = h.parts[q][0].xpad;
+                }
+                plan.a.err = derr.p;  // this call's own error word (launches on the same sector may run concurrently)
+                plan.rows_total = row0[h.p0 + h.n] - row0[h.p0];
+                if (h.n > 1) {
+                    FTLM_CUDA(h.d_parts[q].alloc(h.n, stream));
+                    FTLM_CUDA(cudaMemcpyAsync(h.d_parts[q].p, h.parts[q].data(), h.n * sizeof(HvpPart<VT>),
+                                              cudaMemcpyHostToDevice, stream));
+                    plan.a.parts = h.d_parts[q].p;
+                }
             }
-            ftlm_status s0 = hvp_plan<VT>(sets[0].sec, ps0, hparts[q], B, (int)sizeof(ST), plan[q], stream);
-            if (s0 != FTLM_OK) return s0;
-            const size_t pb = hvp_pad_bytes(plan[q], rows / ps0->W);
-            if (pb && !pad.p && !no_pad && pad.alloc(pb, stream) != cudaSuccess) {
-                cudaGetLastError();
-                no_pad = true;
-            }
-            if (pb && !no_pad) {  // the parts' rows follow one another in the vector
-                plan[q].a.pad_x = vb[q].p;
-                plan[q].a.pad_out = pad.p;
-                plan[q].a.pad_n = rows / ps0->W;
-                for (int p = 0; p < P; ++p)
-                    hparts[q][p].xpad = pad.p + row0[p] / ps0->W * (size_t)plan[q].ops->pad_bytes;
-                if (P == 1) plan[q].a.part0.xpad = hparts[q][0].xpad;
-            }
-            plan[q].a.err = derr.p;  // this call's own error word (launches on the same sector may run concurrently)
-            plan[q].rows_total = rows;
-            if (P > 1) {
-                FTLM_CUDA(d_hparts[q].alloc(P, stream));
-                FTLM_CUDA(cudaMemcpyAsync(d_hparts[q].p, hparts[q].data(), P * sizeof(HvpPart<VT>),
-                                          cudaMemcpyHostToDevice, stream));
-                plan[q].a.parts = d_hparts[q].p;
-            }
+            h.row = hv_rows;
+            hv_rows += (size_t)h.n * h.plan[0].geo.grid;
         }
-        const int hv_grid = plan[0].geo.grid;
         ScratchBuf<double> hv_part, lz_part;
-        FTLM_CUDA(hv_part.alloc((size_t)P * hv_grid * K * B, stream));
-        ScratchBuf<uint64_t> tiles;  // hv tile0, hv ntile, lz tile0, lz ntile
-        FTLM_CUDA(tiles.alloc(4 * (size_t)P, stream));
+        FTLM_CUDA(hv_part.alloc(hv_rows * K * B, stream));
+        ScratchBuf<LzFin> fin;  // partials of the H·v, of the start vectors and of the update
+        FTLM_CUDA(fin.alloc(3 * (size_t)P, stream));
+        std::vector<LzFin> hfin(3 * (size_t)P);
+        auto cta_partials = [](uint64_t tile0, uint64_t ntile, uint64_t row, int local, int grid) {
+            const uint64_t g = (uint64_t)grid;  // CTA t mod grid took tile t and wrote [local part][CTA]
+            return LzFin{row + (uint64_t)local * g, g, tile0 % g, std::min(ntile, g)};
+        };
+        for (const LzHv<VT> &h : hv)
+            for (int i = 0; i < h.n; ++i)
+                hfin[h.p0 + i] = cta_partials(h.plan[0].tile0[i], h.plan[0].ntile[i], h.row, i, h.plan[0].geo.grid);
         // ---- recurrence kernels: tiles of 64 representatives, up to 8 CTAs per SM
         const int lz_tile = 64;
-        std::vector<uint64_t> tinfo(4 * (size_t)P);
-        uint64_t lz_tiles = 0;
-        for (int p = 0; p < P; ++p) {
-            tinfo[p] = plan[0].tile0[p];
-            tinfo[P + p] = plan[0].ntile[p];
-            const uint64_t nt = (sets[p].sec->n_reps + lz_tile - 1) / lz_tile;
-            tinfo[2 * P + p] = lz_tiles;
-            tinfo[3 * P + p] = nt;
-            lz_tiles += nt;
-        }
+        std::vector<uint64_t> lz_tile0(P + 1, 0);
+        for (int p = 0; p < P; ++p) lz_tile0[p + 1] = lz_tile0[p] + (sets[p].sec->n_reps + lz_tile - 1) / lz_tile;
+        const uint64_t lz_tiles = lz_tile0[P];
         const int lz_grid = (int)std::max<uint64_t>(1, std::min<uint64_t>(lz_tiles, (uint64_t)sms * 8));
         FTLM_CUDA(lz_part.alloc((size_t)P * lz_grid * K * B, stream));
-        FTLM_CUDA(cudaMemcpyAsync(tiles.p, tinfo.data(), tinfo.size() * 8, cudaMemcpyHostToDevice, stream));
+        for (int p = 0; p < P; ++p)
+            hfin[P + p] = cta_partials(lz_tile0[p], lz_tile0[p + 1] - lz_tile0[p], 0, p, lz_grid);
         std::vector<LzPart<VT>> lparts(P);  // start vectors
         ScratchBuf<LzPart<VT>> d_lparts;
         LzArgs<VT> la;
@@ -636,7 +666,7 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
             LzPart<VT> &lp = lparts[p];
             memset(&lp, 0, sizeof(lp));
             lp.n_reps = sets[p].sec->n_reps;
-            lp.tile0 = tinfo[2 * P + p];
+            lp.tile0 = lz_tile0[p];
             lp.rec = sets[p].sec->d_rec;
             lp.ntab = sets[p].ps->d_ntab;
             for (int k = 0; k < K; ++k) {
@@ -662,8 +692,8 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
         la.n_tiles = lz_tiles;
         la.tile_reps = lz_tile;
         la.B = B;
-        la.BT = plan[0].a.BT;
-        la.lgBT = plan[0].a.lgBT;
+        la.BT = hv[n_table ? 0 : 1].plan[0].a.BT;
+        la.lgBT = hv[n_table ? 0 : 1].plan[0].a.lgBT;
         {
             int z = 0;
             for (int k = 0; k < K; ++k) {
@@ -676,14 +706,13 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
         la.chain0 = (uint32_t)chain0;
         la.key0 = (uint32_t)seed;
         la.norm_part = lz_part.p;
-        const uint64_t *hv_t0 = tiles.p, *hv_nt = tiles.p + P, *lz_t0 = tiles.p + 2 * P, *lz_nt = tiles.p + 3 * P;
         // flat update: W B 2^k elements per CTA at a time, one run of representatives per CTA
         const int WB = ps0->W * B, up_vec = B % 4 == 0 ? 4 : 1;
         int n_sub = 1;
         while (2 * n_sub * WB <= (up_vec == 4 ? kUpdElems : kUpdElems / 2)) n_sub *= 2;
         const int up_threads = n_sub * WB / up_vec;
         const uint64_t up_ctas = (uint64_t)sms * std::max(1, std::min(8, kUpdThreads / up_threads));
-        std::vector<uint64_t> elem0(P + 1), ut(3 * (size_t)P);  // runs: first, count, representatives
+        std::vector<uint64_t> elem0(P + 1), ut(2 * (size_t)P);  // runs: first, representatives
         std::vector<int> ent(P);
         uint64_t up_runs = 0;
         for (int p = 0; p <= P; ++p) elem0[p] = row0[p] * (uint64_t)B;
@@ -692,19 +721,21 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
             const uint64_t len = n_sub * std::max<uint64_t>(kUpdMinSteps, (steps + up_ctas - 1) / up_ctas);
             ent[p] = p * K * B;
             ut[p] = up_runs;
-            ut[P + p] = (n + len - 1) / len;
-            ut[2 * P + p] = len;
-            up_runs += ut[P + p];
+            ut[P + p] = len;
+            const uint64_t runs = (n + len - 1) / len;
+            hfin[2 * P + p] = LzFin{up_runs, runs, 0, runs};
+            up_runs += runs;
         }
         ScratchBuf<double> up_part;
         FTLM_CUDA(up_part.alloc(std::max<uint64_t>(1, up_runs) * K * B, stream));
         ScratchBuf<uint64_t> d_elem0, d_ut;
         ScratchBuf<int> d_ent;
         FTLM_CUDA(d_elem0.alloc(P + 1, stream));
-        FTLM_CUDA(d_ut.alloc(3 * (size_t)P, stream));
+        FTLM_CUDA(d_ut.alloc(2 * (size_t)P, stream));
         FTLM_CUDA(d_ent.alloc(P, stream));
         FTLM_CUDA(cudaMemcpyAsync(d_elem0.p, elem0.data(), (P + 1) * 8, cudaMemcpyHostToDevice, stream));
-        FTLM_CUDA(cudaMemcpyAsync(d_ut.p, ut.data(), 3 * (size_t)P * 8, cudaMemcpyHostToDevice, stream));
+        FTLM_CUDA(cudaMemcpyAsync(d_ut.p, ut.data(), 2 * (size_t)P * 8, cudaMemcpyHostToDevice, stream));
+        FTLM_CUDA(cudaMemcpyAsync(fin.p, hfin.data(), hfin.size() * sizeof(LzFin), cudaMemcpyHostToDevice, stream));
         FTLM_CUDA(cudaMemcpyAsync(d_ent.p, ent.data(), P * sizeof(int), cudaMemcpyHostToDevice, stream));
         const dim3 fin_grid(P, (K * B + 31) / 32);
         constexpr int kFinThreads = 32 * kFinSlices;
@@ -722,7 +753,7 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
             for (int k = 0; k < K; ++k) U.zrow[k + 1] = U.zrow[k] + ps0->dims[k];
             U.n_sub = n_sub;
             U.run0 = d_ut.p;
-            U.run_reps = d_ut.p + 2 * P;
+            U.run_reps = d_ut.p + P;
             U.elem0 = d_elem0.p;
             U.entry0 = d_ent.p;
             U.y = vb[(q + 1) % 3].p;
@@ -736,7 +767,7 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
         ftlm_status s1 = lzp_start_launch<VT, ST>(K, la, lz_grid, stream);
         if (s1 != FTLM_OK) return s1;
         count_launch();
-        lzp_finalize<<<fin_grid, kFinThreads, 0, stream>>>(0, 0, K, B, lz_grid, lz_t0, lz_nt, lz_part.p, st, tol, kScaled);
+        lzp_finalize<<<fin_grid, kFinThreads, 0, stream>>>(0, 0, K, B, fin.p + P, lz_part.p, st, tol, kScaled);
         FTLM_CUDA(cudaGetLastError());
         // ---- the step loop (while profiling: captured once on a private stream, replayed once on the caller's)
         // Each launch overlaps the end of the one before: jobs of 8 to 14 steps on small sectors take 533, 745 and
@@ -757,23 +788,26 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
                     FTLM_CUDA(capture ? cudaEventRecordWithFlags(e0, ss, cudaEventRecordExternal)
                                       : cudaEventRecord(e0, ss));
                 }
-                plan[q].a.overlap = overlap && j > 0;
-                ftlm_status s2 = hvp_launch_plan<VT>(plan[q], hv_part.p, ss, false);
-                if (s2 != FTLM_OK) return s2;
+                for (LzHv<VT> &h : hv) {
+                    if (h.n == 0) continue;
+                    h.plan[q].a.overlap = overlap && j > 0;
+                    ftlm_status s2 = hvp_launch_plan<VT>(h.plan[q], hv_part.p + h.row * K * B, ss, false);
+                    if (s2 != FTLM_OK) return s2;
+                }
                 if (prof)
                     FTLM_CUDA(capture ? cudaEventRecordWithFlags(ev.back(), ss, cudaEventRecordExternal)
                                       : cudaEventRecord(ev.back(), ss));
                 count_launch();
-                FTLM_CUDA(launch_overlapped(overlap, lzp_finalize, fin_grid, kFinThreads, 0, ss, 1, j, K, B, hv_grid, hv_t0,
-                                            hv_nt, hv_part.p, st, tol, kScaled));
+                FTLM_CUDA(launch_overlapped(overlap, lzp_finalize, fin_grid, kFinThreads, 0, ss, 1, j, K, B, fin.p,
+                                            hv_part.p, st, tol, kScaled));
                 LzUpd<VT> U = ua[q];
                 U.has_prev = j > 0;
                 count_launch();
                 FTLM_CUDA(launch_overlapped(overlap, up_vec == 4 ? lzp_update<VT, ST, 4> : lzp_update<VT, ST, 1>,
                                             (unsigned)up_runs, up_threads, 0, ss, U));
                 count_launch();
-                FTLM_CUDA(launch_overlapped(overlap, lzp_finalize, fin_grid, kFinThreads, 0, ss, 2, j, K, B, 0, d_ut.p,
-                                            d_ut.p + P, up_part.p, st, tol, kScaled));
+                FTLM_CUDA(launch_overlapped(overlap, lzp_finalize, fin_grid, kFinThreads, 0, ss, 2, j, K, B, fin.p + 2 * P,
+                                            up_part.p, st, tol, kScaled));
             }
             return FTLM_OK;
         };
@@ -837,7 +871,7 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets, int R, int n_ste
             for (int k = 0; k < K; ++k)
                 for (int b = 0; b < B; ++b) {
                     const size_t e = ((size_t)p * K + k) * B + b;
-                    const size_t o = ((size_t)p * K + k) * R + chain0 + b;
+                    const size_t o = ((size_t)orig[p] * K + k) * R + chain0 + b;
                     const int m = hs[e];
                     steps_done[o] = m;
                     for (int jj = 0; jj < m; ++jj) {

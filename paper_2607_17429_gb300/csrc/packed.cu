@@ -396,7 +396,8 @@ std::atomic<int> g_autotune{0};
 // round counts: one representative per warp; below that a part is spread over all CTAs (18
 // representatives of the s = 1/2 icosahedron, FP64, on one SM's FP64 pipe before: 118 us a call, 39 us
 // spread; 1.7e3 of the s = 1 cuboctahedron, on 17 CTAs before: 186 us, 55 us).  The one-thread kernel takes
-// whole warps.  A part's tiles depend on the part alone, so its partial sums are the same in any mix.
+// whole warps.  A part's tiles depend on the part alone (but for the autotuner's choice), so its partial
+// sums are the same in any mix.
 template <typename VT>
 void hvp_retile(HvpPlan<VT> &plan, std::vector<HvpPart<VT>> &parts) {
     uint64_t tiles = 0;

@@ -33,3 +33,17 @@ def test_more_tiles_than_ctas(name, two_s, Ms, irreps, R, dtype):
         F.ftlm_sector_build_entries(sec)
     sets = [F.ftlm_build_multiblock(sec, list(irreps)) for sec in secs]
     _mix_equals_alone(F, sets, getattr(F, dtype), R, 4)
+
+
+@pytest.mark.parametrize("entries", [None, 1])
+@pytest.mark.parametrize("dtype", ["F64", "F32", "F16"])
+def test_a_large_part_leaves_the_others_their_tables(dtype, entries):
+    """At four chains of dimension 3 the sector of 1.2e5 representatives has its flips searched once a call, those of
+    2.5e5 and 4.6e5 (64 MB and twice the vectors are less than their tables) search in every step; with an entry
+    table on one of them, too."""
+    F = ftlm()
+    g = product_group("icosidodecahedron")
+    secs = [F.ftlm_build_sector(g, 1, m) for m in (8, 12, 10)]
+    if entries is not None:
+        F.ftlm_sector_build_entries(secs[entries])
+    _mix_equals_alone(F, [F.ftlm_build_multiblock(sec, [2]) for sec in secs], getattr(F, dtype), 4, 4)
