@@ -395,7 +395,10 @@ ftlm_status ftlm_basis_rows(const ftlm_basis *b, int n, const uint64_t *labels, 
  * a representative) takes at most twice the block's vectors or 64 MB; a larger
  * one is not built, and every step searches.  With several sets the bound is
  * that of each set.  Device work memory (3 packed [rows][B] vectors, those
- * tables and reduction scratch) is allocated and freed by the call.  Synchronises cuda_stream before returning.
+ * tables, for one chain of a block in FP32 arithmetic a copy of the gathered
+ * vector with rows of up to 32 bytes, and reduction scratch) is allocated and
+ * freed by the call; where it does not fit, the call runs without the tables
+ * and the copy (equal to rounding).  Synchronises cuda_stream before returning.
  * FTLM_ETIMEOUT / FTLM_EINTERNAL report device-side failures of the H·v.
  */
 ftlm_status ftlm_lanczos(const ftlm_basis *b, ftlm_dtype dtype, int R, int n_steps, uint64_t seed,

@@ -468,9 +468,10 @@ struct LzHv {
     size_t row = 0;              // first row of its dot partials
 };
 
+// spare: in, whether the call may take memory that it can do without (flip tables, padded rows); out, whether it did
 template <typename VT, typename ST>
 ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets_in, int R, int n_steps, uint64_t seed, int rng,
-                              cudaStream_t stream, double *alpha, double *beta, int *steps_done) {
+                              cudaStream_t stream, double *alpha, double *beta, int *steps_done, bool &spare) {
     constexpr bool kScaled = sizeof(ST) < sizeof(VT);
     const int P = (int)sets_in.size();
     const PackedSet *ps0 = sets_in[0].ps;
@@ -501,7 +502,7 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets_in, int R, int n_
     {
         std::vector<size_t> by(P);
         size_t total = 0;
-        for (int i = 0; i < P; ++i)
+        for (int i = 0; i < P && spare; ++i)
             total += by[i] = lanczos_flip_bytes(sets_in[i].sec, sets_in[i].ps, Bmax, (int)sizeof(ST));
         if (total && flips.alloc(total, stream) != cudaSuccess) {
             cudaGetLastError();
@@ -518,6 +519,8 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets_in, int R, int n_
                 n_table += table;
             }
     }
+    const bool may_pad = spare;
+    spare = flips.p != nullptr;
     std::vector<uint64_t> row0(P + 1, 0);
     std::vector<int> m_max((size_t)P * K);
     for (int p = 0; p < P; ++p) {
@@ -596,7 +599,7 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets_in, int R, int n_
         hv[0].n = hv[1].p0 = n_table;
         hv[1].n = P - n_table;
         ScratchBuf<uint8_t> pad;  // padded rows of the vector an H·v gathers from (B = 1)
-        bool no_pad = false;
+        bool no_pad = !may_pad;
         size_t hv_rows = 0;  // rows of dot partials
         for (LzHv<VT> &h : hv) {
             if (h.n == 0) continue;
@@ -618,6 +621,7 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets_in, int R, int n_
                     cudaGetLastError();
                     no_pad = true;
                 }
+                spare = spare || pad.p;
                 if (pb && !no_pad) {  // the parts' rows follow one another in the vector
                     plan.a.pad_x = vb[q].p + row0[h.p0] * B;
                     plan.a.pad_out = pad.p;
@@ -883,14 +887,27 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets_in, int R, int n_
     return FTLM_OK;
 }
 
+// A call that runs out of memory with flip tables or padded rows runs again without them.
+template <typename VT, typename ST>
+ftlm_status lanczos_packed_any(const std::vector<LzSetIn> &sets, int R, int n_steps, uint64_t seed, int rng,
+                               cudaStream_t stream, double *alpha, double *beta, int *steps_done) {
+    bool spare = true;
+    ftlm_status st = lanczos_packed_st<VT, ST>(sets, R, n_steps, seed, rng, stream, alpha, beta, steps_done, spare);
+    if (st != FTLM_ENOMEM || !spare) return st;
+    cudaGetLastError();
+    scratch_trim();
+    spare = false;
+    return lanczos_packed_st<VT, ST>(sets, R, n_steps, seed, rng, stream, alpha, beta, steps_done, spare);
+}
+
 template <typename VT>
 ftlm_status lanczos_packed(const std::vector<LzSetIn> &sets, int R, int n_steps, uint64_t seed, int rng,
                            cudaStream_t stream, double *alpha, double *beta, int *steps_done, int esize) {
     if (esize == (int)sizeof(VT))
-        return lanczos_packed_st<VT, VT>(sets, R, n_steps, seed, rng, stream, alpha, beta, steps_done);
+        return lanczos_packed_any<VT, VT>(sets, R, n_steps, seed, rng, stream, alpha, beta, steps_done);
     if constexpr (sizeof(VT) == 4) {
         if (esize == 2)
-            return lanczos_packed_st<float, __half>(sets, R, n_steps, seed, rng, stream, alpha, beta, steps_done);
+            return lanczos_packed_any<float, __half>(sets, R, n_steps, seed, rng, stream, alpha, beta, steps_done);
     }
     return fail(FTLM_EINVAL, "no %d-byte storage for this arithmetic type", esize);
 }
