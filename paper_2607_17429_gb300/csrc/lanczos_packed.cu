@@ -503,7 +503,8 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets_in, int R, int n_
         std::vector<size_t> by(P);
         size_t total = 0;
         for (int i = 0; i < P && spare; ++i)
-            total += by[i] = lanczos_flip_bytes(sets_in[i].sec, sets_in[i].ps, Bmax, (int)sizeof(ST));
+            if (sets_in[i].spare)
+                total += by[i] = lanczos_flip_bytes(sets_in[i].sec, sets_in[i].ps, Bmax, (int)sizeof(ST));
         if (total && flips.alloc(total, stream) != cudaSuccess) {
             cudaGetLastError();
             by.assign(P, 0);
@@ -600,6 +601,7 @@ ftlm_status lanczos_packed_st(const std::vector<LzSetIn> &sets_in, int R, int n_
         hv[1].n = P - n_table;
         ScratchBuf<uint8_t> pad;  // padded rows of the vector an H·v gathers from (B = 1)
         bool no_pad = !may_pad;
+        for (int p = 0; p < n_table; ++p) no_pad = no_pad || !sets[p].spare;
         size_t hv_rows = 0;  // rows of dot partials
         for (LzHv<VT> &h : hv) {
             if (h.n == 0) continue;

@@ -15,6 +15,7 @@ struct LzSetIn {
     const ftlm_basis *const *blocks;
     const uint64_t *block_ids;
     int n_steps = 0;  // this set's step limit (0: the launch's n_steps; never above it)
+    bool spare = true;  // whether the call may take memory for this set that it can do without (flip table, padded rows)
 };
 
 // Bytes of the flip table a Lanczos call on the search path builds for one set and keeps for its

@@ -63,6 +63,7 @@ struct Job {
     double t_submit = 0, t_admit = -1, t_start = -1, t_done = -1;
     BlkEnt *be = nullptr;
     size_t vec_bytes = 0;
+    bool spare = true;  // charged for its flip table as well
     int d_gamma = 0;
     uint64_t dim = 0;
     std::vector<double> alpha, beta;  // [R][n_steps]
@@ -187,15 +188,20 @@ void fail_job(ftlm_server *S, Job *J, ftlm_status st, const std::string &msg) {
     S->cv_done.notify_all();
 }
 
-// Bytes a job's Lanczos launch allocates: three packed vectors, the flips it searches once for its
-// steps, the scale and coefficient state, and the per-CTA dot partials.
+size_t job_esize(const ftlm_job &j) { return j.dtype == FTLM_F64 ? 8 : (j.dtype == FTLM_F16 ? 2 : 4); }
+
+// Bytes a job's Lanczos launch cannot do without: three packed vectors, the scale and coefficient
+// state, and the per-CTA dot partials.
 size_t vector_bytes(const ftlm_basis *b, const ftlm_job &j) {
-    const size_t e = j.dtype == FTLM_F64 ? 8 : (j.dtype == FTLM_F16 ? 2 : 4);
     const size_t B = (size_t)std::min(j.R, kMaxB);
     const size_t rows = b->ps ? b->ps->rows : b->dim;
-    const size_t flips = b->ps ? lanczos_flip_bytes(b->sec, b->ps, (int)B, (int)e) : 0;
-    return 3 * std::max<size_t>(rows, 1) * B * e + flips + (2 * (size_t)j.n_steps + 16) * B * 8 + 4 * kNumSMs * B * 8 +
-           (1u << 20);
+    return 3 * std::max<size_t>(rows, 1) * B * job_esize(j) + (2 * (size_t)j.n_steps + 16) * B * 8 +
+           4 * kNumSMs * B * 8 + (1u << 20);
+}
+
+// Bytes it takes where there is room: the flips it searches once for its steps.
+size_t spare_bytes(const ftlm_basis *b, const ftlm_job &j) {
+    return b->ps ? lanczos_flip_bytes(b->sec, b->ps, std::min(j.R, kMaxB), (int)job_esize(j)) : 0;
 }
 
 // One step of admission for the head job.  Returns false when the scheduler
@@ -298,8 +304,11 @@ bool admit_head(ftlm_server *S, std::unique_lock<std::mutex> &lk, cudaStream_t b
     } else {
         ++S->st.block_hits;
     }
-    const size_t need = vector_bytes(be->blk, js);
-    if (!make_room(S, need)) {
+    const size_t spare = spare_bytes(be->blk, js);
+    size_t need = vector_bytes(be->blk, js);
+    J->spare = make_room(S, need + spare);  // else it runs without its flip table, as soon as its vectors fit
+    if (J->spare) need += spare;
+    if (!J->spare && !make_room(S, need)) {
         --be->refs;
         if (!idle()) return false;
         S->queue.pop_front();
@@ -369,7 +378,8 @@ void worker_main(ftlm_server *S) {
         std::vector<LzSetIn> sets(P);
         for (int p = 0; p < P; ++p) {
             blks[p] = wave[p]->be->blk;
-            sets[p] = LzSetIn{blks[p]->sec, blks[p]->ps, &blks[p], &wave[p]->spec.block_id, wave[p]->spec.n_steps};
+            sets[p] = LzSetIn{blks[p]->sec,      blks[p]->ps, &blks[p], &wave[p]->spec.block_id, wave[p]->spec.n_steps,
+                              wave[p]->spare};
             nmax = std::max(nmax, wave[p]->spec.n_steps);
         }
         std::vector<double> A((size_t)P * R * nmax), Bt((size_t)P * R * nmax);
