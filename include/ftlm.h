@@ -519,9 +519,10 @@ ftlm_status ftlm_thermo_noalloc(int n_chains, int ld, const int *m, const double
  *    (one per group, 2s, 2M; shared by every job on them), the resident
  *    block tables (one per sector and irrep) and each admitted job's Lanczos
  *    vectors and state (3 packed vectors of rows x min(R, 32) elements and a
- *    few MB) and, where it fits as well, the flip table of ftlm_lanczos; a job
- *    whose vectors fit and whose table does not is admitted without the table
- *    and searches in every step (equal to rounding).  A sector is estimated
+ *    few MB) and, where they fit as well, the flip table and the padded copy of
+ *    ftlm_lanczos; a job whose vectors fit and whose table does not is admitted
+ *    without it and searches in every step (equal to rounding).  Scratch of
+ *    the table builds, given back when they end, is not charged.  A sector is estimated
  *    from its dimension before it is built and charged its actual size after.  Tables that no admitted job references
  *    are evicted least recently used first when room is needed.  A job that
  *    does not fit even with nothing else admitted fails with FTLM_ENOMEM; a

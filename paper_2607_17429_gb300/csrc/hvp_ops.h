@@ -76,6 +76,8 @@ template <typename VT>
 size_t hvp_pad_bytes(const HvpPlan<VT> &plan, uint64_t n_rows) {
     return plan.a.B == 1 && n_rows >= (1u << 18) ? (size_t)n_rows * plan.ops->pad_bytes : 0;
 }
+// bytes of one padded row at B right-hand sides of esize bytes (0: the block has none)
+size_t hvp_pad_row_bytes(const ftlm_sector *s, const PackedSet *ps, int B, int esize);
 template <typename VT>
 ftlm_status hvp_launch_plan(const HvpPlan<VT> &plan, double *dot_part, cudaStream_t stream, bool timed);
 // the part as the build kernel sees it (no vectors, no blocks)

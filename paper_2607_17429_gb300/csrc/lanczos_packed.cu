@@ -455,6 +455,11 @@ size_t lanczos_flip_bytes(const ftlm_sector *sec, const PackedSet *ps, int B, in
     return bytes <= std::max<size_t>(64u << 20, 2 * vectors) ? (bytes + 255) / 256 * 256 : 0;
 }
 
+size_t lanczos_spare_bytes(const ftlm_sector *sec, const PackedSet *ps, int B, int esize) {
+    const size_t flips = lanczos_flip_bytes(sec, ps, B, esize);
+    return flips + (flips || sec->d_ent ? (size_t)sec->n_reps * hvp_pad_row_bytes(sec, ps, B, esize) : 0);
+}
+
 // A launch over the parts with flip tables and one over those without run in turn in every step: a large
 // sector that keeps searching leaves the others their tables (and their sums: the kernel of a part, and so its
 // bits, do not depend on what runs with it).  Five icosidodecahedron sectors at four chains of dimension 3,

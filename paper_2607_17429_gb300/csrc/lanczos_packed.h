@@ -22,6 +22,11 @@ struct LzSetIn {
 // steps; 0 when the sector has a table or the call does without one.
 size_t lanczos_flip_bytes(const ftlm_sector *sec, const PackedSet *ps, int B, int esize);
 
+// Bytes a Lanczos call takes for one set beside its vectors where there is room: that table, and the padded copy of
+// the rows it gathers from (one chain of a block in FP32 arithmetic; taken when the call's sets have 2^18
+// representatives or more together).
+size_t lanczos_spare_bytes(const ftlm_sector *sec, const PackedSet *ps, int B, int esize);
+
 // R chains on every block of every set, n_steps steps (Section 2.2).  alpha,
 // beta: host [n_sets][K][R][n_steps]; steps_done: host [n_sets][K][R].  All
 // sets share the group, spin, block shape and irreps.  esize: bytes of a stored

@@ -224,6 +224,23 @@ const HvpOps<double> *hvp_ops<double>(int shape, int gpl, bool half, int esize, 
     return shape <= kShapeD5 ? hvp_ops_single_f64(shape, gpl, half) : hvp_ops_multi_f64(shape, gpl, half);
 }
 
+// one thread per representative, table mode, single blocks (FP64: one right-hand side)
+template <typename VT>
+const HvpOps<VT> *hvp_lane_ops(int shape, bool half, int esize) {
+    if constexpr (sizeof(VT) == 8)
+        return shape_is_wide(shape) ? hvp_ops_wide_f64(shape, half, 2) : hvp_ops_lane_f64(shape);
+    else if (shape_is_wide(shape))
+        return esize == 2 ? hvp_ops_wide_f16(shape, half, 2) : hvp_ops_wide_f32(shape, half, 2);
+    else
+        return esize == 2 ? hvp_ops_lane_f16(shape) : hvp_ops_lane_f32(shape);
+}
+
+size_t hvp_pad_row_bytes(const ftlm_sector *s, const PackedSet *ps, int B, int esize) {
+    if (ps->K != 1 || ps->shape < 0 || B != 1 || esize == 8) return 0;
+    const HvpOps<float> *lane = hvp_lane_ops<float>(ps->shape, s->half, esize);
+    return lane ? (size_t)lane->pad_bytes : 0;
+}
+
 // Sector-wide part of the arguments (search tables, coefficients, irreps of the set).
 template <typename VT>
 void hvp_fill_common(const ftlm_sector *s, const PackedSet *ps, int B, int esize, HvpArgs<VT> &a) {
@@ -522,13 +539,7 @@ ftlm_status hvp_plan(const ftlm_sector *s, const PackedSet *ps, std::vector<HvpP
     if (mode == 1 && ps->K == 1 && (B == 1 || sizeof(VT) == 4)) {
         // one thread per representative: every B in FP32 arithmetic (2 to 9 times the warp kernel's
         // rate); FP64 operations bind either kernel, so FP64 keeps the warp kernel above B = 1
-        const HvpOps<VT> *lane = nullptr;
-        if constexpr (sizeof(VT) == 8)
-            lane = shape_is_wide(ps->shape) ? hvp_ops_wide_f64(ps->shape, s->half, 2) : hvp_ops_lane_f64(ps->shape);
-        else if (shape_is_wide(ps->shape))
-            lane = esize == 2 ? hvp_ops_wide_f16(ps->shape, s->half, 2) : hvp_ops_wide_f32(ps->shape, s->half, 2);
-        else
-            lane = esize == 2 ? hvp_ops_lane_f16(ps->shape) : hvp_ops_lane_f32(ps->shape);
+        const HvpOps<VT> *lane = hvp_lane_ops<VT>(ps->shape, s->half, esize);
         // its rho table lives in shared memory: keep the warp kernel when the table does not fit
         if (lane && lane->occupancy(a, lane->max_threads / 32, 1) > 0) plan.ops = lane;
     }

@@ -63,7 +63,7 @@ struct Job {
     double t_submit = 0, t_admit = -1, t_start = -1, t_done = -1;
     BlkEnt *be = nullptr;
     size_t vec_bytes = 0;
-    bool spare = true;  // charged for its flip table as well
+    bool spare = true;  // charged for its flip table and padded rows as well
     int d_gamma = 0;
     uint64_t dim = 0;
     std::vector<double> alpha, beta;  // [R][n_steps]
@@ -199,9 +199,9 @@ size_t vector_bytes(const ftlm_basis *b, const ftlm_job &j) {
            4 * kNumSMs * B * 8 + (1u << 20);
 }
 
-// Bytes it takes where there is room: the flips it searches once for its steps.
+// Bytes it takes where there is room: the flips it searches once for its steps, the padded copy of one chain's rows.
 size_t spare_bytes(const ftlm_basis *b, const ftlm_job &j) {
-    return b->ps ? lanczos_flip_bytes(b->sec, b->ps, std::min(j.R, kMaxB), (int)job_esize(j)) : 0;
+    return b->ps ? lanczos_spare_bytes(b->sec, b->ps, std::min(j.R, kMaxB), (int)job_esize(j)) : 0;
 }
 
 // One step of admission for the head job.  Returns false when the scheduler
