@@ -26,11 +26,17 @@ namespace ftlm {
 namespace {
 
 constexpr int kEnumThreads = 256;
+// Findings take half a byte per live label (two bits each, an offset per 32).  The second test costs up to
+// what it saved (36-site ring, 7.8e8 live labels: 136 ms a sector with findings, 252 without), so they are
+// kept where all the labels' counts over chunks of 256 would take as much (12 bytes each).
+constexpr bool enum_keeps(uint64_t live, uint64_t sector_dim) { return live <= (1ull << 29) || live <= sector_dim / 32 * 3; }
 
 // Labels are enumerated under the prefixes (digits of the top sites) that can still be an orbit
 // minimum.  A prefix is dead when some element maps the state to a smaller label whatever the other
 // digits are; the labels under live prefixes are ranked consecutively, in ascending order.  The count
-// pass keeps its findings as one bit per label, so the write pass tests nothing.  Icosidodecahedron,
+// pass keeps its findings as one bit per label, so the write pass tests nothing; where bits and offsets would
+// take more than 256 MB and more than 3/64 byte per label of the sector (enum_keeps: few dead prefixes, so
+// small groups), it keeps counts over longer chunks and the write pass tests again.  Icosidodecahedron,
 // M = 0 (1.55e8 labels, 1.3e6 representatives): 8.5 ms a sector with a test of every label in both passes,
 // 2.5 ms now; the dodecahedron's 1.65e9 labels at s = 3/2, M = 14: 59 ms, 13.5 ms.
 struct EnumArgs {
@@ -188,7 +194,9 @@ __device__ int rep_test(const EnumArgs &a, const uint8_t *src, uint64_t n, uint6
     return 1 + nontrivial;
 }
 
-// per thread: bit i of found[t].x for label r0 + i a representative, of found[t].y with a nontrivial stabilizer
+// per thread: KEEP: bit i of found[t].x for label r0 + i a representative, of found[t].y with a nontrivial
+// stabilizer; else found[t].x counts the representatives
+template <bool KEEP>
 __global__ void enum_count(EnumArgs a, uint2 *found, unsigned long long *n_nontrivial) {
     extern __shared__ uint8_t s_src[];
     for (int i = threadIdx.x; i < a.G * a.N; i += blockDim.x) s_src[i] = a.src[i];
@@ -202,17 +210,23 @@ __global__ void enum_count(EnumArgs a, uint2 *found, unsigned long long *n_nontr
         uint2 f = make_uint2(0u, 0u);
         for (uint64_t r = r0; r < r1; ++r) {
             const int k = rep_test(a, s_src, n, nullptr);
-            f.x |= (unsigned)(k > 0) << (r - r0);
-            f.y |= (unsigned)(k == 2) << (r - r0);
+            if constexpr (KEEP) {
+                f.x |= (unsigned)(k > 0) << (r - r0);
+                f.y |= (unsigned)(k == 2) << (r - r0);
+            } else {
+                f.x += k > 0;
+                nt += k == 2;
+            }
             if (r + 1 < r1) n = step_label(a, n, r + 1, p, end);
         }
         found[t] = f;
-        nt = __popc(f.y);
+        if (KEEP) nt = __popc(f.y);
     }
     for (int o = 16; o; o >>= 1) nt += __shfl_down_sync(kFull, nt, o);
     if ((threadIdx.x & 31) == 0 && nt) atomicAdd(n_nontrivial, (unsigned long long)nt);
 }
 
+template <bool KEEP>
 __global__ void enum_write(EnumArgs a, const uint2 *found, const uint64_t *offsets, uint64_t *labels,
                            unsigned long long *side_count, uint64_t *side, unsigned long long side_cap) {
     extern __shared__ uint8_t s_src[];
@@ -223,16 +237,17 @@ __global__ void enum_write(EnumArgs a, const uint2 *found, const uint64_t *offse
     const uint2 f = found[t];
     if (!f.x) return;
     uint64_t pos = offsets[t];
-    uint64_t r0 = t * a.chunk;
+    const uint64_t r0 = t * a.chunk, last = min(a.chunk, a.dim - r0) - 1;
     uint32_t p = prefix_of(a, r0);
     uint64_t n = unrank_under(a, p, r0 - a.first[p]), end = a.first[p + 1];
     uint64_t mask[4];
-    const int last = 31 - __clz((int)f.x);
-    for (int i = 0;; ++i) {
-        if ((f.x >> i) & 1u) {
+    unsigned left = KEEP ? __popc(f.x) : f.x;  // representatives of the chunk still to write
+    for (uint64_t i = 0;; ++i) {
+        const int k = KEEP ? (int)((f.x >> i) & 1u) + (int)((f.y >> i) & 1u) : rep_test(a, s_src, n, mask);
+        if (k) {
             labels[pos] = n;
-            if ((f.y >> i) & 1u) {
-                rep_test(a, s_src, n, mask);
+            if (k == 2) {
+                if (KEEP) rep_test(a, s_src, n, mask);
                 unsigned long long q = atomicAdd(side_count, 1ull);
                 if (q < side_cap) {
                     side[5 * q] = pos;
@@ -240,8 +255,9 @@ __global__ void enum_write(EnumArgs a, const uint2 *found, const uint64_t *offse
                 }
             }
             ++pos;
+            --left;
         }
-        if (i == last) break;
+        if (left == 0 || i == last) break;
         n = step_label(a, n, r0 + i + 1, p, end);
     }
 }
@@ -308,7 +324,8 @@ struct NGammaOf {
 
 struct CountsOf {
     const uint2 *found;
-    __device__ uint64_t operator()(uint64_t i) const { return (uint64_t)__popc(found[i].x); }
+    bool keep;
+    __device__ uint64_t operator()(uint64_t i) const { return keep ? (uint64_t)__popc(found[i].x) : found[i].x; }
 };
 
 int bits_for(int two_s) {
@@ -518,8 +535,11 @@ ftlm_status build_sector_impl(const GroupData &grp_in, int two_s, int two_M, int
         const uint64_t ends[2] = {0, s->sector_dim};
         FTLM_CUDA(cudaMemcpyAsync(first.p, ends, sizeof(ends), cudaMemcpyHostToDevice, stream));
     }
-    // labels per thread: few enough that every SM has its threads, at most the 32 bits of a thread's findings
-    ea.chunk = std::min<uint64_t>(32, std::max<uint64_t>(1, ea.dim / (kNumSMs * 4096ull)));
+    // labels per thread: few enough that every SM has its threads, at most the 32 bits of a thread's findings;
+    // without findings 256 or more, so that at most 2^24 threads' counts and offsets (256 MB) are held
+    const bool keep = enum_keeps(ea.dim, s->sector_dim);
+    ea.chunk = keep ? std::min<uint64_t>(32, std::max<uint64_t>(1, ea.dim / (kNumSMs * 4096ull)))
+                    : std::max<uint64_t>(256, (ea.dim >> 24) + 1);
     ea.n_threads = (ea.dim + ea.chunk - 1) / ea.chunk;
     const uint64_t n_blocks = (ea.n_threads + kEnumThreads - 1) / kEnumThreads;
     ScratchBuf<uint2> found;
@@ -530,11 +550,12 @@ ftlm_status build_sector_impl(const GroupData &grp_in, int two_s, int two_M, int
     FTLM_CUDA(nontriv.alloc(2, stream));
     FTLM_CUDA(cudaMemsetAsync(nontriv.p, 0, 2 * sizeof(unsigned long long), stream));
     count_launch();
-    enum_count<<<(unsigned)n_blocks, kEnumThreads, smem, stream>>>(ea, found.p, nontriv.p);
+    (keep ? enum_count<true> : enum_count<false>)<<<(unsigned)n_blocks, kEnumThreads, smem, stream>>>(ea, found.p,
+                                                                                                     nontriv.p);
     FTLM_CUDA(cudaGetLastError());
     uint64_t n_reps = 0;
     {
-        ftlm_status st = exclusive_scan(CountsOf{found.p}, ea.n_threads, offsets.p, stream, &n_reps);
+        ftlm_status st = exclusive_scan(CountsOf{found.p, keep}, ea.n_threads, offsets.p, stream, &n_reps);
         if (st != FTLM_OK) return st;
     }
     if (n_reps >= 0xffffffffull) return fail(FTLM_EUNSUPPORTED, "more than 2^32-1 representatives");
@@ -550,8 +571,8 @@ ftlm_status build_sector_impl(const GroupData &grp_in, int two_s, int two_M, int
     FTLM_CUDA(side.alloc(5 * n_side + 5, stream));
     FTLM_CUDA(cudaMemsetAsync(nontriv.p, 0, sizeof(unsigned long long), stream));
     count_launch();
-    enum_write<<<(unsigned)n_blocks, kEnumThreads, smem, stream>>>(ea, found.p, offsets.p, s->d_labels, nontriv.p, side.p,
-                                                                   n_side);
+    (keep ? enum_write<true> : enum_write<false>)<<<(unsigned)n_blocks, kEnumThreads, smem, stream>>>(
+        ea, found.p, offsets.p, s->d_labels, nontriv.p, side.p, n_side);
     FTLM_CUDA(cudaGetLastError());
     // stabilizer subgroups: dedupe masks on the host, ids ordered by mask
     std::vector<uint64_t> h_side(5 * n_side);
