@@ -336,7 +336,8 @@ void hvp_part_of(const ftlm_sector *s, const PackedSet *ps, const ftlm_basis *co
 // at that warp count, rho tables in shared memory before reading them through
 // L1 (FP32), the own-row prefetch before plain loads, and the most staging
 // buffers in flight (bulk-copy path, up to kMaxBuf).  FTLM_HV_WARPS,
-// FTLM_HV_NBUF, FTLM_HV_RHO (smem|l1) and FTLM_HV_OWN (0|1) override the choice.
+// FTLM_HV_NBUF, FTLM_HV_RHO (smem|l1) and FTLM_HV_OWN (0|1) override the choice
+// (but for the warps of the one-thread kernel, which has one size of CTA).
 template <typename VT>
 ftlm_status hvp_choose_geom(const HvpOps<VT> *ops, HvpArgs<VT> a, bool tma, HvpGeom &geo) {
     int dev = 0, sms = kNumSMs;
@@ -347,7 +348,7 @@ ftlm_status hvp_choose_geom(const HvpOps<VT> *ops, HvpArgs<VT> a, bool tma, HvpG
     const char *er = getenv("FTLM_HV_RHO");
     const char *eo = getenv("FTLM_HV_OWN");
     const int max_warps = ops->max_threads / 32;
-    const int want_warps = ew ? std::min(atoi(ew), max_warps) : 0;
+    const int want_warps = ew && !ops->tile_fixed ? std::min(atoi(ew), max_warps) : 0;
     const int want_nbuf = eb ? std::max(1, std::min(atoi(eb), kMaxBuf)) : 0;
     std::vector<int> rho_opts = sizeof(VT) == 4 ? std::vector<int>{1, 0} : std::vector<int>{0};
     if (er && sizeof(VT) == 4) rho_opts = {strcmp(er, "l1") == 0 ? 0 : 1};
