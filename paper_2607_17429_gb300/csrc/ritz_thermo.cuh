@@ -234,21 +234,22 @@ static __global__ void ground_energy(ThermoIn in, double *E0) {
 // memory, in rank order.  FP64 instructions bind, so one pass takes every moment: with x = theta - E0,
 // z = sum W e, sum W e x and sum W e x^2, and C = beta^2 (<x^2> - <x>^2); where that difference would
 // cancel more than six bits, a second pass takes the centred moment instead.  The exponential is
-// table-driven (Tang, ACM TOMS 15, 1989): e^{-beta x} = 2^{k / 256} 2^{r / 256} with the argument scaled by
-// 256 / ln 2 up front, so the reduction needs no split constant (the rounding of the scaled argument
-// is that of beta x), 16 FP64 operations per pair and temperature instead of about 60 in two passes.
+// table-driven (Tang, ACM TOMS 15, 1989): e^{-beta x} = 2^{k / 256} 2^{r / 256} with k the nearest integer to
+// -256 beta x / ln 2 and r the rest, -256 beta / ln 2 held as a sum of two doubles per temperature: r is exact
+// to its own rounding, so the result does not carry the rounding of beta x.  17 FP64 operations per pair and
+// temperature instead of about 60 in two passes.
 // 273,600 pairs and 200 temperatures: 7.3 ms with two passes of one CTA per temperature, 2.3 ms now.
 constexpr int kThermoCluster = 8;
 constexpr int kExpTab = 256;
 
-// 2^{y / 256} for -1024 * 256 < y <= 0 from tab[j] = 2^{j / 256}: y = 256 q + j + r, |r| <= 1/2, and the Taylor
-// polynomial of 2^{r / 256} - 1 to fourth order (its remainder is below 4e-17)
-static __device__ __forceinline__ double exp2_256(double y, const double *tab) {
+// 2^{x (s_hi + s_lo) / 256}, y = x s_hi rounded, -1100 * 256 < y <= 0, from tab[j] = 2^{j / 256}: the exponent is
+// 256 q + j + r, |r| <= 1/2, and 2^{r / 256} - 1 its Taylor polynomial to fourth order (its remainder is below 4e-17)
+static __device__ __forceinline__ double exp2_256(double x, double y, double s_hi, double s_lo, const double *tab) {
     constexpr double kShift = 6755399441055744.0;  // 1.5 * 2^52: adding it rounds to an integer
     constexpr double a = 0.0027076061740622863;    // ln 2 / 256
     const double s = y + kShift;
     const int k = __double2loint(s);
-    const double r = y - (s - kShift);
+    const double r = fma(x, s_lo, fma(x, s_hi, -(s - kShift)));
     const double p = fma(r, fma(r, fma(r, a * a * a * a / 24.0, a * a * a / 6.0), a * a / 2.0), a);
     const double t = tab[k & (kExpTab - 1)];
     const double v = fma(t, r * p, t);  // in [1, 2)
@@ -284,16 +285,17 @@ static __global__ void __cluster_dims__(kThermoCluster, 1, 1) __launch_bounds__(
     const double beta = 1.0 / T[it], E0 = *E0p;
     for (int i = threadIdx.x; i < kExpTab; i += blockDim.x) tab[i] = exp2(i * (1.0 / kExpTab));
     __syncthreads();
-    const double scale = -beta * (kExpTab / 0.69314718055994530942);
+    constexpr double c_hi = kExpTab / 0.69314718055994530942, c_lo = 5.2109500776783445e-15;  // 256 / ln 2
+    const double s_hi = -beta * c_hi, s_lo = fma(-beta, c_hi, -s_hi) - beta * c_lo;
     auto boltzmann = [&](unsigned c, size_t t, double &x) {  // W e^{-beta x}
         x = in.theta[t] - E0;
-        const double y = x * scale;
+        const double y = x * s_hi;
         const unsigned hi = (unsigned)__double2hiint(y);
         if (hi > 0xC1110000u || hi < 0x80000000u) {  // below -2^18 - 2^14, NaN, infinite or not negative
             if (hi < 0xFFF00000u && hi >= 0x80000000u) return 0.0;  // finite: e^{-beta x} rounds to 0
             return in.Wc[c] * in.w[t] * exp(-beta * x);
         }
-        return in.Wc[c] * in.w[t] * exp2_256(y, tab);
+        return in.Wc[c] * in.w[t] * exp2_256(x, y, s_hi, s_lo, tab);
     };
     // sums of v[0..3] over the cluster, valid in rank 0's thread 0
     auto cluster_sum = [&](double(&v)[4]) {
