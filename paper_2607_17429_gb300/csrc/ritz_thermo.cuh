@@ -231,14 +231,18 @@ static __global__ void ground_energy(ThermoIn in, double *E0) {
 }
 
 // One cluster of kThermoCluster CTAs per temperature; the CTAs' sums meet through distributed shared
-// memory, in rank order.  FP64 instructions bind, so one pass takes every moment: with x = theta - E0,
-// z = sum W e, sum W e x and sum W e x^2, and C = beta^2 (<x^2> - <x>^2); where that difference would
-// cancel more than six bits, a second pass takes the centred moment instead.  The exponential is
+// memory, in rank order.  FP64 instructions bind, so one pass takes every moment: with x = theta - c for a c near
+// the mean energy, z = sum W e, sum W e x and sum W e x^2, E = c + <x> and C = beta^2 (<x^2> - <x>^2).  c comes from a
+// pass in FP32; any c gives the moments, and where this one is so far off that the difference would cancel
+// more than a bit (energies far from zero beside their spread, values out of FP32's range), a second pass takes the
+// centred moment.  (Error of C in units of 2^-53, 1e4 normal levels, the lowest 7.5 spreads down, T from 0.4 to 300
+// spreads: up to 210 with c = E0 and six bits of cancellation allowed, 1.8 so, 2.3 with two centred FP64 passes.)
+// The exponential is
 // table-driven (Tang, ACM TOMS 15, 1989): e^{-beta x} = 2^{k / 256} 2^{r / 256} with k the nearest integer to
 // -256 beta x / ln 2 and r the rest, -256 beta / ln 2 held as a sum of two doubles per temperature: r is exact
 // to its own rounding, so the result does not carry the rounding of beta x.  17 FP64 operations per pair and
 // temperature instead of about 60 in two passes.
-// 273,600 pairs and 200 temperatures: 7.3 ms with two passes of one CTA per temperature, 2.3 ms now.
+// 273,600 pairs and 200 temperatures: 7.3 ms with two FP64 passes of one CTA per temperature, 2.9 ms now.
 constexpr int kThermoCluster = 8;
 constexpr int kExpTab = 256;
 
@@ -256,6 +260,16 @@ static __device__ __forceinline__ double exp2_256(double x, double y, double s_h
     const int q = k >> 8;
     if (q < -1021) return ldexp(v, q);
     return __hiloint2double(__double2hiint(v) + (q << 20), __double2loint(v));
+}
+
+// a double cut to float by its bits (a conversion instruction would occupy the FP64 pipe); 0 below FP32's range,
+// infinite or NaN above it
+static __device__ __forceinline__ float coarse(double v) {
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    const int e = (int)((hi >> 20) & 0x7ffu) - 1023 + 127;
+    const unsigned m = ((hi << 3) | (lo >> 29)) & 0x7fffffu;
+    const unsigned mag = e <= 0 ? 0u : e >= 255 ? 0x7f800000u | m : ((unsigned)e << 23) | m;
+    return __uint_as_float((hi & 0x80000000u) | mag);
 }
 
 // (chain, step) of this thread's pairs: a flat walk over [n_chains][ld] with the division done once
@@ -318,12 +332,28 @@ static __global__ void __cluster_dims__(kThermoCluster, 1, 1) __launch_bounds__(
                 for (int r = 0; r < kThermoCluster; ++r) v[q] += *cl.map_shared_rank(&part[q], r);
             }
     };
-    double v[4] = {0.0, 0.0, 0.0, 0.0};  // z, <x> z, <x^2> z, <M^2> z
+    const float e0f = coarse(E0), sf = -1.442695f * (float)beta;
+    float f0 = 0.f, f1 = 0.f;  // z and <theta - E0> z, to FP32's accuracy
     thermo_pairs(in, rank, [&](unsigned c, size_t t) {
-        double x;
-        const double b = boltzmann(c, t, x);
-        if (b == 0.0 && x < INFINITY) return;
-        const double bx = b * x;
+        const float x = coarse(in.theta[t]) - e0f;
+        const float b = coarse(in.Wc[c]) * coarse(in.w[t]) * exp2f(sf * x);
+        f0 += b;
+        f1 = fmaf(b, x, f1);
+    });
+    double v[4] = {(double)f0, (double)f1, 0.0, 0.0};
+    cluster_sum(v);
+    if (rank == 0 && threadIdx.x == 0) {
+        const double m = v[1] / v[0];
+        mid[0] = m > 0.0 && m < INFINITY ? E0 + m : E0;
+    }
+    cl.sync();
+    const double ec = *cl.map_shared_rank(&mid[0], 0);
+    v[0] = v[1] = v[2] = v[3] = 0.0;  // z, <x> z, <x^2> z, <M^2> z with x = theta - ec
+    thermo_pairs(in, rank, [&](unsigned c, size_t t) {
+        double x0;
+        const double b = boltzmann(c, t, x0);
+        if (b == 0.0 && x0 < INFINITY) return;
+        const double x = in.theta[t] - ec, bx = b * x;
         v[0] += b;
         v[1] += bx;
         v[2] = fma(bx, x, v[2]);
@@ -333,8 +363,8 @@ static __global__ void __cluster_dims__(kThermoCluster, 1, 1) __launch_bounds__(
     const double z = v[0], xm = v[1] / v[0], zm = v[3];
     double var = v[2] / v[0] - xm * xm;
     if (rank == 0 && threadIdx.x == 0) {
-        mid[0] = xm;
-        mid[1] = var * 64.0 < xm * xm ? 1.0 : 0.0;
+        mid[0] = ec + xm;
+        mid[1] = var < xm * xm ? 1.0 : 0.0;
     }
     cl.sync();
     const double xc = *cl.map_shared_rank(&mid[0], 0);
@@ -342,17 +372,18 @@ static __global__ void __cluster_dims__(kThermoCluster, 1, 1) __launch_bounds__(
     if (again) {
         double u[4] = {0.0, 0.0, 0.0, 0.0};
         thermo_pairs(in, rank, [&](unsigned c, size_t t) {
-            double x;
-            const double b = boltzmann(c, t, x);
-            if (b == 0.0 && x < INFINITY) return;
-            u[0] = fma(b * (x - xc), x - xc, u[0]);
+            double x0;
+            const double b = boltzmann(c, t, x0);
+            if (b == 0.0 && x0 < INFINITY) return;
+            const double x = in.theta[t] - xc;
+            u[0] = fma(b * x, x, u[0]);
         });
         cluster_sum(u);
         var = u[0] / z;
     }
     if (rank == 0 && threadIdx.x == 0) {
         out[it] = log(z) - beta * E0;
-        out[n_T + it] = E0 + xm;
+        out[n_T + it] = ec + xm;
         out[2 * n_T + it] = beta * beta * var;
         out[3 * n_T + it] = g * g * beta * zm / z;
     }
