@@ -10,8 +10,11 @@
 //    rows share a wavefront (a 16-byte shared load costs two wavefronts for up to sixteen addresses
 //    when lane pairs agree, an 8-byte load one);
 //  - rho(g) of all blocks is one record (stride 4 mod 8 words: records start in different banks), so a
-//    flip needs one base address; the coefficient multiplies the gathered values, so products go
-//    straight into the accumulators, pairs of rows through fma.rn.f32x2;
+//    flip needs one base address; pairs of rows go through fma.rn.f32x2.  A flip's products are summed before
+//    they meet the accumulators, which keeps the rounding of the kernel of hvp.cuh; but where 64 accumulators fill
+//    the registers (W = 32) blocks of dimension 1 to 3 scale the gathered values and add every product to them
+//    (icosidodecahedron at B = 8: error 6.6e-8 in hvp.cuh, 6.9e-8 with every product added in 5.86 ms, 6.4e-8 so in
+//    5.78, 6.2e-8 with every block's sums first in 6.41);
 //  - entries stay in registers (lane j holds flips j and 32 + j) and reach the others by shuffles;
 //  - the record, the entry offsets and the entries of the next representative are loaded while the
 //    present one is worked on, and its first gathers are issued as soon as the last of this one's are,
@@ -92,6 +95,14 @@ __device__ __forceinline__ float2 flow_load2(const ST *p) {
         return __half22float2(*reinterpret_cast<const __half2 *>(p));
     else
         return *reinterpret_cast<const float2 *>(p);
+}
+
+// pair q of rows of both columns: a rho pair times the gathered row
+template <int N>
+__device__ __forceinline__ void flow_acc(unsigned long long (&ap)[2][N], int q, bool first, unsigned long long rr, float2 xv) {
+    const unsigned long long u0 = f2_pack(xv.x, xv.x), u1 = f2_pack(xv.y, xv.y);
+    ap[0][q] = first ? f2_mul(rr, u0) : f2_fma(rr, u0, ap[0][q]);
+    ap[1][q] = first ? f2_mul(rr, u1) : f2_fma(rr, u1, ap[1][q]);
 }
 
 // N rows per column held by every lane -> N / 2 after the exchange with the lane M groups of CL away
@@ -374,37 +385,58 @@ __global__ void __launch_bounds__(flow_threads<ST, SH, CL>(), 1) hvp_flow_kernel
                             const float4 v = *reinterpret_cast<const float4 *>(Rk + 20);
                             odd5[0] = v.x, odd5[1] = v.y, odd5[2] = v.z, odd5[3] = v.w, odd5[4] = Rk[24];
                         }
+                        if constexpr (D >= 4 || W <= 20) {  // the flip's sums first (first product a multiply), one addition to z
+                            unsigned long long ap[2][D >= 2 ? D / 2 : 1];
+                            float as[2];
 #pragma unroll
-                        for (int ga = 0; ga < D; ++ga) {
-                            const float2 xv = flow_load2<ST>(xs + (Zk + ga) * B);
-                            const float u0 = xv.x * ck, u1 = xv.y * ck;
-                            if constexpr (D == 1) {
-                                zs[0][SB] = fmaf(Rk[0], u0, zs[0][SB]);
-                                zs[1][SB] = fmaf(Rk[0], u1, zs[1][SB]);
-                            } else {
-                                const unsigned long long uu0 = f2_pack(u0, u0), uu1 = f2_pack(u1, u1);
+                            for (int ga = 0; ga < D; ++ga) {
+                                const float2 xv = flow_load2<ST>(xs + (Zk + ga) * B);
+                                float ro = Rk[0];  // rho of the odd row
                                 if constexpr (D == 2) {
-                                    const unsigned long long rr = *reinterpret_cast<const unsigned long long *>(Rk + 2 * ga);
+                                    flow_acc(ap, 0, ga == 0, *reinterpret_cast<const unsigned long long *>(Rk + 2 * ga), xv);
+                                } else if constexpr (D > 2) {
+                                    const ulonglong2 rr = *reinterpret_cast<const ulonglong2 *>(Rk + 4 * ga);
+                                    flow_acc(ap, 0, ga == 0, rr.x, xv);
+                                    if constexpr (D >= 4) flow_acc(ap, 1, ga == 0, rr.y, xv);
+                                    float pad;
+                                    if constexpr (D == 3) f2_unpack(rr.y, ro, pad);
+                                    if constexpr (D == 5) ro = odd5[ga];
+                                }
+                                if constexpr (D % 2) {
+                                    as[0] = ga == 0 ? ro * xv.x : fmaf(ro, xv.x, as[0]);
+                                    as[1] = ga == 0 ? ro * xv.y : fmaf(ro, xv.y, as[1]);
+                                }
+                            }
+                            const unsigned long long cc = f2_pack(ck, ck);
+#pragma unroll
+                            for (int c = 0; c < 2; ++c) {
+#pragma unroll
+                                for (int q = 0; q < D / 2; ++q) zp[c][PB + q] = f2_fma(cc, ap[c][q], zp[c][PB + q]);
+                                if constexpr (D % 2) zs[c][SB] = fmaf(ck, as[c], zs[c][SB]);
+                            }
+                        } else {  // every product straight into z
+#pragma unroll
+                            for (int ga = 0; ga < D; ++ga) {
+                                const float2 xv = flow_load2<ST>(xs + (Zk + ga) * B);
+                                const float u0 = xv.x * ck, u1 = xv.y * ck;
+                                float ro = Rk[0];
+                                if constexpr (D > 1) {
+                                    const unsigned long long uu0 = f2_pack(u0, u0), uu1 = f2_pack(u1, u1);
+                                    unsigned long long rr;
+                                    if constexpr (D == 2) {
+                                        rr = *reinterpret_cast<const unsigned long long *>(Rk + 2 * ga);
+                                    } else {
+                                        const ulonglong2 r4 = *reinterpret_cast<const ulonglong2 *>(Rk + 4 * ga);
+                                        float pad;
+                                        rr = r4.x;
+                                        f2_unpack(r4.y, ro, pad);
+                                    }
                                     zp[0][PB] = f2_fma(rr, uu0, zp[0][PB]);
                                     zp[1][PB] = f2_fma(rr, uu1, zp[1][PB]);
-                                } else {
-                                    const ulonglong2 rr = *reinterpret_cast<const ulonglong2 *>(Rk + 4 * ga);
-                                    zp[0][PB] = f2_fma(rr.x, uu0, zp[0][PB]);
-                                    zp[1][PB] = f2_fma(rr.x, uu1, zp[1][PB]);
-                                    if constexpr (D >= 4) {
-                                        zp[0][PB + 1] = f2_fma(rr.y, uu0, zp[0][PB + 1]);
-                                        zp[1][PB + 1] = f2_fma(rr.y, uu1, zp[1][PB + 1]);
-                                    }
-                                    if constexpr (D == 3) {
-                                        float r2, pad;
-                                        f2_unpack(rr.y, r2, pad);
-                                        zs[0][SB] = fmaf(r2, u0, zs[0][SB]);
-                                        zs[1][SB] = fmaf(r2, u1, zs[1][SB]);
-                                    }
-                                    if constexpr (D == 5) {
-                                        zs[0][SB] = fmaf(odd5[ga], u0, zs[0][SB]);
-                                        zs[1][SB] = fmaf(odd5[ga], u1, zs[1][SB]);
-                                    }
+                                }
+                                if constexpr (D % 2) {
+                                    zs[0][SB] = fmaf(ro, u0, zs[0][SB]);
+                                    zs[1][SB] = fmaf(ro, u1, zs[1][SB]);
                                 }
                             }
                         }
