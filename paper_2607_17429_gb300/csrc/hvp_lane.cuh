@@ -4,8 +4,8 @@
 // each representative is a chain of dependent memory round trips (record, entry offsets, entries,
 // gathers).  Here every thread walks its own representative's entries, so a warp keeps 32 / (B / CV) such
 // chains in flight.  CV is 1 for B = 1 and odd B, else 2 or 4 neighbouring right-hand sides, one vector
-// load per row.  The contributions are summed in entry order (the warp kernels sum them per flip
-// group and then across groups), so results agree with theirs to rounding.
+// load per row.  The contributions are summed in entry order, a few apart at a time (the warp
+// kernels sum them per flip group and then across groups), so results agree with theirs to rounding.
 //
 // Blocks of dimension 1, 3, 4, 5 of the icosidodecahedron at M = 0, FP32, from the table: B = 1 0.19 to 0.43 ms;
 // B = 8 2.6 to 3.1 ms with a warp per representative, 0.29 to 1.25 ms here; B = 32 7.2 to 9.1 ms, 0.9 to 4.4 ms.
@@ -20,8 +20,21 @@ namespace ftlm {
 constexpr int kLaneThreads = 256;
 // flips whose entries and rows are loaded before the first is summed
 __host__ __device__ constexpr int lane_flips(int D, int CV) { return D * CV <= 4 ? 4 : D * CV <= 16 ? 2 : 1; }
-// right-hand sides per thread and threads per representative
-inline int lane_cols(int B) { return B % 4 == 0 ? 4 : B % 2 == 0 ? 2 : 1; }
+// Flips summed apart before they meet the rest.  FP32 vectors: four, since one chain over all flips carries up to
+// 1.6 times the error of a warp's short sums (icosidodecahedron, d = 5, B = 8: 6.7e-8 with a warp per representative,
+// 9.4e-8 in one chain, 6.9e-8 in fours; B = 24 9.4, 9.4 and 6.9e-8; complete graph of 11 sites, d = 10, 14.1 and 9.5e-8).
+// FP16 vectors round each output to 2^-11 and FP64 operations bind: as many as are loaded at a time.
+template <typename ST, int FL>
+__host__ __device__ constexpr int lane_sum() {
+    return sizeof(ST) == 4 ? 4 : FL;
+}
+// right-hand sides per thread, at most `most`: the sums and accumulators of FP32 vectors fill the registers with four
+// columns from dimension 5 on (d = 5, B = 8: 1.66 ms with four columns, 1.29 with two)
+inline int lane_cols(int B, int most) { return B % 4 == 0 && most == 4 ? 4 : B % 2 == 0 ? 2 : 1; }
+template <typename VT, typename ST, int D>
+constexpr int lane_most_cols() {
+    return sizeof(VT) == 8 ? 1 : D <= 4 || sizeof(ST) == 2 ? 4 : 2;
+}
 
 __host__ __device__ constexpr int lane_gcd(int a, int b) { return b == 0 ? a : lane_gcd(b, a % b); }
 
@@ -82,7 +95,7 @@ __device__ __forceinline__ void lane_row(const ST *__restrict__ x, uint64_t r, u
 
 // Rows whose size is no power of two straddle sectors: a copy of x with rows padded to the next one (PB bytes, 32
 // at most) is made before the launch, and a row then is one aligned load (256 bits for PB = 32) and one
-// sector (s = 3/2 dodecahedron, M = 14, d = 5: 3.84 -> 3.56 ms in FP32, 3.71 -> 3.1 in FP16; what remains is the
+// sector (s = 3/2 dodecahedron, M = 14, d = 5: 3.84 -> 3.66 ms in FP32, 3.71 -> 3.1 in FP16; what remains is the
 // rate of random sectors, 1.1e11 a second here).  0: the rows are aligned already or too long, or FP64,
 // whose operations bind.
 template <typename ST, int D>
@@ -178,7 +191,7 @@ __device__ __forceinline__ void lane_cols_load(const ST *__restrict__ x, size_t 
 // ONE: a single right-hand side (rows of D consecutive elements); PB: bytes of the padded copy's rows, 0 for none
 template <typename VT, typename ST, int D, int CV, bool ONE, int PB>
 __global__ void __launch_bounds__(kLaneThreads) hvp_lane_kernel(const __grid_constant__ HvpArgs<VT> a) {
-    constexpr int RP = rho_row(D), FL = ONE ? 2 : lane_flips(D, CV);
+    constexpr int RP = rho_row(D), FL = ONE ? 2 : lane_flips(D, CV), SUM = lane_sum<ST, FL>();
     extern __shared__ __align__(128) uint8_t smem[];
     VT *s_rho = reinterpret_cast<VT *>(smem);  // rho(g) of the block, [G][D][RP]
     uint8_t *s_bond = smem + (((size_t)a.rho_total * sizeof(VT) + 15) & ~(size_t)15);
@@ -302,7 +315,7 @@ __global__ void __launch_bounds__(kLaneThreads) hvp_lane_kernel(const __grid_con
                 for (int g = 0; g < D; ++g) lane_cols_load<VT, ST, CV>(x, (r * D + g) * B + col, vec, u[g]);
             }
         };
-        // s = cf rho(g*)^T u of the first flip of a group, plus that of the others
+        // cf rho(g*)^T u, the first of a sum or added to it
         auto contract = [&](uint2 raw, VT cf, const VT(&u)[D][CV], VT(&s)[D][CV], bool first) {
             const VT *R = s_rho + (size_t)(raw.y & 127u) * D * RP;
             VT acc[D][CV];
@@ -320,43 +333,47 @@ __global__ void __launch_bounds__(kLaneThreads) hvp_lane_kernel(const __grid_con
 #pragma unroll
                 for (int v = 0; v < CV; ++v) s[be][v] = first ? cf * acc[be][v] : s[be][v] + cf * acc[be][v];
         };
+        // FP32 vectors: SUM flips (or the last few) are summed in s, then added to z; FP16 vectors: those of a step;
+        // FP64, whose operations bind, adds to z at once
+        constexpr bool kApart = sizeof(ST) == 4, kStep = sizeof(ST) == 2;
+        VT s[D][CV];
+        VT(&sum)[D][CV] = kApart || kStep ? s : z;
+        auto add_sum = [&]() {
+#pragma unroll
+            for (int g = 0; g < D; ++g)
+#pragma unroll
+                for (int v = 0; v < CV; ++v) {
+                    z[g][v] += s[g][v];
+                    s[g][v] = (VT)0;
+                }
+        };
+#pragma unroll
+        for (int g = 0; g < D; ++g)
+#pragma unroll
+            for (int v = 0; v < CV; ++v) s[g][v] = (VT)0;
         const uint2 *ent = reinterpret_cast<const uint2 *>(P.ent);
         uint64_t e = e0;
-        for (; e + FL <= e1; e += FL) {  // FL gathers in flight per thread, one addition to z for them all
-            uint2 r[FL];
-            VT u[FL][D][CV], s[D][CV];
+        auto step = [&](auto N) {  // N gathers in flight
+            constexpr int n = decltype(N)::value;
+            uint2 r[n];
+            VT u[n][D][CV];
 #pragma unroll
-            for (int q = 0; q < FL; ++q) r[q] = __ldg(ent + e + q);
+            for (int q = 0; q < n; ++q) r[q] = __ldg(ent + e + q);
 #pragma unroll
-            for (int q = 0; q < FL; ++q) gather(r[q].x, u[q]);
+            for (int q = 0; q < n; ++q) gather(r[q].x, u[q]);
 #pragma unroll
-            for (int q = 0; q < FL; ++q) {
-                if constexpr (sizeof(VT) == 8)  // FP64 operations bind: none for the group's sum
-                    contract(r[q], coef(r[q]), u[q], z, false);
-                else
-                    contract(r[q], coef(r[q]), u[q], s, q == 0);
-            }
-            if constexpr (sizeof(VT) == 4) {
+            for (int q = 0; q < n; ++q) contract(r[q], coef(r[q]), u[q], sum, kStep && q == 0);
+            if (kStep) add_sum();
+            e += n;
+        };
+        while (e + SUM <= e1) {
 #pragma unroll
-                for (int g = 0; g < D; ++g)
-#pragma unroll
-                    for (int v = 0; v < CV; ++v) z[g][v] += s[g][v];
-            }
+            for (int h = 0; h < SUM; h += FL) step(std::integral_constant<int, FL>{});
+            if (kApart) add_sum();
         }
-        for (; e < e1; ++e) {
-            const uint2 r0 = __ldg(ent + e);
-            VT u0[D][CV], s[D][CV];
-            gather(r0.x, u0);
-            if constexpr (sizeof(VT) == 8) {
-                contract(r0, coef(r0), u0, z, false);
-            } else {
-                contract(r0, coef(r0), u0, s, true);
-#pragma unroll
-                for (int g = 0; g < D; ++g)
-#pragma unroll
-                    for (int v = 0; v < CV; ++v) z[g][v] += s[g][v];
-            }
-        }
+        if (FL == 2 && SUM == 4 && e + 2 <= e1) step(std::integral_constant<int, 2>{});
+        while (e < e1) step(std::integral_constant<int, 1>{});
+        if (kApart) add_sum();
         VT xo[D][CV];
         gather(at, xo);
 #pragma unroll
@@ -414,9 +431,12 @@ auto lane_dispatch(const HvpArgs<VT> &a, F f) {
     using std::true_type;
     constexpr int PB = lane_pad_bytes<ST, D>();
     if constexpr (sizeof(VT) == 4) {
-        if (a.B > 1 && lane_cols(a.B) == 4)
-            return f(std::integral_constant<int, 4>{}, false_type{}, std::integral_constant<int, 0>{});
-        if (a.B > 1 && lane_cols(a.B) == 2)
+        constexpr int most = lane_most_cols<VT, ST, D>();
+        const int cols = lane_cols(a.B, most);
+        if constexpr (most == 4)
+            if (a.B > 1 && cols == 4)
+                return f(std::integral_constant<int, 4>{}, false_type{}, std::integral_constant<int, 0>{});
+        if (a.B > 1 && cols == 2)
             return f(std::integral_constant<int, 2>{}, false_type{}, std::integral_constant<int, 0>{});
         if (a.B > 1) return f(std::integral_constant<int, 1>{}, false_type{}, std::integral_constant<int, 0>{});
     }

@@ -371,7 +371,7 @@ ftlm_status hvp_choose_geom(const HvpOps<VT> *ops, HvpArgs<VT> a, bool tma, HvpG
                     geo.tma = tma ? 1 : 0;
                     geo.rho_smem = rho;
                     geo.own = own;
-                    geo.tile_reps = ops->tile_fixed ? ops->tile_fixed / (a.B / lane_cols(a.B)) : warps * 4;
+                    geo.tile_reps = ops->tile_fixed ? ops->tile_fixed / (a.B / lane_cols(a.B, ops->most_cols)) : warps * 4;
                     geo.grid = sms * per_sm;
                     return FTLM_OK;
                 }
