@@ -5,11 +5,11 @@ namespace ftlm {
 
 const HvpOps<float> *hvp_ops_flow_ih_f16(int B) {
     using T = __half;
-    static const HvpOps<float> tab[5] = {FTLM_HVP_FLOW_OPS(T, ShapeIh, 4, 8), FTLM_HVP_FLOW_OPS(T, ShapeIh, 4, 0),
-                                         FTLM_HVP_FLOW_OPS(T, ShapeIh, 8, 0), FTLM_HVP_FLOW_OPS(T, ShapeIh, 16, 24),
+    static const HvpOps<float> fixed[4] = {FTLM_HVP_FLOW_OPS(T, ShapeIh, 4, 8), FTLM_HVP_FLOW_OPS(T, ShapeIh, 8, 16),
+                                           FTLM_HVP_FLOW_OPS(T, ShapeIh, 16, 24), FTLM_HVP_FLOW_OPS(T, ShapeIh, 16, 32)};
+    static const HvpOps<float> any[3] = {FTLM_HVP_FLOW_OPS(T, ShapeIh, 4, 0), FTLM_HVP_FLOW_OPS(T, ShapeIh, 8, 0),
                                          FTLM_HVP_FLOW_OPS(T, ShapeIh, 16, 0)};
-    if (B < 6 || B > 32 || B % 2) return nullptr;
-    return &tab[B == 8 ? 0 : B < 8 ? 1 : B <= 16 ? 2 : B == 24 ? 3 : 4];
+    return flow_pick(B, fixed, any);
 }
 
 }  // namespace ftlm

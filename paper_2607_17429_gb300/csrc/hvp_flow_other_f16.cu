@@ -5,11 +5,13 @@ namespace ftlm {
 
 const HvpOps<float> *hvp_ops_flow_other_f16(int shape, int B) {
     using T = __half;
-    static const HvpOps<float> tab[2][3] = {
-        {FTLM_HVP_FLOW_OPS(T, ShapeOh, 4, 0), FTLM_HVP_FLOW_OPS(T, ShapeOh, 8, 0), FTLM_HVP_FLOW_OPS(T, ShapeOh, 16, 0)},
-        {FTLM_HVP_FLOW_OPS(T, ShapeTd, 4, 0), FTLM_HVP_FLOW_OPS(T, ShapeTd, 8, 0), FTLM_HVP_FLOW_OPS(T, ShapeTd, 16, 0)}};
-    if ((shape != kShapeOh && shape != kShapeTd) || B < 6 || B > 32 || B % 2) return nullptr;
-    return &tab[shape == kShapeTd][B <= 8 ? 0 : B <= 16 ? 1 : 2];
+    static const HvpOps<float> oh_fixed[4] = {FTLM_HVP_FLOW_OPS(T, ShapeOh, 4, 8), FTLM_HVP_FLOW_OPS(T, ShapeOh, 8, 16),
+                                              FTLM_HVP_FLOW_OPS(T, ShapeOh, 16, 24), FTLM_HVP_FLOW_OPS(T, ShapeOh, 16, 32)};
+    static const HvpOps<float> oh_any[3] = {FTLM_HVP_FLOW_OPS(T, ShapeOh, 4, 0), FTLM_HVP_FLOW_OPS(T, ShapeOh, 8, 0),
+                                            FTLM_HVP_FLOW_OPS(T, ShapeOh, 16, 0)};
+    static const HvpOps<float> td_any[3] = {FTLM_HVP_FLOW_OPS(T, ShapeTd, 4, 0), FTLM_HVP_FLOW_OPS(T, ShapeTd, 8, 0),
+                                            FTLM_HVP_FLOW_OPS(T, ShapeTd, 16, 0)};
+    return shape == kShapeOh ? flow_pick(B, oh_fixed, oh_any) : shape == kShapeTd ? flow_pick(B, nullptr, td_any) : nullptr;
 }
 
 }  // namespace ftlm

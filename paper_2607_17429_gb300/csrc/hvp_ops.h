@@ -135,6 +135,14 @@ const HvpOps<float> *hvp_ops_table_f32(int shape);
 const HvpOps<float> *hvp_ops_table_f16(int shape);
 // table mode of the multi-block shapes for an even B in 6..32 (hvp_flow.cuh): lanes per flip and the ops
 constexpr int flow_lanes(int B) { return B <= 8 ? 4 : B <= 16 ? 8 : 16; }
+// Multiples of eight, whose rows are whole 32-byte sectors in FP32, have B as a compile-time constant (row strides as
+// immediates).  FP32, ms a call without and with: ten icosidodecahedron irreps, B = 8 6.34, 5.79; 16 10.41, 9.91; 24
+// 17.6, 16.9; s = 1 dodecahedron, M = 8, B = 32 3.37, 3.27; s = 2 cuboctahedron, M = 0, 8 1.29, 1.27; 16 2.02, 1.98; 24
+// 3.93, 3.70; 32 3.97, 3.73.  T_d's sectors are too small to show it.
+inline const HvpOps<float> *flow_pick(int B, const HvpOps<float> *fixed, const HvpOps<float> *any) {
+    if (B < 6 || B > 32 || B % 2) return nullptr;
+    return fixed && B % 8 == 0 ? &fixed[B / 8 - 1] : &any[B <= 8 ? 0 : B <= 16 ? 1 : 2];
+}
 const HvpOps<float> *hvp_ops_flow_ih_f32(int B);
 const HvpOps<float> *hvp_ops_flow_ih_f16(int B);
 const HvpOps<float> *hvp_ops_flow_other_f32(int shape, int B);
