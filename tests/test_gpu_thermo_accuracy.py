@@ -1,4 +1,5 @@
-"""The exponential of the thermal sums against quadruple precision over its whole range."""
+"""Accuracy of the thermal pipeline against quadruple precision: the exponential over its range, the moments about the mean,
+and the rotation of the eigensolve."""
 from __future__ import annotations
 
 import numpy as np
@@ -64,3 +65,29 @@ def test_moments(n, low, scale, shift):
     assert np.all(np.abs(E - (LD(th.min()) + m)) <= 16 * U * (np.abs(th.min() + m) + np.sqrt(var)))
     assert np.all(np.abs(C / (b * b * var) - 1) <= 16 * U), (np.abs(C / (b * b * var) - 1) / U).astype(float)
     assert np.all(np.abs(chi / (b * (z * msq).sum(1) / Z) - 1) <= 16 * U)
+
+
+@needs_quad
+@pytest.mark.parametrize("scale", [1.0, 1e-140, 3e140])
+def test_rotation_of_two_steps(scale):
+    """Chains of two steps take one rotation (a second sweep only to find the off-diagonal negligible): its 1 / sqrt
+    comes from the hardware's approximation and one step of a third-order iteration.  Shift, rotation and squares
+    add up to at most 32 units of 2^-53 in the weights where the levels are no closer than a tenth of the matrix."""
+    F = ftlm()
+    rng = np.random.default_rng(2)
+    n = 20000
+    a = rng.normal(size=(n, 2))
+    b = np.stack([10.0 ** rng.uniform(-6, 2, n) * rng.choice([-1.0, 1.0], n), np.zeros(n)], 1)
+    half = (a[:, 1] - a[:, 0]) / 2
+    keep = np.hypot(half, b[:, 0]) >= 0.05 * np.maximum(np.abs(a).max(1), np.abs(b[:, 0]))
+    a, b = a[keep] * scale, b[keep] * scale
+    th, w = F.ftlm_ritz(a, b, np.full(len(a), 2, dtype=np.int32))
+    al, bl = a.astype(LD), b.astype(LD)[:, 0]
+    h, mid = (al[:, 1] - al[:, 0]) / 2, (al[:, 1] + al[:, 0]) / 2
+    r = np.sqrt((h / scale) ** 2 + (bl / scale) ** 2) * LD(scale)
+    norm = np.abs(mid) + r
+    assert np.all(np.abs(th[:, 0] - (mid - r)) <= 16 * U * norm) and np.all(np.abs(th[:, 1] - (mid + r)) <= 16 * U * norm)
+    w0 = (1 + h / r) / 2  # weight of the lower level: cos^2, from the side that does not cancel
+    w0 = np.where(h >= 0, w0, (bl / r) ** 2 / (2 * (1 - h / r)))
+    w1 = np.where(h >= 0, (bl / r) ** 2 / (2 * (1 + h / r)), (1 - h / r) / 2)
+    assert np.all(np.abs(w[:, 0] - w0) <= 32 * U) and np.all(np.abs(w[:, 1] - w1) <= 32 * U)
