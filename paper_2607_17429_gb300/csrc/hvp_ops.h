@@ -29,6 +29,7 @@ struct HvpOps {
     int (*occupancy)(const HvpArgs<VT> &, int warps, int nbuf);
     ftlm_status (*launch)(HvpArgs<VT>, const HvpGeom &, cudaStream_t);
     int max_threads;
+    int options;     // 1: rho tables in shared memory or read through L1, own rows prefetched or not (else fixed)
     int tile_fixed;  // one thread per representative: the CTA's threads, the most a tile takes (0: warp kernels)
     int most_cols;   // one thread per representative: right-hand sides per thread, at most
     int pad_bytes;   // one thread per representative, B = 1: bytes of a padded row (0: rows stay as they are)
@@ -37,18 +38,18 @@ struct HvpOps {
 #define FTLM_HVP_OPS_M(VT, ST, SH, GPL, HALF, MODE)                                              \
     HvpOps<VT> {                                                                                   \
         &hvp_occupancy_t<VT, ST, SH, GPL, HALF, MODE>, &hvp_launch_t<VT, ST, SH, GPL, HALF, MODE>, \
-            hvp_max_threads<VT, SH>(), 0, 0, 0                                                        \
+            hvp_max_threads<VT, SH>(), 1, 0, 0, 0                                                        \
     }
 // one thread per representative (table mode, one block; hvp_lane.cuh)
 #define FTLM_HVP_LANE_OPS(VT, ST, D) \
     HvpOps<VT> {                                                                                                   \
-        &hvp_lane_occupancy_t<VT, ST, D>, &hvp_lane_launch_t<VT, ST, D>, kLaneThreads, kLaneThreads,               \
+        &hvp_lane_occupancy_t<VT, ST, D>, &hvp_lane_launch_t<VT, ST, D>, kLaneThreads, 0, kLaneThreads,            \
             lane_most_cols<VT, ST, D>(), lane_pad_bytes<ST, D>()                                                  \
     }
 // table mode, multi-block shapes, FP32 arithmetic (hvp_flow.cuh)
 #define FTLM_HVP_FLOW_OPS(ST, SH, CL, BC)                                                      \
     HvpOps<float> {                                                                             \
-        &hvp_flow_occupancy_t<ST, SH, CL, BC>, &hvp_flow_launch_t<ST, SH, CL, BC>, flow_threads<ST, SH, CL>(), 0, 0, 0 \
+        &hvp_flow_occupancy_t<ST, SH, CL, BC>, &hvp_flow_launch_t<ST, SH, CL, BC>, flow_threads<ST, SH, CL>(), 0, 0, 0, 0 \
     }
 #define FTLM_HVP_OPS(VT, ST, SH, GPL, HALF) FTLM_HVP_OPS_M(VT, ST, SH, GPL, HALF, 0)
 

@@ -387,7 +387,8 @@ ftlm_status hvp_choose_geom(const HvpOps<VT> *ops, HvpArgs<VT> a, bool tma, HvpG
 // times the candidate geometries on the plan's own buffers and keeps the
 // fastest for the rest of the process: warps per CTA (the kernel's bound down
 // to 4), staging buffers in flight (1..4 on the bulk-copy path), rho tables in
-// shared memory or read through L1 (FP32), the own-row prefetch on or off, and
+// shared memory or read through L1 (FP32), the own-row prefetch on or off (both
+// where the kernel has the choice), and
 // the representatives per tile (2, 4 or 8 per warp).  Every candidate computes
 // the same rows (one warp per representative, fixed flip order), so the choice
 // changes timing only.
@@ -482,8 +483,9 @@ ftlm_status hvp_tune(HvpPlan<VT> &plan, std::vector<HvpPart<VT>> &parts, bool tm
     out.ms = out.ms_default = best_ms;
     out.tried = 1;
     const int max_warps = plan.ops->max_threads / 32;
-    std::vector<int> rho_opts = sizeof(VT) == 4 ? std::vector<int>{1, 0} : std::vector<int>{0};
-    std::vector<int> own_opts = tma ? std::vector<int>{0, 1} : std::vector<int>{0};
+    const bool options = plan.ops->options;  // kernels without them compute the same in every variant
+    std::vector<int> rho_opts = sizeof(VT) == 4 && options ? std::vector<int>{1, 0} : std::vector<int>{def.rho_smem};
+    std::vector<int> own_opts = tma && options ? std::vector<int>{0, 1} : std::vector<int>{def.own};
     for (int warps = max_warps; warps >= 4; warps -= 4)
         for (int rho : rho_opts)
             for (int own : own_opts)
