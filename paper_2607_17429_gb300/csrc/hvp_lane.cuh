@@ -117,11 +117,8 @@ __device__ __forceinline__ PadRow<PB> pad_row(const ST *v) {
     for (int g = 0; g < D; ++g) {
         if constexpr (sizeof(ST) == 2) {
             r.w[g >> 1] |= (uint32_t)__half_as_ushort(v[g]) << (16 * (g & 1));
-        } else if constexpr (sizeof(ST) == 4) {
+        } else {  // FP64 rows are not padded
             r.w[g] = __float_as_uint(v[g]);
-        } else {
-            r.w[2 * g] = (uint32_t)__double2loint(v[g]);
-            r.w[2 * g + 1] = (uint32_t)__double2hiint(v[g]);
         }
     }
     return r;
