@@ -309,6 +309,8 @@ def hv_roofline(prof, dtype_name, flips, n_reps, W, B, esize, mode="search",
                 + n_reps * (2*W*B*e + 24)    [own rows, outputs, record and entry offset]
     against the measured STREAM copy bandwidth (MEASURED_PEAKS.json hbm_gbs).  flips per launch is the
     kernel's own device count while profiling (ftlm_profile.hv_flips), else the count from the labels.
+    These bytes count every gathered segment, which L2 serves in part, so frac may pass 1; dram_frac is the
+    recorded DRAM traffic of the same kernel over the same time against the same bandwidth.
     """
     pk, which = peaks()
     if prof["hv_launches"] == 0:
@@ -322,8 +324,9 @@ def hv_roofline(prof, dtype_name, flips, n_reps, W, B, esize, mode="search",
     else:
         byt = flips * (seg + 20) + n_reps * (2 * seg + 16)
     peak = float(pk["hbm_gbs"]) * 1e9
+    traffic = _traffic_record(dtype_name, mode, workload)
     return {"bound": "hbm", "achieved": byt / t / 1e9, "peak": peak / 1e9, "unit": "GB/s", "frac": byt / t / peak,
-            "traffic": _traffic_record(dtype_name, mode, workload), "algorithmic_per_launch": byt,
+            "traffic": traffic, "dram_frac": traffic / t / peak if traffic else None, "algorithmic_per_launch": byt,
             "avg_launch_ms": t * 1e3,
             "flip_path": mode,
             "flips_per_launch": flips,

@@ -164,7 +164,7 @@ struct HvpArgs {
 // into the addresses of the loads that follow, so none of them is moved before the wait.
 // A table kernel behind the build of its entries: 18 representatives of the s = 1/2 icosahedron at B = 8
 // 34.9 -> 28.7 us a call, 1.7e3 of the s = 1 cuboctahedron at B = 24 47.1 -> 44.6, the benchmark sector's five
-// runs of the workspace 8.68 -> 8.51 ms.
+// runs of the workspace 8.68 -> 8.51 ms (8.41 with the present table kernel).
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ unsigned prior_done() {
     unsigned zero;

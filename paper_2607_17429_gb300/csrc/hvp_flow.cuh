@@ -21,7 +21,7 @@
 //    so the copies never drain between representatives;
 //  - the flip groups' sums are combined by a reduce-scatter (each step halves the rows a lane keeps),
 //    which leaves every lane R = ceil(W / Q) rows of its two columns to finish.
-// Icosidodecahedron, M = 0, ten irreps, FP32: B = 8 9.16 -> 5.9 ms, B = 16 16.7 -> 10.5, B = 24 29.9 -> 16.9 (with
+// Icosidodecahedron, M = 0, ten irreps, FP32: B = 8 9.16 -> 5.8 ms, B = 16 16.7 -> 9.9, B = 24 29.9 -> 16.9 (with
 // the contraction left out 4.5, 9.6 and 16.2 ms: at B = 24 the 25 GB of gathers that miss L2 bind, at
 // B = 8 gathers and contraction take 4.5 and 4.4 ms and overlap in part).
 //

@@ -7,8 +7,8 @@
 // load per row.  The contributions are summed in entry order, a few apart at a time (the warp
 // kernels sum them per flip group and then across groups), so results agree with theirs to rounding.
 //
-// Blocks of dimension 1, 3, 4, 5 of the icosidodecahedron at M = 0, FP32, from the table: B = 1 0.19 to 0.43 ms;
-// B = 8 2.6 to 3.1 ms with a warp per representative, 0.29 to 1.25 ms here; B = 32 7.2 to 9.1 ms, 0.9 to 4.4 ms.
+// Blocks of dimension 1, 3, 4, 5 of the icosidodecahedron at M = 0, FP32, from the table: B = 1 0.19 to 0.40 ms;
+// B = 8 2.6 to 3.1 ms with a warp per representative, 0.29 to 1.29 ms here; B = 32 7.2 to 9.1 ms, 0.9 to 4.3 ms.
 // Bound by L1 sector look-ups of the gathers for rows of less than 32 bytes (B = 1: about one per cycle
 // and SM), by the entries' and gathers' latency above.
 #pragma once

@@ -706,7 +706,7 @@ void scratch_trim() {
 // workspace by the build kernel, then the table kernel reads them, run after run.  (Search and
 // contraction in one kernel share its 16 warps per SM and its instruction cache:
 // 15.7 ms a call for the ten icosidodecahedron irreps at B = 8, of which the search alone is 2.5 ms at the
-// build kernel's occupancy; 8.5 ms this way.)  Sums run in the table path's order, so both paths give
+// build kernel's occupancy; 8.4 ms this way.)  Sums run in the table path's order, so both paths give
 // the same bits.  FP64 keeps the search in the kernel: its contraction leaves the integer pipes
 // idle.  FTLM_ENOMEM (no workspace): the caller takes the one-kernel search.
 template <typename VT>
